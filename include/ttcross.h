@@ -186,7 +186,8 @@ typedef struct {
                                 wrote in the same sweep (always 0) */
   int64_t screen_fmas;       /* algorithmic FMAs of the screens: sum over sweeps and
                                 bonds of r_k * |superblock_k| */
-  int64_t error_fmas;        /* algorithmic FMAs of the sampled-error evaluations */
+  int64_t error_fmas;        /* FP64 FMAs of the sampled-error evaluations (the products
+                                that run on the tensor cores are not counted) */
   double tau;                /* final tau */
   double x_rms;              /* rms of X over the error samples */
   double err;                /* sampled relative Frobenius error */

@@ -332,7 +332,7 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
       CU(launch_phase(PH_DECIDE2, ra, h0->grid, s));
     }
     if (user && (us = user_fill(h0, 0, s))) return us;
-    CU(launch_phase(PH_TABLES, ra, h0->grid, s));
+    CU(launch_phase(PH_VERIFY, ra, h0->grid, s));
     CU(launch_phase(PH_UPDATE, ra, h0->grid, s));
   }
   return fail(TTC_ERR_CUDA, "host-stepped run did not finish");
@@ -602,7 +602,12 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     // with at most max(nsamples, 4096) index combinations and 128 MiB
     int64_t tl = 0, trr = 0;
     {
-      const int64_t lim = std::max<int64_t>(ns, 4096), bytes = (int64_t)128 << 20;
+      // (an eighth of the stored residuals where those are larger)
+      double estore = 0.0;
+      if (o.residual == TTC_RESIDUAL_STORED)
+        for (int b = 0; b < d - 1; ++b) estore += 8.0 * (double)I.bond[b].ldT * (double)I.bond[b].ldR;
+      const int64_t lim = std::max<int64_t>(ns, 4096);
+      const int64_t bytes = std::max((int64_t)128 << 20, (int64_t)std::min(estore / 8.0, 1e18));
       int64_t N = n[0];
       for (int a = 2; a < d; ++a) {
         N *= n[a - 1];
@@ -618,8 +623,42 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
         trr = cc;
       }
     }
-    double *tabL = cv.take<double>(tl);
-    double *tabR = cv.take<double>(trr);
+    // the error check on the tensor cores, where the samples are many and the
+    // middle modes small enough to sort by: the samples' orders, and a
+    // workspace that holds its plan at the rank caps with one block of
+    // samples' results (at most 1 GiB, else the FP64 chains do every check)
+    const int64_t tl_up = (tl + 31) / 32 * 32, tr_up = (trr + 31) / 32 * 32;
+    const int64_t tc_blocks = (ns + TC_BLOCK - 1) / TC_BLOCK;
+    bool tc = d >= 3 && ns >= 2 * TC_BLOCK && ns <= (1 << 24);
+    int64_t ews = tl_up + tr_up;
+    if (tc) {
+      auto up16 = [](int64_t v) { return (v + 15) / 16 * 16; };
+      double words = 0.0, cols = 0.0;
+      int64_t kmax = 16;
+      for (int m = 1; m < d - 1; ++m) {
+        const int64_t kp = up16(h->bond_cap[m - 1]), np = up16(h->bond_cap[m]);
+        tc = tc && n[m] <= TC_NMAX;
+        words += (double)n[m] * (np * (kp + 1) + 8);
+        cols += (double)n[m] * (up16(np) * (kp + 1) + 8);
+        kmax = std::max(kmax, kp);
+      }
+      const double NL = (double)n[0] * n[1], NR = (double)n[d - 1] * n[d - 2];
+      words += (NL <= TC_TABLE_MAX ? NL : (double)n[0]) * (up16(h->bond_cap[std::min(1, d - 2)]) + 1) +
+               (double)n[0] * (up16(h->bond_cap[0]) + 1);
+      words += (NR <= TC_TABLE_MAX ? NR : 1.0) * up16(h->bond_cap[std::max(0, d - 3)]);
+      words += 2.0 * TC_BLOCK * (kmax + 1) + 4096;
+      if (words * 8 > (double)((int64_t)1 << 30)) tc = false;
+      // beside the tables: the rows before their last mode, the cores' columns
+      if (tc) ews = std::max(ews + (tl + trr) / 8 + (int64_t)cols + 4096, (int64_t)words);
+    }
+    double *tabL = cv.take<double>(ews);
+    double *tabR = tabL + tl_up;
+    uint16_t *tcperm = tc ? cv.take<uint16_t>((size_t)((d - 2) * tc_blocks * TC_BLOCK)) : nullptr;
+    uint32_t *tctile[TTC_MAXD] = {};
+    if (tc)
+      for (int m = 1; m < d - 1; ++m)
+        tctile[m] = cv.take<uint32_t>((size_t)(tc_blocks * (TC_BLOCK / 16 + n[m])));
+    char *tcplan = cv.take<char>(tc_plan_bytes());
     if (pass == 0) {
       h->pool_bytes = cv.off;
       cudaError_t e = cudaMalloc(&h->pool, h->pool_bytes);
@@ -653,6 +692,12 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
       I.ctrl = ctrl;
       h->core_stage = stage;
       h->core_stage_cap = core_cap;
+      I.ews = tabL;
+      I.ews_cap = ews;
+      I.tcp = reinterpret_cast<TcPlan *>(tcplan);
+      I.tc_perm = tcperm;
+      I.tc_stride = tc_blocks * TC_BLOCK;
+      for (int m = 0; m < TTC_MAXD; ++m) I.tc_tile[m] = tctile[m];
       I.tabL = tabL;
       I.tabR = tabR;
       I.tabL_cap = tl;
@@ -745,6 +790,19 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     return cleanup(fail(TTC_ERR_CUDA, "copy of the instance list failed"));
   ttc_status s = ensure_cands(h, nullptr);
   if (s != TTC_OK) return cleanup(s);
+  if (I.tc_perm) {
+    for (int m = 1; m < d - 1; ++m)
+      if (cudaMemset(const_cast<uint32_t *>(I.tc_tile[m]), 0xFF,
+                     sizeof(uint32_t) * (size_t)(I.tc_stride / TC_BLOCK * (TC_BLOCK / 16 + n[m]))) !=
+          cudaSuccess)
+        return cleanup(fail(TTC_ERR_CUDA, "cudaMemset of the sample tiles failed"));
+    // (the tile arrays' pointers are part of the descriptor on the device)
+    const size_t at = reinterpret_cast<char *>(&I.tc_tile[0]) - reinterpret_cast<char *>(&I);
+    uint32_t *const *tiles = reinterpret_cast<uint32_t *const *>(reinterpret_cast<char *>(h->d_inst) + at);
+    if (launch_tc_perm(h->d_inst, d, I.tc_stride / TC_BLOCK, const_cast<uint16_t *>(I.tc_perm), tiles) !=
+        cudaSuccess)
+      return cleanup(fail(TTC_ERR_CUDA, "sorting the error samples failed"));
+  }
   if (mxtab) {
     if (launch_maxwellian_tables(h->d_inst, const_cast<double *>(I.mx_coef),
                                  const_cast<double *>(I.mx_nh),

@@ -28,6 +28,10 @@ constexpr int TT_GEN_RMAX = 160;  // largest TT rank of a TT-cores generator
 constexpr int BM = 64, BN = 64;   // screen tile (superblock rows x columns)
 constexpr int RCAP = 256;         // largest rank capacity the kernels accept
 constexpr int GRID_CAP = 4096;    // largest persistent grid (partial-sum slots)
+constexpr int TC_BLOCK = 32768;   // error samples sorted together by a middle index
+constexpr int TC_NMAX = 2048;     // largest middle mode size of the sorted samples
+constexpr uint32_t TC_NO_TILE = 0xffffffffu;  // an unused tile slot
+constexpr int64_t TC_TABLE_MAX = 1 << 20;  // prefix / suffix table rows of the tensor-core plan
 
 enum State : int32_t { ST_SCREEN = 0, ST_UPDATE = 1, ST_VERIFY = 2, ST_DONE = 3 };
 enum Prec : int32_t { P_FP64 = 0, P_FP32 = 1, P_SPLIT = 2 };
@@ -138,8 +142,19 @@ struct InstDev {
   BondDev bond[TTC_MAXB];
   SetDev empty;                      // I_{<=0} / J_{>d}: one empty multi-index
   double *xs;                        // X at the error samples
-  double *tabL, *tabR;               // prefix / suffix contractions of the TT (error check)
+  double *ews;                       // workspace of the error check (8-byte words)
+  int64_t ews_cap;
+  double *tabL, *tabR;               // in it: prefix / suffix contractions of the TT (FP64 chains)
   int64_t tabL_cap, tabR_cap;        // their capacities (doubles)
+  // the error check on the tensor cores (ttc_error.cuh): its plan, and for
+  // every middle mode m the samples of each block of TC_BLOCK in the order of
+  // their index i_m (ids within the block, tc_perm + (m - 1) tc_stride), cut
+  // into tiles of one index (tc_tile[m], TC_BLOCK / 16 + n_m slots a block);
+  // tc_perm null: FP64 chains only
+  struct TcPlan *tcp;
+  const uint16_t *tc_perm;
+  int64_t tc_stride;
+  const uint32_t *tc_tile[TTC_MAXD];
   int64_t nsamples;                  // samples used (== prod n when exhaustive)
   int32_t exhaustive;
   uint64_t seed;

@@ -168,6 +168,7 @@ __device__ void decide_bond_sampled(const InstDev &in, Ctrl &cr, int b, DecideSm
 // sampled-error split (defined with the error evaluation below)
 __device__ void choose_split(const InstDev &in, const int32_t *r, int &pL, int &pR);
 __device__ double split_cost(const InstDev &in, const int32_t *r, int pL, int pR);
+__device__ int64_t error_fmas(const InstDev &in, const int32_t *r);
 
 // ---------------------------------------------------------------------------
 // reductions
@@ -2213,11 +2214,9 @@ __device__ void verify_instance(const InstDev &in, Ctrl &cr, DecideSmem &sm) {
     cr.screened = 0;
     const double err = sqrt(num / ld_cg(cr.den));
     cr.err = err;
-    int pL, pR;
     int32_t rr[TTC_MAXD];
     for (int b = 0; b < in.nb; ++b) rr[b] = ld_cg(cr.r[b]);
-    choose_split(in, rr, pL, pR);
-    cr.error_fmas += (int64_t)split_cost(in, rr, pL, pR);
+    cr.error_fmas += error_fmas(in, rr);
     for (int b = 0; b < in.nb; ++b) cr.add[b] = 0;
     sm.flag = 0;
     if (!isfinite(err)) {
@@ -2964,10 +2963,23 @@ __device__ __forceinline__ int mul_core_right(const InstDev &in, const int32_t *
   return rl;
 }
 
-constexpr int TAB_CHUNK = 8;  // last-mode indices per table work item
+}  // namespace ttc
+
+#include "ttc_error.cuh"
+
+namespace ttc {
+
+// last-mode indices per table work item: 8 share the vector of their prefix;
+// fewer (down to 2) when that leaves most threads without an item (the 6D
+// n = 256 tables: 8192 items of 8 rows for 77824 threads)
+__device__ __forceinline__ int64_t table_chunk(int64_t prefixes, int64_t n, int64_t threads) {
+  int64_t c = 8;
+  while (c > 2 && prefixes * ((n + c - 1) / c) * 2 <= threads) c /= 2;
+  return c;
+}
 
 // tables of the verifying instances: a work item is a prefix of pL-1 modes
-// (suffix of pR-1 modes) and a chunk of TAB_CHUNK values of the next mode
+// (suffix of pR-1 modes) and a chunk of values of the next mode
 __device__ void phase_tables(const RunArgs &ra) {
   // items are dealt a warp's worth per CTA in turn (lane l of warp w of CTA
   // c is number (w G + c) 32 + l): when there are fewer items than threads
@@ -2987,15 +2999,49 @@ __device__ void phase_tables(const RunArgs &ra) {
     int nadd = 0;
     for (int b = 0; b < in.nb; ++b) nadd += snap.add[b];
     if (nadd) continue;
-    int pL, pR;
-    choose_split(in, r, pL, pR);
+    // the plan: the same on every CTA; CTA 0 leaves it for the later phases
+    __shared__ TcPlan plan;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc_plan(in, r, plan);
+      if (blockIdx.x == 0) *in.tcp = plan;
+    }
+    __syncthreads();
+    // the tables made here: pL / pR modes, one fewer where the last mode runs
+    // on the tensor cores (phase_stages); fixed-point rows where those read them
     const int d = in.d;
+    const int pL = plan.pL - plan.tl, pR = plan.pR - plan.tr;
+    const bool fixL = plan.on || plan.tl, fixR = plan.tr;
     double v[RCAP], w[RCAP];
+    double *const tabL = fixL ? in.ews + plan.L : in.tabL;
+    double *const tabR = plan.on || fixR ? in.ews + plan.R : in.tabR;
+    int32_t *const Le = reinterpret_cast<int32_t *>(in.ews + plan.Le);
+    int32_t *const Re = reinterpret_cast<int32_t *>(in.ews + plan.Re);
+    const int64_t sl = core_s(in, r, pL), ll = fixL ? tc_up(sl, 16) : sl;      // a prefix row
+    const int64_t sr = core_s(in, r, d - pR), lr = fixR ? tc_up(sr, 16) : sr;  // a suffix row
+    if (fixL && pL == 1) {
+      const BondDev &B0 = in.bond[0];
+      for (int64_t x = first_item(base, gt, NTOT); x < base + in.n[0]; x += NTOT) {
+        double *row = tabL + (x - base) * ll;
+        copy8(row, B0.T + (x - base), B0.ldT, (int)sl);
+        Le[x - base] = tc_fix_row(row, (int)sl, (int)ll);
+      }
+      base += in.n[0];
+    }
+    if (fixR && pR == 1) {
+      const BondDev &BL = in.bond[d - 2];
+      for (int64_t x = first_item(base, gt, NTOT); x < base + in.n[d - 1]; x += NTOT) {
+        double *row = tabR + (x - base) * lr;
+        copy8(row, BL.R + (x - base), BL.ldR, (int)sr);
+        Re[x - base] = tc_fix_row(row, (int)sr, (int)lr);
+      }
+      base += in.n[d - 1];
+    }
     if (pL >= 2) {
       int64_t np = 1;
       for (int m = 0; m < pL - 1; ++m) np *= in.n[m];
-      const int64_t nl = in.n[pL - 1], nch = (nl + TAB_CHUNK - 1) / TAB_CHUNK;
-      const int64_t sl = core_s(in, r, pL);
+      const int64_t nl = in.n[pL - 1], chunk = table_chunk(np, nl, NTOT / 2);
+      const int64_t nch = (nl + chunk - 1) / chunk;
       const int64_t items = np * nch;
       for (int64_t x = first_item(base, gt, NTOT); x < base + items; x += NTOT) {
         const int64_t pre = (x - base) / nch, ch = (x - base) - pre * nch;
@@ -3011,8 +3057,11 @@ __device__ void phase_tables(const RunArgs &ra) {
         for (int m = 1; m < pL - 1; ++m) len = mul_core(in, r, m, idx[m], v, w);
         // last mode of the prefix: core pL-1 (a middle core, pL-1 <= d-2)
         const BondDev &B = in.bond[pL - 1];
-        for (int64_t i = ch * TAB_CHUNK; i < min(nl, (ch + 1) * TAB_CHUNK); ++i)
-          contract4(v, len, B.T + i, B.ldT, nl, in.tabL + (pre + i * np) * sl, (int)sl);
+        for (int64_t i = ch * chunk; i < min(nl, (ch + 1) * chunk); ++i) {
+          double *row = tabL + (pre + i * np) * ll;
+          contract4(v, len, B.T + i, B.ldT, nl, row, (int)sl);
+          if (fixL) Le[pre + i * np] = tc_fix_row(row, (int)sl, (int)ll);
+        }
       }
       base += items;
     }
@@ -3020,8 +3069,8 @@ __device__ void phase_tables(const RunArgs &ra) {
       int64_t np = 1;
       for (int m = d - pR + 1; m < d; ++m) np *= in.n[m];
       const int mf = d - pR;  // first mode of the suffix
-      const int64_t nf = in.n[mf], nch = (nf + TAB_CHUNK - 1) / TAB_CHUNK;
-      const int64_t sr = core_s(in, r, mf);
+      const int64_t nf = in.n[mf], chunk = table_chunk(np, nf, NTOT / 2);
+      const int64_t nch = (nf + chunk - 1) / chunk;
       const int64_t items = np * nch;
       for (int64_t x = first_item(base, gt, NTOT); x < base + items; x += NTOT) {
         const int64_t suf = (x - base) / nch, ch = (x - base) - suf * nch;
@@ -3036,11 +3085,74 @@ __device__ void phase_tables(const RunArgs &ra) {
         copy8(w, BL.R + idx[d - 1], BL.ldR, len);
         for (int m = d - 2; m > mf; --m) len = mul_core_right(in, r, m, idx[m], w, v);
         const BondDev &B = in.bond[mf];
-        for (int64_t i = ch * TAB_CHUNK; i < min(nf, (ch + 1) * TAB_CHUNK); ++i)
-          contract4(w, len, B.T + i, nf, B.ldT, in.tabR + (i + nf * suf) * sr, (int)sr);
+        for (int64_t i = ch * chunk; i < min(nf, (ch + 1) * chunk); ++i) {
+          double *row = tabR + (i + nf * suf) * lr;
+          contract4(w, len, B.T + i, nf, B.ldT, row, (int)sr);
+          if (fixR) Re[i + nf * suf] = tc_fix_row(row, (int)sr, (int)lr);
+        }
       }
       base += items;
     }
+    if (plan.on)
+      for (int m = pL; m < d - pR; ++m) tc_columns(in, r, plan, m, false, base, gt, NTOT);
+    if (plan.tl) tc_columns(in, r, plan, pL, false, base, gt, NTOT);
+    if (plan.tr) tc_columns(in, r, plan, d - 1 - pR, true, base, gt, NTOT);
+  }
+}
+
+// FP64 FMAs of an error check: the tables', then the chains per sample, or the
+// samples' products with the suffix rows where the middle cores run on the
+// tensor cores
+__device__ int64_t error_fmas(const InstDev &in, const int32_t *r) {
+  const TcPlan &p = *in.tcp;
+  const int pL = ld_cg(p.pL), pR = ld_cg(p.pR);
+  const int tl = ld_cg(p.tl), tr = ld_cg(p.tr);
+  double per = 0.0;
+  if (!ld_cg(p.on))
+    per = split_cost(in, r, pL, pR) - (double)tc_table_cost(in, r, pL, pR);
+  else
+    per = (double)in.nsamples * (double)core_s(in, r, in.d - pR);
+  return (int64_t)((double)tc_table_cost(in, r, pL - tl, pR - tr) + per);
+}
+
+// the middle cores of the checks planned on the tensor cores, a grid barrier
+// after every stage of every step (all instances' stages side by side)
+__device__ bool phase_stages(const RunArgs &ra, PhaseSmem &sm) {
+  __shared__ CtrlSnap snap;
+  __shared__ TcPlan plan;
+  const int NW = (int)gridDim.x * (NT / 32);
+  const int gw = (int)blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
+  for (int step = 0;; ++step) {
+    bool any = false;
+    for (int ii = 0; ii < ra.count; ++ii) {
+      const InstDev &in = inst(ra, ii);
+      if (!in.tc_perm) continue;
+      snap_ctrl(*in.ctrl, in.nb, snap);
+      if (snap.state == ST_DONE || !snap.screened) continue;
+      int nadd = 0;
+      for (int b = 0; b < in.nb; ++b) nadd += snap.add[b];
+      if (nadd) continue;
+      for (int k = threadIdx.x; k < (int)(sizeof(TcPlan) / 4); k += NT)
+        reinterpret_cast<int32_t *>(&plan)[k] = __ldcg(reinterpret_cast<const int32_t *>(in.tcp) + k);
+      __syncthreads();
+      if (step == 0 && (plan.tl || plan.tr)) {
+        any = true;
+        if (plan.tl) tc_extend(in, snap.r, plan, 0, gw, NW);
+        if (plan.tr) tc_extend(in, snap.r, plan, 1, gw, NW);
+        continue;
+      }
+      if (!plan.on || step >= plan.nst * plan.nsb) continue;
+      any = true;
+      const int st = step % plan.nst, sb = step / plan.nst;
+      const double part = tc_stage(in, snap.r, plan, st, sb, gw, NW);
+      if (st == plan.nst - 1) {
+        const double s = block_sum(part, sm.red);
+        if (threadIdx.x == 0) in.err_part[blockIdx.x] = sb == 0 ? s : __dadd_rn(in.err_part[blockIdx.x], s);
+        __syncthreads();
+      }
+    }
+    if (!any) return true;
+    if (!grid_barrier(ra, 13)) return false;
   }
 }
 
@@ -3108,11 +3220,12 @@ __device__ double sample_residual(const InstDev &in, const int32_t *r, int pL, i
 
 
 // The error's samples when the prefix and suffix tables meet (pL + pR = d,
-// rows of len <= 16): lane l of a warp takes the l-th of 32 consecutive
-// samples, as in the thread dealing of the plain loop.  The warp loads the
-// 32 samples' rows together, two rows per instruction, into shared memory,
-// and each lane then runs the contract's chain on its own two rows.  The
-// operations and their order per thread are those of sample_residual.
+// rows of len): lane l of a warp takes the l-th of 32 consecutive samples, as
+// in the thread dealing of the plain loop.  Sixteen entries at a time, the
+// warp loads the 32 samples' rows together, two rows per instruction, into
+// shared memory, and each lane runs the contract's chain on its own two rows
+// (a thread reading its own rows touches 32 lines per load).  The operations
+// and their order per thread are those of sample_residual.
 __device__ __noinline__ double samples_joined(const InstDev &in, int pL, int pR, int len,
                                               int64_t base, int64_t ns, int64_t gs, int64_t NTOT,
                                               SampleSmem &sw) {
@@ -3136,35 +3249,38 @@ __device__ __noinline__ double samples_joined(const InstDev &in, int pL, int pR,
       eR += sample_coord(in, k, m) * st;
       st *= in.n[m];
     }
-    double xv[16], yv[16];
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const double *tab = side == 0 ? in.tabL : in.tabR;
-      const int64_t e = side == 0 ? eL : eR;
-      double v[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const int sr = 2 * q + half;
-        const int64_t es = __shfl_sync(FULL, e, sr);
-        const int vs = __shfl_sync(FULL, valid, sr);
-        v[q] = (vs && el < len) ? tab[es * len + el] : 0.0;
-      }
-      __syncwarp();  // the previous rows are read
-#pragma unroll
-      for (int q = 0; q < 16; ++q) buf[(2 * q + half) * 17 + el] = v[q];
-      __syncwarp();
-#pragma unroll
-      for (int t = 0; t < 16; ++t) {
-        if (side == 0)
-          xv[t] = buf[lane * 17 + t];
-        else
-          yv[t] = buf[lane * 17 + t];
-      }
-    }
     double acc = 0.0;
+    for (int c = 0; c < len; c += 16) {
+      const bool has = c + el < len;
+      double xv[16], yv[16];
 #pragma unroll
-    for (int t = 0; t < 16; ++t)
-      if (t < len) acc = __fma_rn(xv[t], yv[t], acc);
+      for (int side = 0; side < 2; ++side) {
+        const double *tab = (side == 0 ? in.tabL : in.tabR) + c + el;
+        const int64_t e = side == 0 ? eL : eR;
+        double v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          const int sr = 2 * q + half;
+          const int64_t es = __shfl_sync(FULL, e, sr);
+          const int vs = __shfl_sync(FULL, valid, sr);
+          v[q] = (vs && has) ? tab[es * len] : 0.0;
+        }
+        __syncwarp();  // the previous rows are read
+#pragma unroll
+        for (int q = 0; q < 16; ++q) buf[(2 * q + half) * 17 + el] = v[q];
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          if (side == 0)
+            xv[t] = buf[lane * 17 + t];
+          else
+            yv[t] = buf[lane * 17 + t];
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 16; ++t)
+        if (c + t < len) acc = __fma_rn(xv[t], yv[t], acc);
+    }
     if (valid) {
       const double e = __dsub_rn(xk, acc);
       part = __fma_rn(e, e, part);
@@ -3308,12 +3424,12 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
         }
       }
     } else if (screened) {
+      if (ld_cg(in.tcp->on)) continue;  // done by phase_stages
       double part = 0.0;
       const int64_t ns = in.nsamples;
-      int pL, pR;
-      choose_split(in, rn, pL, pR);
+      const int pL = ld_cg(in.tcp->pL), pR = ld_cg(in.tcp->pR);
       const int jl = pL >= 2 && pR >= 2 && pL + pR == in.d ? (int)core_s(in, rn, pL) : 0;
-      if (jl > 0 && jl <= 16) {
+      if (jl > 0) {
         part = samples_joined(in, pL, pR, jl, base, ns, gs, NTOT, sm.sw);
       } else {
         for (int64_t x = first_item(base, gs, NTOT); x < base + ns; x += NTOT) {
@@ -3678,6 +3794,7 @@ __global__ void __launch_bounds__(NT, 2) k_persistent(RunArgs ra) {
     if (verify) {
       phase_tables(ra);
       if (!grid_barrier(ra, 9)) return;
+      if (!phase_stages(ra, sm)) return;
     }
     phase_update(ra, sm);
     if (!grid_barrier(ra, 5)) return;
@@ -3725,9 +3842,14 @@ __global__ void __launch_bounds__(NT, 2) k_finalize(RunArgs ra) {
   cache_inst0(ra);
   phase_finalize(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem));
 }
-__global__ void __launch_bounds__(NT, 2) k_tables(RunArgs ra) {
+// the error check up to its samples' FP64 chains (a cooperative launch: its
+// phases meet at grid barriers); nothing when no instance verifies
+__global__ void __launch_bounds__(NT, 2) k_verify(RunArgs ra) {
   cache_inst0(ra);
+  if (!any_verify(ra)) return;
   phase_tables(ra);
+  if (!grid_barrier(ra, 9)) return;
+  phase_stages(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem));
 }
 __global__ void __launch_bounds__(NT, 2) k_update(RunArgs ra) {
   cache_inst0(ra);
@@ -3878,7 +4000,7 @@ cudaError_t launch_phase(int phase, const RunArgs &ra, int grid, cudaStream_t s)
     case PH_UPDATE: f = (const void *)k_update; break;
     case PH_REFINE: f = (const void *)k_refine; break;
     case PH_DECIDE2: f = (const void *)k_decide2; break;
-    case PH_TABLES: f = (const void *)k_tables; break;
+    case PH_VERIFY: f = (const void *)k_verify; break;
     case PH_ROOK_SCAN: f = (const void *)k_rook_scan; break;
     case PH_ROOK_DECIDE: f = (const void *)k_rook_decide; break;
     case PH_FINALIZE: f = (const void *)k_finalize; break;
@@ -3887,6 +4009,12 @@ cudaError_t launch_phase(int phase, const RunArgs &ra, int grid, cudaStream_t s)
   cudaError_t e = prep(f);
   if (e != cudaSuccess) return e;
   void *args[] = {(void *)&ra};
+  if (phase == PH_VERIFY) {
+    // its grid barriers count from zero
+    e = cudaMemsetAsync(&ra.bar->count, 0, sizeof ra.bar->count, s);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(NT), args, sizeof(PhaseSmem), s);
+  }
   return cudaLaunchKernel(f, dim3(grid), dim3(NT), args, sizeof(PhaseSmem), s);
 }
 
@@ -4113,6 +4241,90 @@ cudaError_t launch_user_samples(const InstDev *d_inst, int32_t *idx, cudaStream_
   k_user_samples<<<152 * 4, 256, 0, s>>>(d_inst, idx);
   return cudaGetLastError();
 }
+
+// The samples of block blockIdx.x in the order of their index of mode
+// m = 1 + blockIdx.y (stable), and their tiles (create time; the tile slots
+// are all TC_NO_TILE before).  Eight warps take eighths of the block: each
+// counts its samples per index, the counts (and the tiles they make) are
+// scanned over (index, warp), each warp places its samples.
+constexpr int TC_PW = 8;
+__global__ void __launch_bounds__(32 * TC_PW) k_tc_perm(const InstDev *inp, uint16_t *perm,
+                                                        uint32_t *const *tiles) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int SEG = TC_BLOCK / TC_PW;
+  __shared__ uint16_t cnt[TC_PW][TC_NMAX];
+  __shared__ int32_t wsum[TC_PW], wtile[TC_PW];
+  const InstDev &in = *inp;
+  const int m = 1 + blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int n = (int)in.n[m];
+  const int64_t k0 = (int64_t)blockIdx.x * TC_BLOCK;
+  for (int x = threadIdx.x; x < TC_PW * n; x += blockDim.x) cnt[x / n][x % n] = 0;
+  __syncthreads();
+  for (int pass = 0; pass < 2; ++pass) {
+    uint16_t *pm = perm + (int64_t)(m - 1) * in.tc_stride + k0;
+    for (int s = 0; s < SEG; s += 32) {
+      const int id = w * SEG + s + lane;
+      const bool ok = k0 + id < in.nsamples;
+      const int key = ok ? sample_coord(in, k0 + id, m) : n;
+      const unsigned peers = __match_any_sync(FULL, key);
+      const int rank = __popc(peers & ((1u << lane) - 1));
+      if (pass == 1 && ok) pm[cnt[w][key] + rank] = (uint16_t)id;
+      __syncwarp();
+      if (ok && rank == 0) cnt[w][key] += (uint16_t)__popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    if (pass == 1) return;
+    // exclusive scan in (index, warp) order: thread x takes indices [x c, (x + 1) c)
+    const int c = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int i0 = min(n, (int)threadIdx.x * c), i1 = min(n, i0 + c);
+    int sum = 0, nti = 0;
+    for (int i = i0; i < i1; ++i) {
+      int v = 0;
+      for (int q = 0; q < TC_PW; ++q) v += cnt[q][i];
+      sum += v;
+      nti += (v + 15) / 16;
+    }
+    int inc = sum, tinc = nti;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(FULL, inc, o), u = __shfl_up_sync(FULL, tinc, o);
+      if (lane >= o) {
+        inc += v;
+        tinc += u;
+      }
+    }
+    if (lane == 31) {
+      wsum[w] = inc;
+      wtile[w] = tinc;
+    }
+    __syncthreads();
+    int at = inc - sum, ta = tinc - nti;
+    for (int q = 0; q < w; ++q) {
+      at += wsum[q];
+      ta += wtile[q];
+    }
+    uint32_t *tl = tiles[m] + (int64_t)blockIdx.x * (TC_BLOCK / 16 + n);
+    for (int i = i0; i < i1; ++i) {
+      const int first = at;
+      for (int q = 0; q < TC_PW; ++q) {
+        const int v = cnt[q][i];
+        cnt[q][i] = (uint16_t)at;
+        at += v;
+      }
+      for (int o = first; o < at; o += 16)
+        tl[ta++] = ((uint32_t)i << 19) | ((uint32_t)o << 4) | (uint32_t)(min(16, at - o) - 1);
+    }
+    __syncthreads();
+  }
+}
+
+cudaError_t launch_tc_perm(const InstDev *d_inst, int d, int64_t blocks, uint16_t *perm,
+                           uint32_t *const *tiles) {
+  k_tc_perm<<<dim3((unsigned)blocks, (unsigned)(d - 2)), 32 * TC_PW>>>(d_inst, perm, tiles);
+  return cudaGetLastError();
+}
+
+size_t tc_plan_bytes() { return sizeof(TcPlan); }
 
 // Maxwellian tables of an instance (create time)
 __global__ void k_maxwellian_tables(const InstDev *inp, double *coef, double *nh, double *cosx) {

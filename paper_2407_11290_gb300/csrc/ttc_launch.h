@@ -8,7 +8,7 @@ namespace ttc {
 
 enum Phase {
   PH_INIT1 = 0, PH_INIT2 = 1, PH_INIT3 = 2, PH_SCREEN = 3, PH_DECIDE = 4, PH_UPDATE = 5,
-  PH_REFINE = 6, PH_DECIDE2 = 7, PH_TABLES = 8, PH_ROOK_SCAN = 9, PH_ROOK_DECIDE = 10,
+  PH_REFINE = 6, PH_DECIDE2 = 7, PH_VERIFY = 8, PH_ROOK_SCAN = 9, PH_ROOK_DECIDE = 10,
   PH_FINALIZE = 11
 };
 
@@ -28,6 +28,12 @@ cudaError_t launch_user_gather(const InstDev *d_inst, int first, const int64_t *
 cudaError_t launch_user_scatter(const InstDev *d_inst, int first, const int64_t *counts,
                                 const double *vals, cudaStream_t s);
 cudaError_t launch_user_samples(const InstDev *d_inst, int32_t *idx, cudaStream_t s);
+// error check on the tensor cores: the samples sorted by every middle index
+// (perm and the device array of tile arrays, on the legacy stream), the bytes
+// of a plan
+cudaError_t launch_tc_perm(const InstDev *d_inst, int d, int64_t blocks, uint16_t *perm,
+                           uint32_t *const *tiles);
+size_t tc_plan_bytes();
 cudaError_t launch_maxwellian_tables(const InstDev *d_inst, double *coef, double *nh, double *cosx);
 
 // tile geometry used to size the candidate buffer (host mirror of tile_geo)
