@@ -8,13 +8,13 @@
 //            max |E| (ties: lowest column-major linear index);
 //   decide : one CTA per instance merges the tile candidates (the Allgather
 //            of Alg. 3), applies the stop test and appends the pivots:
-//            nested index sets (eq. nestedpivots), pivot history, and the
-//            bordered Sherman-Morrison update of P^{-1} (Sec. 3.1.1);
+//            nested index sets (eq. nestedpivots) and pivot history;
 //   update : every CTA applies eq. aca_approx_T_sub to the old rows of T,
 //            replays the pivot history on rows that entered the superblock
-//            (Alg. 4), and generates the new rows / columns of R; or, when an
-//            instance has converged at its threshold, evaluates the sampled
-//            error of Sec. 5.
+//            (Alg. 4), borders P^{-1} (Sherman-Morrison, Sec. 3.1.1), and
+//            generates the new rows / columns of R; or, when an instance has
+//            converged at its threshold, the sampled error of Sec. 5 is
+//            evaluated.
 // The phases run either in one persistent cooperative launch separated by
 // grid barriers (every wait bounded in time) or as separate launches.
 #include <algorithm>
@@ -67,8 +67,6 @@ struct DecideSmem {
   double ua[RCAP], bu[RCAP], brow[RCAP];
   double hcs[RCAP], hps[RCAP];  // R(:, c*) and T(a*, :) of the pivot step
   double us[DEC_US * DEC_US];   // U before the step (z <= DEC_US)
-  int32_t key[RCAP];            // pivot t's column: index sum (Hilbert) or coordinate
-  int32_t lsum, rsum;           // index sums of the pivot's row part / column part
   int64_t q_nt;                 // control words of the decide item
   int32_t q_r, q_maxr, q_prow, q_pcol;
   double q_tau, q_xrms;
@@ -82,7 +80,6 @@ struct DecideSmem {
   uint64_t rk[NT / 32];
   int64_t rl[NT / 32];
   int32_t rr[NT / 32], rc[NT / 32];
-  double delta;
   int32_t flag;
   // the eight warps' top candidates of the mixed stored decide
   uint64_t wk[NT / 32 * 8];
@@ -100,14 +97,17 @@ struct SpreadSmem {
   int32_t k, place, bad, nsm, not2;
 };
 
-// replays of up to 32 pivots (Alg. 4): the history triangles (row z at
-// z (z - 1) / 2) and delta, shared by the CTA's replay warps; after the
-// block reductions' words, which the CTA's other warps may be using meanwhile
-constexpr int LANE_NZ = 32;
+// replays (Alg. 4): per replay warp (the first RB_WARPS of a CTA) the rows T(a, :)
+// it rebuilds, their entries at the pivot columns, delta, and the history rows
+// of RB_STAGES steps in flight (replay_group's layout); after the block
+// reductions' words, which the CTA's other warps may be using meanwhile
+constexpr int RB_WARPS = 2, RB_STAGES = 3;
+constexpr int RB_SMALL = 64;  // pivots up to which a warp rebuilds eight rows
+constexpr int RB_BUF = 2 * RCAP + RCAP + 2 * RB_STAGES * RCAP;
+static_assert(RB_BUF >= 2 * 8 * (RB_SMALL + 1) + RB_SMALL + 2 * RB_STAGES * RB_SMALL, "replay buffer");
 struct ReplaySmem {
   double red_pad[NT / 32];
-  double hc[LANE_NZ * (LANE_NZ - 1) / 2], hp[LANE_NZ * (LANE_NZ - 1) / 2];
-  double delta[LANE_NZ];
+  double buf[RB_WARPS][RB_BUF];
 };
 
 // the error's samples when the tables meet: a warp's 32 samples' table rows
@@ -1658,8 +1658,8 @@ __device__ void phase_screen(const RunArgs &ra, PhaseSmem &sm) {
 // ---------------------------------------------------------------------------
 // decide: append the pivot (a*, c*) to bond b (block-wide).  I_{<=k} gets
 // (alpha*, i*), J_{>k} gets (j*, beta*) (eq. nestedpivots); the history of
-// step z keeps c_z = R(:, c*), T(a*, :) and delta; U = P^{-1} is bordered
-// by [[U + d U a b U, -d U a], [-d b U, d]] (Sec. 3.1.1).
+// step z keeps c_z = R(:, c*), T(a*, :) and delta.  P^{-1} is bordered in the
+// update phase (border_inverse): no decision reads it.
 __device__ bool append_pivot(const InstDev &in, Ctrl &cr, int b, int64_t as, int64_t cs, int z,
                              DecideSmem &sm) {
   const BondDev &B = in.bond[b];
@@ -1671,10 +1671,8 @@ __device__ bool append_pivot(const InstDev &in, Ctrl &cr, int b, int64_t as, int
   const SetDev &L = left_set(in, b);
   const SetDev &Rset = right_set(in, b);
   const bool hil = in.gen == 0;
-  const bool ustage = z <= DEC_US;
   // one round of independent loads: warp 1 appends the index sets (a lane
-  // per index), threads t < z gather the history (R(t, c*), T(a*, t)) and
-  // the pivot columns' index sums (Hilbert) or coordinates, the rest stage U
+  // per index), threads t < z gather the history (R(t, c*), T(a*, t))
   if (tid >= 32 && tid < 64) {
     const int lane = tid - 32;
     const int wl = b, wj = in.d - 1 - b;
@@ -1695,29 +1693,18 @@ __device__ bool append_pivot(const InstDev &in, Ctrl &cr, int b, int64_t as, int
   double *hp = B.hpiv + (int64_t)z * cap;
   for (int t = tid; t < z; t += NT) {
     const double c = B.R[(int64_t)t * B.ldR + cs], v = B.T[(int64_t)t * B.ldT + as];
-    sm.key[t] = hil ? B.J.sum[t] : B.pcol[t];
     hc[t] = c;
     hp[t] = v;
     sm.hcs[t] = c;
     sm.hps[t] = v;
   }
-  if (tid == NT - 1) sm.lsum = L.sum[p] + (int32_t)i;
-  if (tid == NT - 2) sm.rsum = Rset.sum[q] + (int32_t)j;
-  if (ustage)
-    for (int x = tid; x < z * z; x += NT) {
-      const int t = x / z, u = x - t * z;
-      sm.us[x] = B.U[(int64_t)t * cap + u];
-    }
-  __syncthreads();
-  // the pivot row's entries A(a*, c_t) and A(a*, c*)
-  for (int t = tid; t < z; t += NT)
-    sm.brow[t] = hil ? in.hilb[sm.lsum + sm.key[t]] : sb_entry(in, b, as, sm.key[t]);
-  if (tid == NT - 1) sm.apiv = hil ? in.hilb[sm.lsum + sm.rsum] : sb_entry(in, b, as, cs);
+  // the pivot entry A(a*, c*), by a thread of its own beside the gathers
+  if (tid == NT - 1)
+    sm.apiv = hil ? in.hilb[L.sum[p] + (int32_t)i + (int32_t)j + Rset.sum[q]] : sb_entry(in, b, as, cs);
   __syncthreads();
   if (tid == 0) {
     const double piv = __dsub_rn(sm.apiv, chain(sm.hps, 1, sm.hcs, 1, z));
     const double delta = 1.0 / piv;
-    sm.delta = delta;
     // 1: a usable pivot; 0: the residual formed afresh at the pivot is zero
     // (or its reciprocal overflows), so the screened value was rounding
     // noise and the bond takes no pivot; -1: not finite
@@ -1725,9 +1712,34 @@ __device__ bool append_pivot(const InstDev &in, Ctrl &cr, int b, int64_t as, int
     B.delta[z] = delta;
   }
   __syncthreads();
-  if (sm.flag != 1) return false;
-  const double delta = sm.delta;
+  return sm.flag == 1;
+}
+
+// update: P^{-1} of bond b bordered by the pivot of step z (block-wide, one
+// CTA): [[U + d U a b U, -d U a], [-d b U, d]] with a = R(:, c*) and b the
+// pivot row A(a*, c_t), t < z (Sec. 3.1.1).  Nothing but the getters reads U,
+// so it is not on the decide phase's critical path: there its two rounds of
+// chains and the z^2 update on one SM took most of a decide at high ranks
+// (100 us a sweep at ranks 256; beside the replays they cost nothing).
+__device__ __noinline__ void border_inverse(const InstDev &in, int b, int z, DecideSmem &sm) {
+  const BondDev &B = in.bond[b];
+  const int cap = B.cap;
+  const int tid = threadIdx.x;
+  const int64_t as = B.prow[z];
+  const bool ustage = z <= DEC_US;
   double *U = B.U;
+  const double delta = B.delta[z];
+  __syncthreads();
+  for (int t = tid; t < z; t += NT) {
+    sm.hcs[t] = B.hc[(int64_t)z * cap + t];
+    sm.brow[t] = sb_entry(in, b, as, B.pcol[t]);
+  }
+  if (ustage)
+    for (int x = tid; x < z * z; x += NT) {
+      const int t = x / z, u = x - t * z;
+      sm.us[x] = U[(int64_t)t * cap + u];
+    }
+  __syncthreads();
   const double *Ur = ustage ? sm.us : U;
   const int64_t ldu = ustage ? z : cap;
   // U a and b U side by side: lanes [0, z) take the rows, [z, 2z) the columns
@@ -1749,7 +1761,6 @@ __device__ bool append_pivot(const InstDev &in, Ctrl &cr, int b, int64_t as, int
   }
   if (tid == 0) U[(int64_t)z * cap + z] = delta;
   __syncthreads();
-  return true;
 }
 
 // FP64 residual of superblock entry (a, c) with the contract's chain
@@ -2575,29 +2586,21 @@ __device__ __forceinline__ void pivot_col_entries(const InstDev &in, int b, int6
 }
 
 // Alg. 4 for row a of bond b (eq. aca_approx_T_sub for pivots 0..nz-1 in
-// insertion order) by one warp: lane u keeps T(a, 32k + u), k < K, in
-// registers.  Step z runs the contract's chain over t < z on every lane from
-// broadcasts (the serial order is the contract's; the chain's FP64 latency
-// is the cost), then each lane updates its own entries - one instruction
-// per 32 entries.  A row per warp issues one FP64 instruction per chain
-// element; an SMSP's FP64 unit takes one warp instruction per ~64 cycles,
-// the latency of the chain itself.  History row z (hc, hpiv, delta) comes
-// from the triangles staged in shared memory (ST: row z at z (z - 1) / 2)
-// or from the bond's arrays (row z at z * cap), the next row loading
-// during this step when PF.
-__device__ void stage_history(const BondDev &B, int nz, int nw, ReplaySmem &rs);
-
+// insertion order) by one warp (core construction from the pivots): lane u
+// keeps T(a, 32k + u), k < K, in registers.  Step z runs the contract's chain
+// over t < z on every lane from broadcasts (the serial order is the
+// contract's), then each lane updates its own entries.  The next history row
+// loads during this step when PF.
 template <int K, bool PF>
-__device__ __noinline__ void replay_row_warp(const InstDev &in, int b, int64_t a, int nz,
-                                             ReplaySmem *st, bool valid, int nw) {
+__device__ __noinline__ void replay_row_warp(const InstDev &in, int b, int64_t a, int nz) {
   const BondDev &B = in.bond[b];
   const int lane = threadIdx.x & 31;
   const int64_t cap = B.cap;
   constexpr unsigned FULL = 0xffffffffu;
-  const double *hcb = st ? st->hc : B.hc;
-  const double *hpb = st ? st->hp : B.hpiv;
-  const double *dlb = st ? st->delta : B.delta;
-  auto off = [&](int z) -> int64_t { return st ? (int64_t)z * (z - 1) / 2 : (int64_t)z * cap; };
+  const double *hcb = B.hc;
+  const double *hpb = B.hpiv;
+  const double *dlb = B.delta;
+  auto off = [&](int z) -> int64_t { return (int64_t)z * cap; };
   double tr[K], en[K], hc[K], hp[K], hcn[K], hpn[K];
   if (in.gen == 0) {
     const int64_t nb0 = in.n[b];
@@ -2615,10 +2618,6 @@ __device__ __noinline__ void replay_row_warp(const InstDev &in, int b, int64_t a
       en[k] = t < nz ? sb_entry(in, b, a, B.pcol[t]) : 0.0;
     }
   }
-  // the staging's round trip overlaps the entries'; every replay warp of
-  // the CTA takes part in it, rows past n_b included
-  if (st) stage_history(B, nz, nw, *st);
-  if (!valid) return;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     tr[k] = 0.0;
@@ -2679,123 +2678,112 @@ __device__ __noinline__ void replay_row_warp(const InstDev &in, int b, int64_t a
   }
 }
 
-// history of bond b (nz <= 32 pivots) into the triangles of shared memory by
-// the nw replay warps of the CTA (named barrier 1: the other warps are busy
-// elsewhere); every load is issued before the first store
-__device__ void stage_history(const BondDev &B, int nz, int nw, ReplaySmem &rs) {
-  constexpr int TRI = LANE_NZ * (LANE_NZ - 1) / 2;
-  constexpr int PER = (TRI + 31) / 32;
-  const int nthr = nw * 32;
-  const int64_t cap = B.cap;
-  const int tri = nz * (nz - 1) / 2;
-  double vc[PER], vp[PER];
-#pragma unroll
-  for (int m = 0; m < PER; ++m) {
-    const int k = threadIdx.x + nthr * m;
-    vc[m] = vp[m] = 0.0;
-    if (k < tri) {
-      int z = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)k)) * 0.5f);
-      while (z * (z - 1) / 2 > k) --z;
-      while ((z + 1) * z / 2 <= k) ++z;
-      const int64_t o = (int64_t)z * cap + (k - z * (z - 1) / 2);
-      vc[m] = B.hc[o];
-      vp[m] = B.hpiv[o];
-    }
-  }
-  const double dl = (int)threadIdx.x < nz ? B.delta[threadIdx.x] : 0.0;
-  asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");  // earlier readers are done
-#pragma unroll
-  for (int m = 0; m < PER; ++m) {
-    const int k = threadIdx.x + nthr * m;
-    if (k < tri) {
-      rs.hc[k] = vc[m];
-      rs.hp[k] = vp[m];
-    }
-  }
-  if ((int)threadIdx.x < nz) rs.delta[threadIdx.x] = dl;
-  asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
-}
-
-// Alg. 4 replay of up to 32 rows of bond b at once, a row per lane: lane l
-// rebuilds T(a0 + l, 0..nz-1) from the pivot history (R(:, c_z) and T(a_z, :)
-// of every step z, delta_z) by the steps of update_row, the same FMAs in the
-// same order, its row in local memory.  A chain instruction then serves 32
-// rows: the FP64 unit, shared by the SM's warps at two FMAs per clock (an
-// instruction costs it 16 cycles whatever lanes are active), takes 1/32 of
-// the issue of a warp per row.  st: the history staged in shared memory;
-// nz <= LANE_NZ.
-__device__ __noinline__ void replay_rows_lane(const InstDev &in, int b, int64_t a0, int nrows,
-                                              int nz, const ReplaySmem *st) {
+// Alg. 4 for up to 32 / LPR rows of bond b by one warp, LPR lanes a row: the
+// steps of update_row, the same FMAs in the same order.  The contract's chain
+// of step z is z dependent FMAs; its operands T(a, t) and c_z(t) come from
+// shared memory as broadcasts, eight of each ahead of their FMAs, and one
+// chain instruction serves all the warp's rows.  A row's lanes then share the
+// step's z independent updates.  The history rows come by asynchronous copies
+// RB_STAGES - 1 steps ahead.
+// A warp issues one FP64 instruction per 63 cycles whatever its lanes do, so a
+// row of nz pivots takes nz^2 / 2 (1 + 1 / LPR) of them and the floor is
+// nz^2 / 2: eight rows a warp (LPR 4) keep the number of replay warps small
+// where rows are many and short (1024 rows of 23 pivots on the 6D n = 256
+// cross: 36 us a sweep with a row per lane, which runs its updates serially
+// and in local memory), one row a warp (LPR 32) where they are long.  (With
+// the row in registers and two shuffles per chain element a row of 256 pivots
+// took 2.3 times its floor: 200 ms of update phases in the 6D Maxwellian.)
+template <int LPR>
+__device__ __noinline__ void replay_group(const InstDev &in, int b, int64_t a0, int nrows, int nz,
+                                          double *buf) {
+  constexpr int RPW = 32 / LPR;                                // rows of the warp
+  constexpr int NZM = LPR == 32 ? RCAP : RB_SMALL;             // pivots at most
+  constexpr int LD = LPR == 32 ? RCAP : RB_SMALL + 1;          // row stride (bank spread)
   const BondDev &B = in.bond[b];
-  const int lane = threadIdx.x & 31;
-  const int64_t a = a0 + min(lane, nrows - 1);
-  const double *hcb = st->hc, *hpb = st->hp, *dlb = st->delta;
-  double tr[LANE_NZ], en[LANE_NZ];  // nz <= LANE_NZ (the staged histories)
-  // the row's entries at the pivot columns, gathered before the steps
+  const int lane = threadIdx.x & 31, s = lane % LPR, rI = min(lane / LPR, nrows - 1);
+  const int64_t cap = B.cap, a = a0 + rI;
+  double *row = buf + (lane / LPR) * LD, *ent = buf + RPW * LD + (lane / LPR) * LD;
+  double *dl = buf + 2 * RPW * LD, *hcr = dl + NZM, *hpr = hcr + RB_STAGES * NZM;
+  auto fetch = [&](int z) {
+    if (z < nz) {
+      double *c = hcr + (z % RB_STAGES) * NZM, *p = hpr + (z % RB_STAGES) * NZM;
+      for (int t = lane; t < z; t += 32) {
+        const uint32_t sc = (uint32_t)__cvta_generic_to_shared(c + t);
+        const uint32_t sp = (uint32_t)__cvta_generic_to_shared(p + t);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sc), "l"(B.hc + z * cap + t) : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sp), "l"(B.hpiv + z * cap + t) : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int z = 0; z < RB_STAGES - 1; ++z) fetch(z);
+  for (int t = lane; t < nz; t += 32) dl[t] = B.delta[t];
+  // the row's entries at the pivot columns
   if (in.gen == 0) {
     const int64_t nb0 = in.n[b];
     const int64_t p = a / nb0, i = a - p * nb0;
     const int32_t rs = left_set(in, b).sum[p] + (int32_t)i;
-    for (int z = 0; z < nz; ++z) en[z] = in.hilb[rs + B.J.sum[z]];
+    for (int t0 = s; t0 < nz; t0 += 8 * LPR) {
+      int32_t js[8];
+      double v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) js[k] = t0 + k * LPR < nz ? B.J.sum[t0 + k * LPR] : 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = t0 + k * LPR < nz ? in.hilb[rs + js[k]] : 0.0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (t0 + k * LPR < nz) ent[t0 + k * LPR] = v[k];
+    }
   } else {
-    for (int z = 0; z < nz; ++z) en[z] = sb_entry(in, b, a, B.pcol[z]);
+    for (int t = s; t < nz; t += LPR) ent[t] = sb_entry(in, b, a, B.pcol[t]);
   }
   for (int z = 0; z < nz; ++z) {
-    const int o = z * (z - 1) / 2;  // row z of the staged triangles
-    const double *hc = hcb + o, *hp = hpb + o;
-    const double ez = en[z];
-    const double dz = dlb[z];
+    fetch(z + RB_STAGES - 1);
+    asm volatile("cp.async.wait_group %0;" ::"n"(RB_STAGES - 1) : "memory");
+    __syncwarp();  // every lane's copies of step z have landed; the rows are whole
+    const double *c = hcr + (z % RB_STAGES) * NZM, *p = hpr + (z % RB_STAGES) * NZM;
     double acc = 0.0;
     int t = 0;
-    for (; t + 4 <= z; t += 4) {
-      double x[4], y[4];
+    for (; t + 8 <= z; t += 8) {
+      double x[8], y[8];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        x[k] = tr[t + k];
-        y[k] = hc[t + k];
+      for (int k = 0; k < 8; ++k) {
+        x[k] = row[t + k];
+        y[k] = c[t + k];
       }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) acc = __fma_rn(x[k], y[k], acc);
+      for (int k = 0; k < 8; ++k) acc = __fma_rn(x[k], y[k], acc);
     }
-    for (; t < z; ++t) acc = __fma_rn(tr[t], hc[t], acc);
-    const double w = __dmul_rn(dz, __dsub_rn(acc, ez));
-    for (t = 0; t < z; ++t) tr[t] = __fma_rn(w, hp[t], tr[t]);
-    tr[z] = -w;
+    for (; t < z; ++t) acc = __fma_rn(row[t], c[t], acc);
+    const double w = __dmul_rn(dl[z], __dsub_rn(acc, ent[z]));
+    __syncwarp();  // the chains have read the rows
+    for (t = s; t < z; t += LPR) row[t] = __fma_rn(w, p[t], row[t]);
+    if (s == z % LPR) row[z] = -w;
+    __syncwarp();  // step z's buffers are free for step z + RB_STAGES
   }
-  if (lane < nrows)
-    for (int t = 0; t < nz; ++t) putT(in, B, (int64_t)t * B.ldT + a, tr[t]);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  // neighbouring rows are neighbours in T: lanes take rows first
+  for (int x = lane; x < nz * RPW; x += 32) {
+    const int rr = x % RPW, t = x / RPW;
+    if (rr < nrows) putT(in, B, (int64_t)t * B.ldT + a0 + rr, buf[rr * LD + t]);
+  }
+  __syncwarp();
 }
 
-// the replays of the n_b rows that the new prefix of bond b-1 adds to bond b:
-// chunks of W <= 8 rows, a row per warp (warps 0..W-1; W <= 4 keeps one per
-// SMSP, the smallest W that gives every row a warp is taken), chunk
-// g to place (cbase + g) mod G, so that the first chunks land on distinct
-// SMs and the dependent FP64 chains run at their latency
-__device__ int32_t replay_chunks(const InstDev &in, int b, int64_t p, int nz, int32_t &cbase,
-                                 int W, ReplaySmem &rs) {
-  const int64_t nit = in.n[b];
-  const int32_t G = gridDim.x;
-  const int32_t nch = (int32_t)((nit + W - 1) / W);
-  const int warp = threadIdx.x >> 5;
-  if (warp < W) {
-    // places and cbase are in [0, G)
-    for (int32_t ch = (s_place - cbase + G) % G; ch < nch; ch += G) {
-      const int64_t i = (int64_t)ch * W + warp;
-      if (nz <= LANE_NZ) {
-        replay_row_warp<1, true>(in, b, p * nit + min(i, nit - 1), nz, &rs, i < nit, W);
-      } else if (i < nit) {
-        const int64_t a = p * nit + i;
-        if (nz <= 64)
-          replay_row_warp<2, true>(in, b, a, nz, nullptr, true, W);
-        else if (nz <= 128)
-          replay_row_warp<4, true>(in, b, a, nz, nullptr, true, W);
-        else
-          replay_row_warp<8, false>(in, b, a, nz, nullptr, true, W);
-      }
-    }
-  }
-  cbase = (int32_t)(((int64_t)cbase + nch) % G);
-  return nch;
+// rows of bond b's replays that one warp takes, and the warps they need
+__device__ __forceinline__ int replay_rows_per_warp(int nz) { return nz <= RB_SMALL ? 8 : 1; }
+__device__ __forceinline__ int replay_warps(const InstDev &in, int b, int nz) {
+  const int rpw = replay_rows_per_warp(nz);
+  return (int)((in.n[b] + rpw - 1) / rpw);
+}
+
+// group g of the replays of the n_b rows that prefix p of bond b-1 adds to bond b
+__device__ void replay_rows(const InstDev &in, int b, int64_t p, int nz, int g, double *buf) {
+  const int64_t nit = in.n[b], i0 = (int64_t)g * replay_rows_per_warp(nz);
+  if (nz <= RB_SMALL)
+    replay_group<4>(in, b, p * nit + i0, (int)min((int64_t)8, nit - i0), nz, buf);
+  else
+    replay_group<32>(in, b, p * nit + i0, 1, nz, buf);
 }
 
 __device__ void update_row(const InstDev &in, int b, int64_t a, int z) {
@@ -3315,63 +3303,53 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
       if (nadd > 0) write_plan_warp(in, *in.ctrl, rn, gridDim.x);  // next screen's tiles
     }
     if (nadd > 0) {
-      // the replays are the longest items.  One instance on a grid of two
-      // CTAs per SM: the replays go a row per lane to warps 0..RW-1 of the
-      // first places (distinct SMs, at most a quarter of them), whose SMs
-      // take no other item, so that their dependent FP64 chains do not
-      // queue behind other warps' FP64 work on the SM's shared unit; the
-      // thread-dealt items go to the other places.  Otherwise a row per
-      // warp, and the thread-dealt items start on the place after the last
-      // replay chunk.
-      const int32_t S = s_sm2;
-      int64_t lch = 0;
+      // The replays are the longest items: RB_WARPS warps of a CTA take them,
+      // the groups of all bonds numbered in order.  One instance on a grid of
+      // two CTAs per SM: they go to the first places (distinct SMs), at most
+      // three quarters of them, whose SMs take no other item, so that their
+      // dependent FP64 chains do not queue behind other warps' FP64 work on
+      // the SM's shared unit (362 cycles a step instead of 63 beside seven busy
+      // warps); the thread-dealt items go to the other places.  Otherwise the
+      // groups are dealt over all places, and the items start on the place
+      // after the last.
+      const int32_t S = s_sm2, G = gridDim.x;
+      int32_t ng = 0;
       for (int b = 1; b < in.nb; ++b)
-        if (ad[b - 1]) lch += (in.n[b] + 31) / 32;
-      const int32_t RW = (int32_t)min((int64_t)4, (lch + (S / 4) - 1) / max(1, S / 4));
-      const int32_t nsr = RW > 0 ? (int32_t)((lch + RW - 1) / RW) : 0;  // replay SMs
-      bool small = true;  // every replayed history fits the staging (rank <= LANE_NZ)
-      for (int b = 1; b < in.nb; ++b)
-        if (ad[b - 1] && rn[b] > LANE_NZ) small = false;
-      const bool iso = ra.count == 1 && S > 0 && (int32_t)gridDim.x == 2 * S && lch > 0 &&
-                       RW == 1 && nsr <= S / 4 && 2 * nsr < (int32_t)gridDim.x && small;
+        if (ad[b - 1]) ng += replay_warps(in, b, rn[b]);
+      const int32_t nsr = (ng + RB_WARPS - 1) / RB_WARPS;  // CTAs they take
+      const bool iso = ra.count == 1 && S > 0 && G == 2 * S && 4 * nsr <= 3 * S;
       int64_t gti = gt, NTI = NTOT;
+      const int32_t cb0 = iso ? 0 : (int32_t)((base / NT) % G);  // first replay place
       bool idle = false;  // a thread of a replay SM: no thread-dealt item
-      if (iso) {
-        const int32_t pl = s_place;
-        const bool rsm = pl < nsr || (pl >= S && pl < S + nsr);
-        idle = rsm;
-        if (pl < nsr && (threadIdx.x >> 5) == 0) {
-          // replay chunk g = pl of this SM (bonds in order), by warp 0 from
-          // the history staged in shared memory
-          const int64_t g = pl;
-          int64_t first = 0;
-          for (int b = 1; b < in.nb && g >= first; ++b) {
+      const int warp = threadIdx.x >> 5;
+      if (warp < RB_WARPS) {
+        for (int32_t ch = (s_place - cb0 + G) % G; ch < nsr; ch += G) {
+          int32_t g = ch * RB_WARPS + warp;
+          for (int b = 1; b < in.nb; ++b) {
             if (!ad[b - 1]) continue;
-            const int64_t nc = (in.n[b] + 31) / 32;
-            if (g < first + nc) {
-              const int64_t i0 = (g - first) * 32;
-              stage_history(in.bond[b], rn[b], 1, sm.rp);
-              replay_rows_lane(in, b, (int64_t)ro[b - 1] * in.n[b] + i0,
-                               (int)min((int64_t)32, in.n[b] - i0), rn[b], &sm.rp);
+            const int32_t nw = replay_warps(in, b, rn[b]);
+            if (g < nw) {
+              replay_rows(in, b, ro[b - 1], rn[b], g, sm.rp.buf[warp]);
+              break;
             }
-            first += nc;
+            g -= nw;
           }
         }
-        // item threads: the places of the other SMs, renumbered from 0
-        NTI = (int64_t)(gridDim.x - 2 * nsr) * NT;
-        gti = rsm ? 0 : (int64_t)(pl < S ? pl - nsr : pl - 2 * nsr) * NT + threadIdx.x;
-      } else {
-        int32_t cbase = (int32_t)((base / NT) % gridDim.x);
-        int64_t nchunks = 0, rrows = 0;
-        for (int b = 1; b < in.nb; ++b)
-          if (ad[b - 1]) rrows += in.n[b];
-        const int W = (int)min((int64_t)(NT / 32), max((int64_t)1, (rrows + gridDim.x - 1) / gridDim.x));
-        for (int b = 1; b < in.nb; ++b) {
-          if (!ad[b - 1]) continue;
-          nchunks += replay_chunks(in, b, ro[b - 1], rn[b], cbase, W, sm.rp);
-        }
-        base += nchunks * NT;
       }
+      if (iso) {
+        const int32_t pl = s_place;
+        idle = pl < nsr || (pl >= S && pl < S + nsr);
+        // item threads: the places of the other SMs, renumbered from 0
+        NTI = (int64_t)(G - 2 * nsr) * NT;
+        gti = idle ? 0 : (int64_t)(pl < S ? pl - nsr : pl - 2 * nsr) * NT + threadIdx.x;
+      } else {
+        base += (int64_t)nsr * NT;
+      }
+      // P^{-1} of every bond that added, a CTA each, counted back from the
+      // first replay: places the replays reach last
+      for (int b = 0; b < in.nb; ++b)
+        if (ad[b] && s_place == (cb0 + G - 1 - b % G) % G)
+          border_inverse(in, b, ro[b], sm.d);
       auto item0 = [&](int64_t bs) -> int64_t {
         return idle ? LLONG_MAX : first_item(bs, gti, NTI);
       };
@@ -4086,13 +4064,13 @@ __global__ void __launch_bounds__(NT, 2) k_rebuild_rows(const InstDev *inp) {
     const int64_t rows = (int64_t)(b == 0 ? 1 : in.ctrl->r[b - 1]) * in.n[b];
     for (int64_t a = ((gw - base) % nwarps + nwarps) % nwarps; a < rows; a += nwarps) {
       if (r <= 32)
-        replay_row_warp<1, true>(in, b, a, r, nullptr, true, 1);
+        replay_row_warp<1, true>(in, b, a, r);
       else if (r <= 64)
-        replay_row_warp<2, true>(in, b, a, r, nullptr, true, 1);
+        replay_row_warp<2, true>(in, b, a, r);
       else if (r <= 128)
-        replay_row_warp<4, true>(in, b, a, r, nullptr, true, 1);
+        replay_row_warp<4, true>(in, b, a, r);
       else
-        replay_row_warp<8, false>(in, b, a, r, nullptr, true, 1);
+        replay_row_warp<8, false>(in, b, a, r);
     }
     base += rows;
   }
