@@ -507,7 +507,11 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
   }
   int64_t tt_total = 0;
   if (gen->kind == TTC_GEN_TT) {
-    for (int m = 0; m <= d; ++m) I.rho[m] = gen->tt_ranks[m];
+    I.tt_small = 1;
+    for (int m = 0; m <= d; ++m) {
+      I.rho[m] = gen->tt_ranks[m];
+      if (I.rho[m] > TT_SMALL) I.tt_small = 0;
+    }
     for (int m = 0; m < d; ++m) {
       I.core_off[m] = tt_total;
       tt_total += (int64_t)I.rho[m] * n[m] * I.rho[m + 1];

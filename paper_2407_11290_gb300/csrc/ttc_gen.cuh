@@ -6,23 +6,18 @@
 namespace ttc {
 
 // TT given by cores: left-to-right product of the slices, each dot product a
-// serial FMA chain (ranks <= TT_GEN_RMAX; the vectors live in local memory).
+// serial FMA chain, four of them side by side with their loads ahead (ranks
+// <= TT_GEN_RMAX; the vectors live in local memory).
 __device__ __noinline__ double gen_tt(const InstDev &in, const int32_t *idx) {
   double v[TT_GEN_RMAX], w[TT_GEN_RMAX];
   const int d = in.d;
-  int rl = in.rho[1];
-  const double *G0 = in.tt + in.core_off[0];
-  for (int t = 0; t < rl; ++t) v[t] = G0[(int64_t)idx[0] * rl + t];
+  const int rl = in.rho[1];
+  copy8(v, in.tt + in.core_off[0] + (int64_t)idx[0] * rl, 1, rl);
   for (int m = 1; m < d; ++m) {
     const int ra = in.rho[m], rb = in.rho[m + 1];
-    const double *G = in.tt + in.core_off[m];
-    for (int q = 0; q < rb; ++q) {
-      double acc = 0.0;
-      const double *g = G + (int64_t)idx[m] * rb + q;
-      const int64_t sg = in.n[m] * rb;
-      for (int t = 0; t < ra; ++t) acc = __fma_rn(v[t], g[t * sg], acc);
-      w[q] = acc;
-    }
+    const double *G = in.tt + in.core_off[m] + (int64_t)idx[m] * rb;
+    if (m == d - 1) return chain(v, 1, G, in.n[m], ra);  // (rb = 1)
+    contract4(v, ra, G, 1, in.n[m] * rb, w, rb);
     for (int q = 0; q < rb; ++q) v[q] = w[q];
   }
   return v[0];

@@ -25,6 +25,7 @@
 namespace ttc {
 
 constexpr int TT_GEN_RMAX = 160;  // largest TT rank of a TT-cores generator
+constexpr int TT_SMALL = 16;      // ranks up to which a tile's rows share their prefix vectors
 constexpr int BM = 64, BN = 64;   // screen tile (superblock rows x columns)
 constexpr int RCAP = 256;         // largest rank capacity the kernels accept
 constexpr int GRID_CAP = 4096;    // largest persistent grid (partial-sum slots)
@@ -121,6 +122,7 @@ struct InstDev {
   const double *hilb;                // [sum_m (n_m-1) + 1] = 1/(s+1)
   const float *hilb_hi, *hilb_lo;    // its (hi, lo) FP32 split
   const double *tt;                  // TT cores
+  int32_t tt_small;                  // every rank of them is at most TT_SMALL
   int32_t rho[TTC_MAXD + 1];
   int64_t core_off[TTC_MAXD + 1];
   int32_t dx, dv;
@@ -276,6 +278,71 @@ __device__ __forceinline__ double chain(const double *x, int64_t sx, const doubl
   }
   for (; t < K; ++t) acc = __fma_rn(x[t * sx], y[t * sy], acc);
   return acc;
+}
+
+// dst[t] = src[t * s] for t < n, eight loads in flight (a plain copy loop
+// waits for each load before it issues the next)
+__device__ __forceinline__ void copy8(double *dst, const double *src, int64_t s, int n) {
+  int t = 0;
+  for (; t + 8 <= n; t += 8) {
+    double x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = src[(int64_t)(t + k) * s];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) dst[t + k] = x[k];
+  }
+  for (; t < n; ++t) dst[t] = src[(int64_t)t * s];
+}
+
+// out[o] = sum_p x[p] * col_o[p * s] for o < n, col_o = base + o * so: four
+// outputs at a time, each its own serial FMA chain in p (so the FP64 pipe
+// has four independent chains to overlap instead of one)
+__device__ __forceinline__ void contract4(const double *x, int len, const double *base, int64_t so,
+                                          int64_t s, double *out, int n) {
+  int o = 0;
+  for (; o + 4 <= n; o += 4) {
+    const double *c0 = base + (int64_t)o * so, *c1 = c0 + so, *c2 = c1 + so, *c3 = c2 + so;
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    int p = 0;
+    for (; p + 4 <= len; p += 4) {
+      // 20 loads in flight, then the 16 FMAs in chain order
+      double xv[4], v0[4], v1[4], v2[4], v3[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int64_t q = (int64_t)(p + k) * s;
+        xv[k] = x[p + k];
+        v0[k] = c0[q];
+        v1[k] = c1[q];
+        v2[k] = c2[q];
+        v3[k] = c3[q];
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        a0 = __fma_rn(xv[k], v0[k], a0);
+        a1 = __fma_rn(xv[k], v1[k], a1);
+        a2 = __fma_rn(xv[k], v2[k], a2);
+        a3 = __fma_rn(xv[k], v3[k], a3);
+      }
+    }
+    for (; p < len; ++p) {
+      const double xp = x[p];
+      const int64_t q = (int64_t)p * s;
+      a0 = __fma_rn(xp, c0[q], a0);
+      a1 = __fma_rn(xp, c1[q], a1);
+      a2 = __fma_rn(xp, c2[q], a2);
+      a3 = __fma_rn(xp, c3[q], a3);
+    }
+    out[o] = a0;
+    out[o + 1] = a1;
+    out[o + 2] = a2;
+    out[o + 3] = a3;
+  }
+  for (; o < n; ++o) {
+    const double *c = base + (int64_t)o * so;
+    double a = 0.0;
+    for (int p = 0; p < len; ++p) a = __fma_rn(x[p], c[(int64_t)p * s], a);
+    out[o] = a;
+  }
 }
 
 __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t k) {

@@ -342,7 +342,8 @@ __host__ __device__ TileGeo tile_geo_e(const InstDev &in, const Ctrl &cr, const 
 // superblocks give under a quarter wave of them on this grid while the
 // contraction is deep (rank >= 24): then 32 x 32 tiles put four times the
 // CTAs to work.  At small ranks the per-tile overhead dominates and 64 x 64
-// stays faster (measured on the 6D Hilbert workloads).
+// stays faster (measured on the 6D Hilbert workloads).  Entries from TT cores
+// cost hundreds of FMAs each: 32 x 32 tiles below four waves of 64 x 64.
 // the tile plan of the next screen at ranks r, computed by one warp of the
 // owner CTA (lane b handles bond b)
 __device__ void write_plan_warp(const InstDev &in, Ctrl &cr, const int32_t *r, int grid) {
@@ -396,7 +397,8 @@ __device__ void write_plan_warp(const InstDev &in, Ctrl &cr, const int32_t *r, i
   } else if (pieces32) {
     te = 32;
     if (act) g = tile_geo_e(in, cr, r, lane, 32);
-  } else if (!in.stored && in.prec == P_FP64 && 4 * t64 < (int64_t)grid && kmax >= 24) {
+  } else if (!in.stored && in.prec == P_FP64 &&
+             ((4 * t64 < (int64_t)grid && kmax >= 24) || (in.gen == 1 && t64 < 4 * (int64_t)grid))) {
     // 32 x 32 tiles when the candidate slots of every bond allow them
     int ok = 1;
     if (act) {
@@ -505,10 +507,58 @@ __device__ void stage_meta(const InstDev &in, int b, int64_t r0, int nr, int64_t
   }
 }
 
+// TT cores of small ranks: the product of the slices of modes 0..b is the same
+// for every entry of a row, so the tile forms it once per row (four threads a
+// row), in the operands' shared memory (the tile's contraction is done).  The
+// entries then run modes b + 1..d - 1 only: the operations and their order per
+// entry are gen_tt's.  (A product per entry from mode 0 on, its vectors in
+// local memory, took 4.0 of 5.3 ms of a 5D n = 48 cross of ranks 8.)
+__device__ __noinline__ void tt_prefix_rows(const InstDev &in, int b, int nr, ScreenSmem &sm) {
+  static_assert(2 * BM * (TT_SMALL + 1) * sizeof(double) <= sizeof(sm.op), "prefix rows");
+  double *buf = &sm.op.d.Ts[0][0];
+  const int row = threadIdx.x >> 2, s = threadIdx.x & 3;
+  __syncthreads();  // the operands are read
+  for (int m = 0; m <= b; ++m) {
+    // ping-pong, the last mode's vectors in the first half
+    double *dst = buf + ((b - m) & 1) * BM * (TT_SMALL + 1);
+    const double *src = buf + ((b - m + 1) & 1) * BM * (TT_SMALL + 1);
+    if (row < nr) {
+      const int ra = in.rho[m], rb = in.rho[m + 1];
+      const double *G = in.tt + in.core_off[m] + (int64_t)sm.ridx[row][m] * rb;
+      for (int q = s; q < rb; q += 4)
+        dst[row * (TT_SMALL + 1) + q] =
+            m == 0 ? G[q] : chain(src + row * (TT_SMALL + 1), 1, G + q, in.n[m] * rb, ra);
+    }
+    __syncthreads();
+  }
+}
+
+// an entry of a tile whose rows' prefix vectors are formed
+__device__ double tt_tail_entry(const InstDev &in, const ScreenSmem &sm, int wl, int wr, int rr,
+                                int cc) {
+  double v[TT_SMALL], w[TT_SMALL];
+  const double *x = &sm.op.d.Ts[0][0] + rr * (TT_SMALL + 1);
+  for (int j = 0; j <= wr; ++j) {
+    const int m = wl + 1 + j, ra = in.rho[m], rb = in.rho[m + 1];
+    const double *G = in.tt + in.core_off[m] + (int64_t)sm.cidx[cc][j] * rb;
+    if (j == wr) return chain(x, 1, G, in.n[m], ra);  // (rb = 1)
+    contract4(x, ra, G, 1, in.n[m] * rb, w, rb);
+    for (int q = 0; q < rb; ++q) v[q] = w[q];
+    x = v;
+  }
+  return x[0];
+}
+
+// what a tile's entries need beyond its metadata, once its contraction is done
+__device__ __forceinline__ void begin_entries(const InstDev &in, int b, int nr, ScreenSmem &sm) {
+  if (in.gen == 1 && in.tt_small) tt_prefix_rows(in, b, nr, sm);
+}
+
 __device__ __noinline__ double tile_entry(const InstDev &in, const ScreenSmem &sm, int wl, int wr,
                                              int rr, int cc) {
   if (in.gen == 0) return in.hilb[sm.srow[rr] + sm.scol[cc]];
   if (in.gen == 4) return sm.acache[rr * sm.acache_ld + cc];
+  if (in.gen == 1 && in.tt_small) return tt_tail_entry(in, sm, wl, wr, rr, cc);
   int32_t idx[TTC_MAXD];
   for (int m = 0; m <= wl; ++m) idx[m] = sm.ridx[rr][m];
   for (int m = 0; m <= wr; ++m) idx[wl + 1 + m] = sm.cidx[cc][m];
@@ -674,6 +724,7 @@ __device__ __noinline__ void screen_tile_fp64_t(const InstDev &in, int b, int K,
   stage_meta(in, b, r0, nr, c0, nc, sm);
   double acc[U][U];
   tile_chain_fp64<TE>(B, K, r0, nr, c0, nc, acc, sm);
+  if (!HIL) begin_entries(in, b, nr, sm);
   KeyBest best{0ull, LLONG_MAX, -1, -1};
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -854,6 +905,7 @@ __device__ __noinline__ void screen_tile_stored_t(const InstDev &in, int b, int 
       tile_chain_fp64<TE>(B, K, r0, nr, c0, nc, acc, sm);
     else
       tile_chain_ff<TE, MIX == 2>(B, K, r0, nr, c0, nc, fh, fl, sm);
+    if (!HIL) begin_entries(in, b, nr, sm);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int rr = ty + 16 * u;
@@ -1044,6 +1096,7 @@ __device__ __noinline__ void screen_tile_mixed_t(const InstDev &in, int b, int K
         }
     }
   }
+  if (!HIL) begin_entries(in, b, nr, sm);
   float bv = -1.f, v2 = 0.f, amax = 0.f;
   int64_t bl = LLONG_MAX;
   int32_t brow = -1, bcol = -1;
@@ -2862,72 +2915,6 @@ __device__ void choose_split(const InstDev &in, const int32_t *r, int &pL, int &
         pR = c;
       }
     }
-  }
-}
-
-// v (length s_m) <- v G_m(i) for a middle core 1 <= m <= d-2
-// dst[t] = src[t * s] for t < n, eight loads in flight (a plain copy loop
-// waits for each load before it issues the next)
-__device__ __forceinline__ void copy8(double *dst, const double *src, int64_t s, int n) {
-  int t = 0;
-  for (; t + 8 <= n; t += 8) {
-    double x[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) x[k] = src[(int64_t)(t + k) * s];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) dst[t + k] = x[k];
-  }
-  for (; t < n; ++t) dst[t] = src[(int64_t)t * s];
-}
-
-// out[o] = sum_p x[p] * col_o[p * s] for o < n, col_o = base + o * so: four
-// outputs at a time, each its own serial FMA chain in p (so the FP64 pipe
-// has four independent chains to overlap instead of one)
-__device__ __forceinline__ void contract4(const double *x, int len, const double *base, int64_t so,
-                                          int64_t s, double *out, int n) {
-  int o = 0;
-  for (; o + 4 <= n; o += 4) {
-    const double *c0 = base + (int64_t)o * so, *c1 = c0 + so, *c2 = c1 + so, *c3 = c2 + so;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    int p = 0;
-    for (; p + 4 <= len; p += 4) {
-      // 20 loads in flight, then the 16 FMAs in chain order
-      double xv[4], v0[4], v1[4], v2[4], v3[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int64_t q = (int64_t)(p + k) * s;
-        xv[k] = x[p + k];
-        v0[k] = c0[q];
-        v1[k] = c1[q];
-        v2[k] = c2[q];
-        v3[k] = c3[q];
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        a0 = __fma_rn(xv[k], v0[k], a0);
-        a1 = __fma_rn(xv[k], v1[k], a1);
-        a2 = __fma_rn(xv[k], v2[k], a2);
-        a3 = __fma_rn(xv[k], v3[k], a3);
-      }
-    }
-    for (; p < len; ++p) {
-      const double xp = x[p];
-      const int64_t q = (int64_t)p * s;
-      a0 = __fma_rn(xp, c0[q], a0);
-      a1 = __fma_rn(xp, c1[q], a1);
-      a2 = __fma_rn(xp, c2[q], a2);
-      a3 = __fma_rn(xp, c3[q], a3);
-    }
-    out[o] = a0;
-    out[o + 1] = a1;
-    out[o + 2] = a2;
-    out[o + 3] = a3;
-  }
-  for (; o < n; ++o) {
-    const double *c = base + (int64_t)o * so;
-    double a = 0.0;
-    for (int p = 0; p < len; ++p) a = __fma_rn(x[p], c[(int64_t)p * s], a);
-    out[o] = a;
   }
 }
 
