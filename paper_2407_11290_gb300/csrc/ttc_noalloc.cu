@@ -17,10 +17,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
 
+#include "ttc_split.cuh"
 #include "ttcross.h"
 
 namespace ttc {
@@ -31,7 +33,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int64_t kChunk = 4096;          // samples per partial-sum slot
+constexpr int64_t kChunk = 4096;          // samples per partial-sum slot (at most)
 constexpr int kMaxChunks = 4096;          // slots -> at most 16,777,216 samples
 constexpr int kMaxRank = 256;             // core sizes s_m: 8 register slots per lane
 constexpr int kMaxD = 16;
@@ -190,6 +192,292 @@ __global__ void __launch_bounds__(kThreads) k_chunk_sums(ErrArgs a, int64_t nchu
   }
 }
 
+// ---------------------------------------------------------------------------
+// Cores of sizes up to 32 and middle modes of up to kTcN indices: the middle
+// cores on the tensor cores, as exact split-integer products (ttc_error.cuh
+// describes the scheme), with everything a CTA needs in its shared memory.
+// A CTA takes S = 16384 / KP samples at a time (KP: the core sizes rounded up
+// to 16 or 32), keeps their vectors there as fixed-point rows (128 KB), sorts
+// the samples by each middle index in turn and multiplies every run of up to
+// 16 samples of one index by that index's core slice, whose columns a warp
+// brings to fixed point itself.
+// A warp per sample in FP64 issued one FMA per core row with half its lanes
+// idle at size 16: 6.57 ms for 1e6 samples of a 6D n = 64 TT of ranks 16 (its
+// 1.04e9 FMAs take 1.7 ms at the FP64 pipe's rate).
+constexpr int kTcThreads = 512, kTcN = 256;
+
+template <int KP>
+struct TcSmem {
+  static constexpr int S = 16384 / KP;
+  uint64_t vec[S][KP];       // fixed-point rows (interleaved pairs)
+  int32_t unit[S];           // exponents of their units
+  double res[S];             // X - X~
+  uint16_t key[S], order[S];
+  uint32_t tile[S / 16 + kTcN];
+  int32_t cnt[kTcN];
+  int32_t ntiles;
+  double red[kTcThreads / 32];
+};
+
+// the samples' order by index of mode m, and their tiles: index (bits 16..),
+// first place (bits 4..15), rows - 1 (bits 0..3)
+template <int KP>
+__device__ void tc_sort(const ErrArgs &a, int64_t k0, int ns, int m, TcSmem<KP> &sm) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int tid = threadIdx.x, n = (int)a.n[m];
+  if (tid < kTcN) sm.cnt[tid] = 0;
+  __syncthreads();
+  for (int s = tid; s < ns; s += kTcThreads) {
+    const int i = coord(a, k0 + s, m);
+    sm.key[s] = (uint16_t)i;
+    atomicAdd(&sm.cnt[i], 1);
+  }
+  __syncthreads();
+  if (tid < 32) {
+    // eight indices a lane: exclusive scans of the samples and of the tiles
+    int c[8], sum = 0, nt = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      c[q] = tid * 8 + q < n ? sm.cnt[tid * 8 + q] : 0;
+      sum += c[q];
+      nt += (c[q] + 15) / 16;
+    }
+    int is = sum, it = nt;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(FULL, is, o), v = __shfl_up_sync(FULL, it, o);
+      if (tid >= o) {
+        is += u;
+        it += v;
+      }
+    }
+    if (tid == 31) sm.ntiles = it;
+    int at = is - sum, ta = it - nt;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (tid * 8 + q < n) sm.cnt[tid * 8 + q] = at;
+      for (int o = 0; o < c[q]; o += 16)
+        sm.tile[ta++] = ((uint32_t)(tid * 8 + q) << 16) | ((uint32_t)(at + o) << 4) |
+                        (uint32_t)(min(16, c[q] - o) - 1);
+      at += c[q];
+    }
+  }
+  __syncthreads();
+  // (the order within a group is free: every row's result is its own)
+  for (int s = tid; s < ns; s += kTcThreads) sm.order[atomicAdd(&sm.cnt[sm.key[s]], 1)] = (uint16_t)s;
+  __syncthreads();
+}
+
+// one middle core: rows of the vectors times G_m(i), in place; the last one
+// meets the last core and leaves the residuals
+template <int KP>
+__device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
+  using namespace ttc;
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int KS = KP / 16, CT = KP / 8;
+  constexpr int sh = 25 - (KP == 16 ? 4 : 5);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const int K = a.s[m], N = a.s[m + 1];
+  const bool last = m == a.d - 2;
+  const int64_t ld = a.n[m] * N;
+  for (int x = warp; x < sm.ntiles; x += kTcThreads / 32) {
+    const uint32_t tl = sm.tile[x];
+    const int i = (int)(tl >> 16), at = (int)(tl >> 4) & 0xfff, rows = (int)(tl & 15) + 1;
+    const int sg = sm.order[at + min(g, rows - 1)], sg8 = sm.order[at + min(g + 8, rows - 1)];
+    uint4 A[KS][4];
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+      A[ks][0] = *reinterpret_cast<const uint4 *>(&sm.vec[sg][ks * 16 + 2 * t]);
+      A[ks][1] = *reinterpret_cast<const uint4 *>(&sm.vec[sg8][ks * 16 + 2 * t]);
+      A[ks][2] = *reinterpret_cast<const uint4 *>(&sm.vec[sg][ks * 16 + 8 + 2 * t]);
+      A[ks][3] = *reinterpret_cast<const uint4 *>(&sm.vec[sg8][ks * 16 + 8 + 2 * t]);
+    }
+    const int32_t e0 = sm.unit[sg], e1 = sm.unit[sg8];
+    __syncwarp();  // the rows are read
+    const double *G = a.core[m] + (int64_t)i * N;
+    const double *Y = a.core[a.d - 1];
+    const int64_t yn = a.n[a.d - 1];
+    int j0 = 0, j1 = 0;
+    if (last) {
+      j0 = coord(a, k0 + sg, a.d - 1);
+      j1 = coord(a, k0 + sg8, a.d - 1);
+    }
+    int64_t out[CT][4];
+    int32_t ea[CT], eb[CT];
+    int top0 = INT_MIN, top1 = INT_MIN;
+    bool bad = e0 == TC_BAD || e1 == TC_BAD;
+    double v0 = 0.0, v1 = 0.0;
+#pragma unroll
+    for (int c = 0; c < CT; ++c) {
+      if (8 * c >= N) break;
+      // the lane's entries of column u, their largest exponent over the column
+      const int u = 8 * c + g;
+      double w[KS][4];
+      int emax = 0;
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int k = ks * 16 + 2 * t + (q & 1) + 8 * (q >> 1);
+          w[ks][q] = k < K && u < N ? G[k * ld + u] : 0.0;
+        }
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) emax = max(emax, tc_expo(w[ks][q]));
+      emax = max(emax, __shfl_xor_sync(FULL, emax, 1));
+      emax = max(emax, __shfl_xor_sync(FULL, emax, 2));
+      const int32_t ge = tc_unit(emax);
+      ea[c] = __shfl_sync(FULL, ge, 8 * t);      // columns 2t, 2t + 1: lanes 4 (2t), 4 (2t + 1)
+      eb[c] = __shfl_sync(FULL, ge, 8 * t + 4);
+      bad |= ge == TC_BAD;
+      float acc[8][4];
+#pragma unroll
+      for (int l = 0; l < 8; ++l)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[l][q] = TC_MAGIC;
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) {
+        const uint4 z0 = tc_pack(tc_fix(w[ks][0], emax), tc_fix(w[ks][1], emax));
+        const uint4 z1 = tc_pack(tc_fix(w[ks][2], emax), tc_fix(w[ks][3], emax));
+        uint32_t db[8][2];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          db[j][0] = tc_digits(z0, j);
+          db[j][1] = tc_digits(z1, j);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const uint32_t da[4] = {tc_digits(A[ks][0], k), tc_digits(A[ks][1], k),
+                                  tc_digits(A[ks][2], k), tc_digits(A[ks][3], k)};
+#pragma unroll
+          for (int j = 0; k + j < 8; ++j) tc_mma(acc[k + j], da, db[j][0], db[j][1]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t hi = tc_join(tc_int(acc[0][q], true), tc_int(acc[1][q], true),
+                                   tc_int(acc[2][q], true), tc_int(acc[3][q], true));
+        const int64_t lo = tc_join(tc_int(acc[4][q], true), tc_int(acc[5][q], true),
+                                   tc_int(acc[6][q], true), tc_int(acc[7][q], true));
+        out[c][q] = (hi << sh) + ((lo + (1ll << (31 - sh))) >> (32 - sh));
+      }
+      if (last) {
+        const int ua = 8 * c + 2 * t;
+        const double ya0 = ua < N ? Y[ua * yn + j0] : 0.0, yb0 = ua + 1 < N ? Y[(ua + 1) * yn + j0] : 0.0;
+        const double ya1 = ua < N ? Y[ua * yn + j1] : 0.0, yb1 = ua + 1 < N ? Y[(ua + 1) * yn + j1] : 0.0;
+        v0 = __fma_rn(tc_real(out[c][0], e0 + ea[c] + 88 - sh), ya0, v0);
+        v0 = __fma_rn(tc_real(out[c][1], e0 + eb[c] + 88 - sh), yb0, v0);
+        v1 = __fma_rn(tc_real(out[c][2], e1 + ea[c] + 88 - sh), ya1, v1);
+        v1 = __fma_rn(tc_real(out[c][3], e1 + eb[c] + 88 - sh), yb1, v1);
+      } else {
+        if (out[c][0]) top0 = max(top0, ea[c] + 64 - __clzll(llabs(out[c][0])));
+        if (out[c][1]) top0 = max(top0, eb[c] + 64 - __clzll(llabs(out[c][1])));
+        if (out[c][2]) top1 = max(top1, ea[c] + 64 - __clzll(llabs(out[c][2])));
+        if (out[c][3]) top1 = max(top1, eb[c] + 64 - __clzll(llabs(out[c][3])));
+      }
+    }
+    bad = __any_sync(FULL, bad);
+    if (last) {
+      for (int o = 1; o < 4; o <<= 1) {
+        v0 = __dadd_rn(v0, __shfl_xor_sync(FULL, v0, o));
+        v1 = __dadd_rn(v1, __shfl_xor_sync(FULL, v1, o));
+      }
+      const double nan = __longlong_as_double(0x7FF8000000000000ll);
+      if (t == 0 && g < rows) sm.res[sg] = bad ? nan : v0;
+      if (t == 1 && g + 8 < rows) sm.res[sg8] = bad ? nan : v1;
+    } else {
+      for (int o = 1; o < 4; o <<= 1) {
+        top0 = max(top0, __shfl_xor_sync(FULL, top0, o));
+        top1 = max(top1, __shfl_xor_sync(FULL, top1, o));
+      }
+      // rescale to 62 bits below each row's largest
+#pragma unroll
+      for (int c = 0; c < CT; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (g + 8 * h >= rows) continue;
+          const int top = h ? top1 : top0;
+          int64_t x0 = 0, x1 = 0;
+          if (8 * c < N && top != INT_MIN) {
+            x0 = tc_shift(out[c][2 * h], 62 - (top - ea[c]));
+            x1 = tc_shift(out[c][2 * h + 1], 62 - (top - eb[c]));
+          }
+          *reinterpret_cast<uint4 *>(&sm.vec[h ? sg8 : sg][8 * c + 2 * t]) =
+              tc_pack((uint64_t)x0 + TC_BIAS, (uint64_t)x1 + TC_BIAS);
+        }
+      if (t == 0) {
+        if (g < rows) sm.unit[sg] = bad ? TC_BAD : top0 == INT_MIN ? 0 : e0 + 88 - sh + top0 - 62;
+        if (g + 8 < rows) sm.unit[sg8] = bad ? TC_BAD : top1 == INT_MIN ? 0 : e1 + 88 - sh + top1 - 62;
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// one slot per chunk of `chunk` samples (a multiple of S); the chunk depends on
+// the sample count alone, and a sample's residual is its own, so the result is
+// the same on any GPU
+template <int KP>
+__global__ void __launch_bounds__(kTcThreads, 1) k_tc_sums(ErrArgs a, int64_t chunk, int64_t nchunks,
+                                                           double *sums) {
+  using namespace ttc;
+  extern __shared__ __align__(16) unsigned char tc_smem_raw[];
+  TcSmem<KP> &sm = *reinterpret_cast<TcSmem<KP> *>(tc_smem_raw);
+  constexpr int S = TcSmem<KP>::S;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    double num = 0.0, den = 0.0;
+    for (int64_t k0 = c * chunk; k0 < min(a.nsamples, (c + 1) * chunk); k0 += S) {
+      const int ns = (int)min((int64_t)S, a.nsamples - k0);
+      // the first core's rows
+      for (int s = tid; s < ns; s += kTcThreads) {
+        const int K = a.s[1];
+        const double *G = a.core[0] + (int64_t)coord(a, k0 + s, 0) * K;
+        int emax = 0;
+        for (int k = 0; k < K; ++k) emax = max(emax, tc_expo(G[k]));
+        for (int k = 0; k < KP; k += 2)
+          *reinterpret_cast<uint4 *>(&sm.vec[s][k]) =
+              tc_pack(k < K ? tc_fix(G[k], emax) : TC_BIAS, k + 1 < K ? tc_fix(G[k + 1], emax) : TC_BIAS);
+        sm.unit[s] = tc_unit(emax);
+      }
+      for (int m = 1; m < a.d - 1; ++m) {
+        tc_sort<KP>(a, k0, ns, m, sm);
+        tc_core<KP>(a, k0, m, sm);
+      }
+      for (int s = tid; s < ns; s += kTcThreads) {
+        const double x = entry(a, k0 + s), e = __dsub_rn(x, sm.res[s]);
+        num = __fma_rn(e, e, num);
+        den = __fma_rn(x, x, den);
+      }
+      __syncthreads();
+    }
+    for (int pass = 0; pass < 2; ++pass) {
+      double v = pass ? den : num;
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if (lane == 0) sm.red[warp] = v;
+      __syncthreads();
+      if (tid == 0) {
+        double s = 0.0;
+        for (int i = 0; i < kTcThreads / 32; ++i) s += sm.red[i];
+        sums[2 * c + pass] = s;
+      }
+      __syncthreads();
+    }
+  }
+}
+
+template <int KP>
+cudaError_t launch_tc(const ErrArgs &a, int64_t chunk, int64_t nchunks, int nsm, double *sums,
+                      cudaStream_t cs) {
+  const void *f = (const void *)k_tc_sums<KP>;
+  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(TcSmem<KP>));
+  if (e != cudaSuccess) return e;
+  const int64_t grid = std::min<int64_t>(nchunks, nsm);
+  k_tc_sums<KP><<<(unsigned)grid, kTcThreads, sizeof(TcSmem<KP>), cs>>>(a, chunk, nchunks, sums);
+  return cudaGetLastError();
+}
+
 __global__ void __launch_bounds__(kThreads) k_finish(const double *sums, int64_t nchunks, double *out) {
   __shared__ double red[kWarps];
   double num = 0.0, den = 0.0;
@@ -305,8 +593,21 @@ extern "C" ttc_status ttcross_sampled_error_noalloc(int d, const int64_t *n, con
   ttc_status st = scratch_on(dev, cap != cudaStreamCaptureStatusNone, &sums);
   if (st != TTC_OK) return st;
   const int64_t grid = std::min<int64_t>(nchunks, (int64_t)nsm * 4);
+  // the tensor-core form: sizes that fit its shared memory, samples enough to
+  // fill the GPU's CTAs, and middle modes small enough that a CTA's 512 or 1024
+  // samples share indices
+  int64_t nmid = 0;
+  for (int m = 1; m < d - 1; ++m) nmid = std::max(nmid, n[m]);
+  const bool tc = d >= 3 && smax <= 32 && nmid <= kTcN && a.nsamples >= 16384;
+  int64_t slots = nchunks;
   cudaError_t e;
-  if (smax <= 32)
+  if (tc) {
+    int64_t chunk = smax <= 16 ? TcSmem<16>::S : TcSmem<32>::S;
+    while ((a.nsamples + chunk - 1) / chunk > kMaxChunks) chunk *= 2;
+    slots = (a.nsamples + chunk - 1) / chunk;
+    e = smax <= 16 ? launch_tc<16>(a, chunk, slots, nsm, sums, cs)
+                   : launch_tc<32>(a, chunk, slots, nsm, sums, cs);
+  } else if (smax <= 32)
     e = launch_sums<1>(a, nchunks, grid, sums, cs);
   else if (smax <= 64)
     e = launch_sums<2>(a, nchunks, grid, sums, cs);
@@ -315,7 +616,7 @@ extern "C" ttc_status ttcross_sampled_error_noalloc(int d, const int64_t *n, con
   else
     e = launch_sums<8>(a, nchunks, grid, sums, cs);
   if (e == cudaSuccess) {
-    k_finish<<<1, kThreads, 0, cs>>>(sums, nchunks, err);
+    k_finish<<<1, kThreads, 0, cs>>>(sums, slots, err);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return bad(TTC_ERR_CUDA, cudaGetErrorString(e));
