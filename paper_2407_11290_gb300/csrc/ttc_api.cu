@@ -518,14 +518,18 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     }
   }
   const int64_t hlen = gen->kind == TTC_GEN_HILBERT ? hsum + 1 : 1;
-  int64_t ncombo = 1, ncos = 1;
+  int64_t ncombo = 1, nuv = 1;
   if (gen->kind == TTC_GEN_MAXWELLIAN) {
-    ncos = 0;
+    nuv = 0;
     for (int m = 0; m < gen->dx; ++m) {
       I.mx_stride[m] = ncombo;
-      I.mx_off[m] = ncos;
+      I.mx_off[m] = nuv;
       ncombo *= n[m];
-      ncos += n[m];
+      nuv += n[m];
+    }
+    for (int m = gen->dx; m < d; ++m) {
+      I.mx_off[m] = nuv;
+      nuv += n[m];
     }
     if (ncombo > ((int64_t)1 << 27)) {
       delete h;
@@ -555,7 +559,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     double *hilb = cv.take<double>(hlen);
     double *mxc = cv.take<double>(mxtab ? ncombo : 1);
     double *mxn = cv.take<double>(mxtab ? ncombo : 1);
-    double *mxcos = cv.take<double>(ncos);
+    double *mxuv = cv.take<double>(nuv);
     float *hilb_hi = cv.take<float>(hlen);
     float *hilb_lo = cv.take<float>(hlen);
     double *tt = cv.take<double>(tt_total);
@@ -681,7 +685,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
       I.hilb = hilb;
       I.mx_coef = mxc;
       I.mx_nh = mxn;
-      I.mx_cos = mxcos;
+      I.mx_uv = mxuv;
       I.hilb_hi = hilb_hi;
       I.hilb_lo = hilb_lo;
       I.tt = tt;
@@ -810,7 +814,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
   if (mxtab) {
     if (launch_maxwellian_tables(h->d_inst, const_cast<double *>(I.mx_coef),
                                  const_cast<double *>(I.mx_nh),
-                                 const_cast<double *>(I.mx_cos)) != cudaSuccess ||
+                                 const_cast<double *>(I.mx_uv)) != cudaSuccess ||
         cudaDeviceSynchronize() != cudaSuccess)
       return cleanup(fail(TTC_ERR_CUDA, "Maxwellian tables failed"));
   }

@@ -24,19 +24,17 @@ __device__ __noinline__ double gen_tt(const InstDev &in, const int32_t *idx) {
 }
 
 // Maxwellian f(x,v) = rho(x) (2 pi T(x))^{-dv/2} exp(-|v - u(x)|^2 / (2 T(x)))
-// from the create-time tables (rho (2 pi T)^{-dv/2} and -1 / (2 T) per
-// combination of the x indices, cos x_m per x mode): one exp per entry.
+// from the create-time tables: rho (2 pi T)^{-dv/2} and -1 / (2 T) per
+// combination of the x indices, a_u cos x_m per x mode and the grid value per
+// velocity mode.  One exp per entry (with the grid values formed here, their
+// divisions cost twice what the exp does).
 __device__ __forceinline__ double gen_maxwellian_tab(const InstDev &in, const int32_t *idx) {
   int64_t combo = 0;
   for (int m = 0; m < in.dx; ++m) combo += (int64_t)idx[m] * in.mx_stride[m];
   double q = 0.0;
   for (int j = 0; j < in.dv; ++j) {
-    const int m = in.dx + j;
-    const int mu = (j + 1) % in.dx;
-    const double v = __dadd_rn(in.vmin, __dmul_rn(__dsub_rn(in.vmax, in.vmin), (double)idx[m]) /
-                                            (double)(in.n[m] - 1));
-    const double u = __dmul_rn(in.a_u, in.mx_cos[in.mx_off[mu] + idx[mu]]);
-    const double dvu = __dsub_rn(v, u);
+    const int m = in.dx + j, mu = (j + 1) % in.dx;
+    const double dvu = __dsub_rn(in.mx_uv[in.mx_off[m] + idx[m]], in.mx_uv[in.mx_off[mu] + idx[mu]]);
     q = __fma_rn(dvu, dvu, q);
   }
   return __dmul_rn(in.mx_coef[combo], exp(__dmul_rn(q, in.mx_nh[combo])));

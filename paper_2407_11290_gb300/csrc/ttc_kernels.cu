@@ -33,6 +33,21 @@ constexpr int NT = 256;  // threads per CTA
 constexpr int KC = 32;   // depth of the T / R chunks staged in shared memory
 
 
+// a Maxwellian tile's entries, per row and per column (fresh tiles; d <= MX_D):
+// the operands' shared memory is free once the contraction is done
+constexpr int MX_D = 8;
+struct MxTile {
+  double r[MX_D][BM], c[MX_D][BN];  // x, v form: mx_uv of the row's / column's modes
+  double q[BM], coef[BM], nh[BM];   // the row's leading terms of |v - u|^2; its x tables
+  int32_t rcombo[BM], ccombo[BN];   // parts of the x combination
+};
+struct XvTile {
+  double rs[BM], bm[BM], bp[BM], h[BM];  // the row's sums; 1 / (2 T) of a position whose
+                                         // velocity is the column's first mode
+  double dm[BN], dp[BN];                 // that velocity's (v - a_u)^2, (v + a_u)^2
+  double c[MX_D / 2][BN], tm[MX_D / 2][BN], tp[MX_D / 2][BN];  // the column's own pairs
+};
+
 struct ScreenSmem {
   union {
     struct {
@@ -43,6 +58,8 @@ struct ScreenSmem {
       float Th[KC][BM], Tl[KC][BM];
       float Rh[KC][BN], Rl[KC][BN];
     } f;
+    MxTile mx;
+    XvTile xv;
   } op;
   int32_t srow[BM], scol[BN];
   int64_t lrow[BM], lcol[BN];
@@ -549,15 +566,141 @@ __device__ double tt_tail_entry(const InstDev &in, const ScreenSmem &sm, int wl,
   return x[0];
 }
 
+// The Maxwellians: what an entry's exponents and factors take from its row or
+// its column alone is formed once per tile; an entry keeps its exps and a few
+// operations (the same ones in the same order: leading sums of the row, then
+// the mode pair split between row and column, then the column's).  Formed per
+// entry from local index arrays they cost as much FP64 time as the exps: 53 of
+// 56 ms of the 2d2v cross at n = 1000 went to its 4.2e8 fresh entries.
+__device__ __noinline__ void mx_tile(const InstDev &in, int b, int nr, int nc, ScreenSmem &sm) {
+  const int x = threadIdx.x & 63, side = threadIdx.x >> 6;  // 64 rows, then 64 columns
+  const int d = in.d;
+  __syncthreads();  // the operands are read
+  if (in.gen == 3) {
+    XvTile &o = sm.op.xv;
+    const int full = (b + 1) / 2;        // pairs whole in the row
+    const bool split = (b & 1) == 0;     // pair `full`: position in the row, velocity in the column
+    if (side == 0 && x < nr) {
+      double rs = 0.0, bm = 0.0, bp = 0.0;
+      for (int q = 0; q < full; ++q) {
+        const int64_t ox = in.mx_off[2 * q] + sm.ridx[x][2 * q];
+        const double h = in.mx_nh[ox];
+        const double v = in.mx_coef[in.mx_off[2 * q + 1] + sm.ridx[x][2 * q + 1]];
+        const double dm = __dsub_rn(v, in.a_u), dp = __dadd_rn(v, in.a_u);
+        rs = __dadd_rn(rs, in.mx_coef[ox]);
+        bm = __dadd_rn(bm, __dmul_rn(__dmul_rn(dm, dm), h));
+        bp = __dadd_rn(bp, __dmul_rn(__dmul_rn(dp, dp), h));
+      }
+      if (split) {
+        const int64_t ox = in.mx_off[b] + sm.ridx[x][b];
+        rs = __dadd_rn(rs, in.mx_coef[ox]);
+        o.h[x] = in.mx_nh[ox];
+      }
+      o.rs[x] = rs;
+      o.bm[x] = bm;
+      o.bp[x] = bp;
+    } else if (side == 1 && x < nc) {
+      if (split) {
+        const double v = in.mx_coef[in.mx_off[b + 1] + sm.cidx[x][0]];
+        const double dm = __dsub_rn(v, in.a_u), dp = __dadd_rn(v, in.a_u);
+        o.dm[x] = __dmul_rn(dm, dm);
+        o.dp[x] = __dmul_rn(dp, dp);
+      }
+      for (int q = full + split, k = 0; q < d / 2; ++q, ++k) {
+        const int64_t ox = in.mx_off[2 * q] + sm.cidx[x][2 * q - b - 1];
+        const double h = in.mx_nh[ox];
+        const double v = in.mx_coef[in.mx_off[2 * q + 1] + sm.cidx[x][2 * q - b]];
+        const double dm = __dsub_rn(v, in.a_u), dp = __dadd_rn(v, in.a_u);
+        o.c[k][x] = in.mx_coef[ox];
+        o.tm[k][x] = __dmul_rn(__dmul_rn(dm, dm), h);
+        o.tp[k][x] = __dmul_rn(__dmul_rn(dp, dp), h);
+      }
+    }
+  } else {
+    MxTile &o = sm.op.mx;
+    const int dx = in.dx, lead = max(0, b - dx + 1);  // velocities in the row (then so is x)
+    if (side == 0 && x < nr) {
+      int32_t combo = 0;
+      for (int m = 0; m <= b; ++m) {
+        o.r[m][x] = in.mx_uv[in.mx_off[m] + sm.ridx[x][m]];
+        if (m < dx) combo += sm.ridx[x][m] * (int32_t)in.mx_stride[m];
+      }
+      o.rcombo[x] = combo;
+      double q = 0.0;
+      for (int j = 0; j < lead; ++j) {
+        const double dvu = __dsub_rn(o.r[dx + j][x], o.r[(j + 1) % dx][x]);
+        q = __fma_rn(dvu, dvu, q);
+      }
+      o.q[x] = q;
+      if (b >= dx - 1) {
+        o.coef[x] = in.mx_coef[combo];
+        o.nh[x] = in.mx_nh[combo];
+      }
+    } else if (side == 1 && x < nc) {
+      int32_t combo = 0;
+      for (int m = b + 1; m < d; ++m) {
+        o.c[m][x] = in.mx_uv[in.mx_off[m] + sm.cidx[x][m - b - 1]];
+        if (m < dx) combo += sm.cidx[x][m - b - 1] * (int32_t)in.mx_stride[m];
+      }
+      o.ccombo[x] = combo;
+    }
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ double mx_tile_entry(const InstDev &in, const ScreenSmem &sm, int b,
+                                                int rr, int cc) {
+  if (in.gen == 3) {
+    const XvTile &o = sm.op.xv;
+    const int full = (b + 1) / 2;
+    const bool split = (b & 1) == 0;
+    double rs = o.rs[rr], bm = o.bm[rr], bp = o.bp[rr];
+    if (split) {
+      const double h = o.h[rr];
+      const double tm = __dmul_rn(o.dm[cc], h), tp = __dmul_rn(o.dp[cc], h);
+      bm = full ? __dadd_rn(bm, tm) : tm;  // (0 + t is t: t is not negative)
+      bp = full ? __dadd_rn(bp, tp) : tp;
+    }
+    for (int q = full + split, k = 0; q < in.d / 2; ++q, ++k) {
+      rs = __dadd_rn(rs, o.c[k][cc]);
+      bm = __dadd_rn(bm, o.tm[k][cc]);
+      bp = __dadd_rn(bp, o.tp[k][cc]);
+    }
+    return __dmul_rn(rs, __dadd_rn(exp(-bm), exp(-bp)));
+  }
+  const MxTile &o = sm.op.mx;
+  const int dx = in.dx;
+  double q = o.q[rr];
+  for (int j = max(0, b - dx + 1); j < in.dv; ++j) {
+    const int m = dx + j, mu = (j + 1) % dx;
+    const double v = m <= b ? o.r[m][rr] : o.c[m][cc];
+    const double dvu = __dsub_rn(v, mu <= b ? o.r[mu][rr] : o.c[mu][cc]);
+    q = __fma_rn(dvu, dvu, q);
+  }
+  double coef, nh;
+  if (b >= dx - 1) {
+    coef = o.coef[rr];
+    nh = o.nh[rr];
+  } else {
+    const int32_t combo = o.rcombo[rr] + o.ccombo[cc];
+    coef = in.mx_coef[combo];
+    nh = in.mx_nh[combo];
+  }
+  return __dmul_rn(coef, exp(__dmul_rn(q, nh)));
+}
+
 // what a tile's entries need beyond its metadata, once its contraction is done
-__device__ __forceinline__ void begin_entries(const InstDev &in, int b, int nr, ScreenSmem &sm) {
+__device__ __forceinline__ void begin_entries(const InstDev &in, int b, int nr, int nc,
+                                              ScreenSmem &sm) {
   if (in.gen == 1 && in.tt_small) tt_prefix_rows(in, b, nr, sm);
+  if ((in.gen == 2 || in.gen == 3) && in.d <= MX_D) mx_tile(in, b, nr, nc, sm);
 }
 
 __device__ __noinline__ double tile_entry(const InstDev &in, const ScreenSmem &sm, int wl, int wr,
                                              int rr, int cc) {
   if (in.gen == 0) return in.hilb[sm.srow[rr] + sm.scol[cc]];
   if (in.gen == 4) return sm.acache[rr * sm.acache_ld + cc];
+  if ((in.gen == 2 || in.gen == 3) && in.d <= MX_D) return mx_tile_entry(in, sm, wl, rr, cc);
   if (in.gen == 1 && in.tt_small) return tt_tail_entry(in, sm, wl, wr, rr, cc);
   int32_t idx[TTC_MAXD];
   for (int m = 0; m <= wl; ++m) idx[m] = sm.ridx[rr][m];
@@ -724,7 +867,7 @@ __device__ __noinline__ void screen_tile_fp64_t(const InstDev &in, int b, int K,
   stage_meta(in, b, r0, nr, c0, nc, sm);
   double acc[U][U];
   tile_chain_fp64<TE>(B, K, r0, nr, c0, nc, acc, sm);
-  if (!HIL) begin_entries(in, b, nr, sm);
+  if (!HIL) begin_entries(in, b, nr, nc, sm);
   KeyBest best{0ull, LLONG_MAX, -1, -1};
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -905,7 +1048,7 @@ __device__ __noinline__ void screen_tile_stored_t(const InstDev &in, int b, int 
       tile_chain_fp64<TE>(B, K, r0, nr, c0, nc, acc, sm);
     else
       tile_chain_ff<TE, MIX == 2>(B, K, r0, nr, c0, nc, fh, fl, sm);
-    if (!HIL) begin_entries(in, b, nr, sm);
+    if (!HIL) begin_entries(in, b, nr, nc, sm);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int rr = ty + 16 * u;
@@ -1096,7 +1239,7 @@ __device__ __noinline__ void screen_tile_mixed_t(const InstDev &in, int b, int K
         }
     }
   }
-  if (!HIL) begin_entries(in, b, nr, sm);
+  if (!HIL) begin_entries(in, b, nr, nc, sm);
   float bv = -1.f, v2 = 0.f, amax = 0.f;
   int64_t bl = LLONG_MAX;
   int32_t brow = -1, bcol = -1;
@@ -4292,7 +4435,7 @@ cudaError_t launch_tc_perm(const InstDev *d_inst, int d, int64_t blocks, uint16_
 size_t tc_plan_bytes() { return sizeof(TcPlan); }
 
 // Maxwellian tables of an instance (create time)
-__global__ void k_maxwellian_tables(const InstDev *inp, double *coef, double *nh, double *cosx) {
+__global__ void k_maxwellian_tables(const InstDev *inp, double *coef, double *nh, double *uv) {
   const InstDev &in = *inp;
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t NTOT = (int64_t)gridDim.x * blockDim.x;
@@ -4308,11 +4451,15 @@ __global__ void k_maxwellian_tables(const InstDev *inp, double *coef, double *nh
   const double two_pi = 6.283185307179586476925286766559;
   for (int m = 0; m < in.dx; ++m)
     for (int64_t i = gt; i < in.n[m]; i += NTOT)
-      cosx[in.mx_off[m] + i] = cos(__dmul_rn(two_pi, (double)i) / (double)in.n[m]);
+      uv[in.mx_off[m] + i] = __dmul_rn(in.a_u, cos(__dmul_rn(two_pi, (double)i) / (double)in.n[m]));
+  for (int m = in.dx; m < in.d; ++m)
+    for (int64_t i = gt; i < in.n[m]; i += NTOT)
+      uv[in.mx_off[m] + i] =
+          __dadd_rn(in.vmin, __dmul_rn(__dsub_rn(in.vmax, in.vmin), (double)i) / (double)(in.n[m] - 1));
 }
 
-cudaError_t launch_maxwellian_tables(const InstDev *d_inst, double *coef, double *nh, double *cosx) {
-  k_maxwellian_tables<<<152 * 4, 256>>>(d_inst, coef, nh, cosx);
+cudaError_t launch_maxwellian_tables(const InstDev *d_inst, double *coef, double *nh, double *uv) {
+  k_maxwellian_tables<<<152 * 4, 256>>>(d_inst, coef, nh, uv);
   return cudaGetLastError();
 }
 

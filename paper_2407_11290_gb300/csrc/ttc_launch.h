@@ -34,7 +34,7 @@ cudaError_t launch_user_samples(const InstDev *d_inst, int32_t *idx, cudaStream_
 cudaError_t launch_tc_perm(const InstDev *d_inst, int d, int64_t blocks, uint16_t *perm,
                            uint32_t *const *tiles);
 size_t tc_plan_bytes();
-cudaError_t launch_maxwellian_tables(const InstDev *d_inst, double *coef, double *nh, double *cosx);
+cudaError_t launch_maxwellian_tables(const InstDev *d_inst, double *coef, double *nh, double *uv);
 
 // tile geometry used to size the candidate buffer (host mirror of tile_geo)
 int64_t host_tiles(int64_t n_b, int64_t n_b1, int64_t rl, int64_t rr, int32_t pr, int32_t pc);
