@@ -184,8 +184,10 @@ typedef struct {
                                 the FP64 argmax and were re-screened in FP64 */
   int64_t unscreened_slots;  /* self-check: candidate slots a merge read that no screen
                                 wrote in the same sweep (always 0) */
-  int64_t screen_fmas;       /* algorithmic FMAs of the screens: sum over sweeps and
-                                bonds of r_k * |superblock_k| */
+  int64_t screen_fmas;       /* FMAs of the screens: sum over sweeps and bonds of
+                                r_k * |superblock_k| (stored form: r_k per entry new
+                                to a superblock, one per step applied to a carried
+                                entry) */
   int64_t error_fmas;        /* FP64 FMAs of the sampled-error evaluations (the products
                                 that run on the tensor cores are not counted) */
   double tau;                /* final tau */

@@ -94,7 +94,7 @@ struct ttc_handle {
   int32_t *ustage_idx = nullptr;
   double *ustage_val = nullptr;
   int64_t ustage_cap = 0;
-  int64_t *ucounts = nullptr;   // device [TTC_MAXD + 1]
+  int64_t *ucounts = nullptr;   // device [TTC_MAXD + 4]
   int32_t plan_te = 0, plan_qsplit = 0;  // ttcross_set_plan
   double *rebuild_scratch = nullptr;     // ttcross_rebuild_cores: pivot rows' T
   cudaEvent_t ev2 = nullptr, ev3 = nullptr;  // around the last core rebuild
@@ -171,7 +171,9 @@ ttc_status ensure_cands(ttc_handle *h, const int32_t *grid) {
     h->cand = nullptr;
   }
   // one allocation: FP64 candidates, mixed candidates, refinement list and results
-  const size_t bytes = (sizeof(Cand) + sizeof(MCand) + 2 * sizeof(int32_t) + sizeof(Cand)) *
+  // (stored form: the carried tiles' states, one per slot)
+  const size_t tbytes = h->hi.stored ? sizeof(TileState) : 0;
+  const size_t bytes = (sizeof(Cand) + sizeof(MCand) + 2 * sizeof(int32_t) + sizeof(Cand) + tbytes) *
                        (size_t)total;
   CU(cudaMalloc(&h->cand, bytes));
   // all bits set: an unwritten slot reads as row -1 with a NaN key, which the
@@ -183,11 +185,14 @@ ttc_status ensure_cands(ttc_handle *h, const int32_t *grid) {
   h->hi.refine_cand = reinterpret_cast<Cand *>(base + (sizeof(Cand) + sizeof(MCand)) * total);
   h->hi.refine_list =
       reinterpret_cast<int32_t *>(base + (2 * sizeof(Cand) + sizeof(MCand)) * total);
+  TileState *ts = reinterpret_cast<TileState *>(
+      base + (2 * sizeof(Cand) + sizeof(MCand) + 2 * sizeof(int32_t)) * total);
   int64_t off = 0;
   for (int b = 0; b < h->nb; ++b) {
     h->bond_cand_cap[b] = need[b];
     h->hi.bond[b].cand_base = off;
     h->hi.bond[b].cand_cap = need[b];
+    h->hi.bond[b].tstate = h->hi.stored ? ts + off : nullptr;
     off += need[b];
   }
   h->hi.cand = h->cand;
@@ -241,12 +246,16 @@ ttc_status user_stage(ttc_handle *h, int64_t cnt, cudaStream_t s) {
 
 // user generator: the entries that entered the superblocks in the last
 // decision (first: every entry of the rank-one superblocks) through the
-// callback into the cache, in stream order
-ttc_status user_fill(ttc_handle *h, int first, cudaStream_t s) {
+// callback into the cache, in stream order; *done and *verify: the run is over,
+// an error check is due (read with the count: one wait per sweep)
+ttc_status user_fill(ttc_handle *h, int first, cudaStream_t s, bool *done, bool *verify) {
   CU(launch_user_count(h->d_inst, first, h->ucounts, s));
-  int64_t tot = 0;
-  CU(cudaMemcpyAsync(&tot, h->ucounts + h->nb, sizeof tot, cudaMemcpyDeviceToHost, s));
+  int64_t got[3] = {};
+  CU(cudaMemcpyAsync(got, h->ucounts + h->nb, sizeof got, cudaMemcpyDeviceToHost, s));
   CU(cudaStreamSynchronize(s));
+  const int64_t tot = got[0];
+  *done = got[1] != 0;
+  *verify = got[2] != 0;
   if (tot == 0) return TTC_OK;
   ttc_status st = user_stage(h, tot, s);
   if (st) return st;
@@ -281,6 +290,9 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
   ra.persistent = (h0->opt.host_loop || user) ? 0 : 1;
   ra.mixed = 0;
   ra.sampled = 0;
+  ra.stored = 0;
+  for (int i = 0; i < count; ++i)
+    if (hs[i]->hi.stored && hs[i]->hi.prec == P_FP64) ra.stored = 1;
   ra.max_rook = 0;
   for (int i = 0; i < count; ++i)
     if (hs[i]->hi.nl > 0) {
@@ -306,17 +318,19 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
   if (user && (us = user_samples(h0, s))) return us;
   CU(launch_phase(PH_INIT1, ra, h0->grid, s));
   CU(launch_phase(PH_INIT2, ra, h0->grid, s));
-  if (user && (us = user_fill(h0, 1, s))) return us;
+  bool done = false, verify = true;
+  if (user && (us = user_fill(h0, 1, s, &done, &verify))) return us;
   CU(launch_phase(PH_INIT3, ra, h0->grid, s));
   for (int64_t it = 0; it <= ra.max_iters; ++it) {
-    bool done = true;
-    for (int i = 0; i < count; ++i) {
+    if (!user) done = true;
+    for (int i = 0; i < count && !user; ++i) {
       int32_t st = 0;
       CU(cudaMemcpyAsync(&st, &hs[i]->d_ctrl->state, sizeof st, cudaMemcpyDeviceToHost, s));
       CU(cudaStreamSynchronize(s));
       if (st != ST_DONE) done = false;
     }
     if (done) return TTC_OK;
+    if (ra.stored) CU(launch_phase(PH_BOUND, ra, h0->grid, s));
     CU(launch_phase(PH_SCREEN, ra, h0->grid, s));
     CU(launch_phase(PH_DECIDE, ra, h0->grid, s));
     if (ra.sampled) {
@@ -331,8 +345,11 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
       CU(launch_phase(PH_REFINE, ra, h0->grid, s));
       CU(launch_phase(PH_DECIDE2, ra, h0->grid, s));
     }
-    if (user && (us = user_fill(h0, 0, s))) return us;
-    CU(launch_phase(PH_VERIFY, ra, h0->grid, s));
+    if (user) {
+      if ((us = user_fill(h0, 0, s, &done, &verify))) return us;
+      if (done) return TTC_OK;
+    }
+    if (verify) CU(launch_phase(PH_VERIFY, ra, h0->grid, s));
     CU(launch_phase(PH_UPDATE, ra, h0->grid, s));
   }
   return fail(TTC_ERR_CUDA, "host-stepped run did not finish");
@@ -567,7 +584,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     double *errp = cv.take<double>(GRID_CAP);
     Cand *spart = cv.take<Cand>(GRID_CAP);
     int32_t *smid = cv.take<int32_t>(GRID_CAP);
-    int64_t *ucnt = cv.take<int64_t>(TTC_MAXD + 1);
+    int64_t *ucnt = cv.take<int64_t>(TTC_MAXD + 4);
     int32_t *eidx = cv.take<int32_t>(TTC_MAXD);
     int64_t *elin = cv.take<int64_t>(1);
     int32_t *esum = cv.take<int32_t>(1);
@@ -721,8 +738,9 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     return s;
   };
   if (o.residual == TTC_RESIDUAL_STORED) {
-    // E [ldT][ldR], ew [ldT], erow [ldR] per bond, in one allocation of its own
-    // (it dominates the footprint: 8 B per superblock entry at the rank caps)
+    // E [ldT][ldR], the steps ew [cap][ldT] and erow [cap][ldR], the step maxima
+    // and the CTAs' best keys per bond, in one allocation of its own (E dominates
+    // the footprint: 8 B per superblock entry at the rank caps)
     Carver ev;
     for (int pass = 0; pass < 2; ++pass) {
       ev.base = static_cast<char *>(h->estore);
@@ -730,12 +748,18 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
       for (int b = 0; b < d - 1; ++b) {
         BondDev &B = I.bond[b];
         double *E = ev.take<double>((size_t)(B.ldT * B.ldR));
-        double *ew = ev.take<double>((size_t)B.ldT);
-        double *er = ev.take<double>((size_t)B.ldR);
+        double *ew = ev.take<double>((size_t)(B.cap * B.ldT));
+        double *er = ev.take<double>((size_t)(B.cap * B.ldR));
+        uint32_t *wm = ev.take<uint32_t>((size_t)B.ldT);
+        uint32_t *em = ev.take<uint32_t>((size_t)B.ldR);
+        uint64_t *low = ev.take<uint64_t>(GRID_CAP);
         if (pass == 1) {
           B.E = E;
           B.ew = ew;
           B.erow = er;
+          B.wmax = wm;
+          B.emax = em;
+          B.low = low;
         }
       }
       if (pass == 0) {

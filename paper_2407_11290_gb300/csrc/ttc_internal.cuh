@@ -50,7 +50,15 @@ struct BondDev {
   double *T, *R, *U, *hpiv, *hc, *delta;
   float *Thi, *Tlo, *Rhi, *Rlo;
   int32_t *prow, *pcol;  // pivot superblock coordinates, insertion order
-  double *E, *ew, *erow; // stored-residual form (null otherwise)
+  // stored-residual form (null otherwise): the residual, and the rank-one steps
+  // of the pivots z = 1, 2, ...: step z is row z of ew [cap][ldT] (the column
+  // -E(a,c*) / E(a*,c*)) and of erow [cap][ldR] (E(a*, :)); the largest |ew| /
+  // |erow| of the newest step per row / column tile of the carried tiles (float
+  // bits, rounded up)
+  double *E, *ew, *erow;
+  uint32_t *wmax, *emax;
+  struct TileState *tstate;  // carried tiles, [row tile][column tile at the rank caps]
+  uint64_t *low;         // [GRID_CAP] each CTA's largest key among the carried tiles' entries
   double *A;             // user generator: the entries of the superblock [ldT][ldR]
   SetDev I, J;
   int64_t cand_base;     // first candidate slot of this bond
@@ -95,6 +103,8 @@ struct Ctrl {
   // pivot (ew, erow) is still to be applied by the next screen
   int32_t st_rows[TTC_MAXD], st_cols[TTC_MAXD];
   int32_t e_pend[TTC_MAXD];
+  int32_t pv_rows[TTC_MAXD], pv_cols[TTC_MAXD];  // the extent before the last screen
+  int32_t nfresh[TTC_MAXD];  // candidate slots of the fresh items (before the carried tiles')
   int32_t steal, steal2;     // stored form: items handed out by the running screen
                              // from its fresh / carried queues (cleared by the
                              // decide phase after it)
@@ -181,6 +191,18 @@ struct MCand {
   int32_t row, col;
 };
 
+// A carried tile of the stored form (ttc_kernels.cu, "lazy carried tiles").
+// The tile's entries have the steps of the pivots up to z applied; U bounds
+// |E| over the tile with every step so far, and (val, lin, row, col) is its
+// best entry when it was last brought up to date, val with every step so far.
+struct TileState {
+  float U;
+  int32_t z;
+  double val;            // FP64, or a float-float pair
+  int64_t lin;
+  int32_t row, col;
+};
+
 struct Cand {            // one screen candidate (max |E| of a tile, or top-k)
   uint64_t key;          // bits of |E| (FP64 or FP32 widened), larger wins
   int64_t lin;           // column-major linear index, smaller wins ties
@@ -215,6 +237,7 @@ struct RunArgs {
   int32_t max_iters;     // sweep cap of the launch (sum of rank caps + refinements)
   int32_t *smid;         // [grid] the SM each CTA of a persistent launch runs on
   int32_t sampled;       // some instance screens a random sample set (Alg. 1)
+  int32_t stored;        // some instance keeps stored residuals
   int32_t max_rook;      // the largest refinement round count of the instances
 };
 

@@ -75,8 +75,7 @@ struct ScreenSmem {
 };
 
 constexpr int TOPK_MAX = 16;
-// stored-residual form: candidate slots per tile (the quarters of a fresh tile;
-// a carried tile uses the first and marks the rest empty, row -2)
+// stored-residual form: items of a fresh tile that goes out in quarters
 constexpr int STORED_SLOTS = 4;
 
 constexpr int DEC_US = 32;  // pivot steps up to this rank stage U in shared memory
@@ -85,7 +84,7 @@ struct DecideSmem {
   double hcs[RCAP], hps[RCAP];  // R(:, c*) and T(a*, :) of the pivot step
   double us[DEC_US * DEC_US];   // U before the step (z <= DEC_US)
   int64_t q_nt;                 // control words of the decide item
-  int32_t q_r, q_maxr, q_prow, q_pcol;
+  int32_t q_nf, q_r, q_maxr, q_prow, q_pcol;
   double q_tau, q_xrms;
   double apiv;                  // A(a*, c*)
   int32_t sel[TOPK_MAX];
@@ -196,11 +195,26 @@ struct KeyBest {
   int32_t row, col;
 };
 
+// a before b: key, then linear index, then superblock coordinates.  (The same
+// multi-index stands twice in a superblock only where a pivot set holds one
+// twice, which takes pivots of rounding noise; then the first in row-major
+// order counts, whatever the order of the candidates.)
+__device__ __forceinline__ bool kb_better(const KeyBest &a, const KeyBest &b) {
+  if (a.key != b.key) return a.key > b.key;
+  if (a.lin != b.lin) return a.lin < b.lin;
+  return a.row < b.row || (a.row == b.row && a.col < b.col);
+}
 __device__ __forceinline__ void kb_take(KeyBest &a, const KeyBest &b) {
   if (b.row >= 0 && (a.row < 0 || key_better(b.key, b.lin, a.key, a.lin))) a = b;
 }
+// for candidates in no fixed order (the stored forms' lists)
+__device__ __forceinline__ void kb_take_any(KeyBest &a, const KeyBest &b) {
+  if (b.row >= 0 && (a.row < 0 || kb_better(b, a))) a = b;
+}
 
-// block-wide max by key; result valid in thread 0
+// block-wide max by key; result valid in thread 0 (ANY: of candidates in no
+// fixed order)
+template <bool ANY = false>
 __device__ KeyBest block_best(KeyBest v, uint64_t *sk, int64_t *sl, int32_t *sr, int32_t *sc) {
   for (int off = 16; off > 0; off >>= 1) {
     KeyBest o;
@@ -208,7 +222,7 @@ __device__ KeyBest block_best(KeyBest v, uint64_t *sk, int64_t *sl, int32_t *sr,
     o.lin = __shfl_down_sync(0xffffffffu, v.lin, off);
     o.row = __shfl_down_sync(0xffffffffu, v.row, off);
     o.col = __shfl_down_sync(0xffffffffu, v.col, off);
-    kb_take(v, o);
+    ANY ? kb_take_any(v, o) : kb_take(v, o);
   }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   __syncthreads();
@@ -217,7 +231,7 @@ __device__ KeyBest block_best(KeyBest v, uint64_t *sk, int64_t *sl, int32_t *sr,
   if (threadIdx.x == 0) {
     for (int i = 1; i < NT / 32; ++i) {
       KeyBest o{sk[i], sl[i], sr[i], sc[i]};
-      kb_take(v, o);
+      ANY ? kb_take_any(v, o) : kb_take(v, o);
     }
   }
   return v;
@@ -478,6 +492,23 @@ __host__ __device__ __forceinline__ void tile_cols(const InstDev &in, const Tile
     c0 = (int64_t)t * g.te;
     nc = min(g.te, g.cols - t * g.te);
   }
+}
+
+// the tile of one block that holds index i (the inverse of piece_tile)
+__device__ __forceinline__ int32_t piece_of(const Pieces &P, int32_t i, int32_t te) {
+  const int32_t big = P.rem * (P.q + 1);
+  if (i < big) return i / (P.q + 1) * P.tq1 + i % (P.q + 1) / te;
+  return P.rem * P.tq1 + (i - big) / P.q * P.tq0 + (i - big) % P.q / te;
+}
+__device__ __forceinline__ int32_t row_tile_of(const InstDev &in, const TileGeo &g, int b, int32_t a) {
+  if (g.pr == 0) return a / g.te;
+  const int32_t n = (int32_t)in.n[b], p = a / n;
+  return p * g.P.tpb + piece_of(g.P, a - p * n, g.te);
+}
+__device__ __forceinline__ int32_t col_tile_of(const InstDev &in, const TileGeo &g, int b, int32_t c) {
+  if (g.pc == 0) return c / g.te;
+  const int32_t n = (int32_t)in.n[b + 1], q = c / n;
+  return q * g.Q.tpb + piece_of(g.Q, c - q * n, g.te);
 }
 
 // ---------------------------------------------------------------------------
@@ -933,6 +964,9 @@ struct SV<0> {
   static __device__ __forceinline__ T step(T w, T e, T a) { return __fma_rn(w, e, a); }
   static __device__ __forceinline__ T from(double x) { return x; }
   static __device__ __forceinline__ uint64_t key(T v) { return abs_key(v); }
+  static __device__ __forceinline__ float up(T v) { return __double2float_ru(fabs(v)); }
+  static __device__ __forceinline__ double bits(T v) { return v; }
+  static __device__ __forceinline__ T unbits(double x) { return x; }
 };
 struct SVff {
   using T = float2;
@@ -963,18 +997,20 @@ struct SVff {
   static __device__ __forceinline__ uint64_t key(T v) {
     return (uint64_t)(__float_as_uint(v.x) & 0x7FFFFFFFu);
   }
+  static __device__ __forceinline__ float up(T v) { return fabsf(v.x); }
+  static __device__ __forceinline__ double bits(T v) {
+    return __hiloint2double(__float_as_int(v.y), __float_as_int(v.x));
+  }
+  static __device__ __forceinline__ T unbits(double x) {
+    return make_float2(__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x)));
+  }
 };
 template <>
 struct SV<1> : SVff {};
 template <>
 struct SV<2> : SVff {};
 
-// value of a stored entry as a double (update phase)
-__device__ __forceinline__ double sv_get(const InstDev &in, const double *E, int64_t i) {
-  if (in.prec == P_FP64) return E[i];
-  const float2 v = reinterpret_cast<const float2 *>(E)[i];
-  return __dadd_rn((double)v.x, (double)v.y);
-}
+// a double into stored form (update phase)
 __device__ __forceinline__ void sv_put(const InstDev &in, double *E, int64_t i, double x) {
   if (in.prec == P_FP64)
     E[i] = x;
@@ -982,14 +1018,15 @@ __device__ __forceinline__ void sv_put(const InstDev &in, double *E, int64_t i, 
     SVff::store(E, i, SVff::from(x));
 }
 
-// stored-residual screen of one tile (eq. aca_approx_E).  Entries inside the
-// stored extent (row < sr and column < sc) are read from E and, when the bond
-// appended a pivot in the last sweep (pend), carried through its rank-one
-// step E(a,c) = E(a,c) + ew[a] erow[c] with ew[a] = -(E(a,c*) / E(a*,c*)) and
-// erow = E(a*, :).  Entries outside it have just entered the superblock and
-// get A - chain(T(a,:), R(:,c)) with the current factors (MIX 0: FP64 chain
-// of the contract; 1 / 2: FP32 / float-float chain).  Both are written back
-// to E; the tile's best |E| is kept as in the FP64 screen.
+// stored-residual screen of one tile that reaches beyond the carried tiles (eq.
+// aca_approx_E).  Its entries inside the stored extent (row < sr and column <
+// sc) are read from E and, when the bond appended a pivot in the last sweep
+// (pend), carried through its rank-one step E(a,c) = E(a,c) + ew[a] erow[c]
+// with ew[a] = -(E(a,c*) / E(a*,c*)) and erow = E(a*, :).  Entries outside it
+// have just entered the superblock and get A - chain(T(a,:), R(:,c)) with the
+// current factors (MIX 0: FP64 chain of the contract; 1 / 2: FP32 /
+// float-float chain).  Both are written back to E; the tile's best |E| is kept
+// as in the FP64 screen.
 template <bool HIL, int TE, int MIX>
 __device__ __noinline__ void screen_tile_stored_t(const InstDev &in, int b, int K, int64_t r0,
                                                   int nr, int64_t c0, int nc, int32_t sr,
@@ -1004,42 +1041,10 @@ __device__ __noinline__ void screen_tile_stored_t(const InstDev &in, int b, int 
   const int64_t ld = B.ldR;
   __syncthreads();
   stage_meta(in, b, r0, nr, c0, nc, sm);
-  const bool carried = r0 + nr <= sr && c0 + nc <= sc;
+  const double *const ew = B.ew + (int64_t)(K - 1) * B.ldT;      // the newest step (pend)
+  const double *const erow = B.erow + (int64_t)(K - 1) * B.ldR;
   VT ev[U][U];
-  if (carried) {
-    // streaming tile: all loads first, then the rank-one step and the stores
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int rr = ty + 16 * u;
-#pragma unroll
-      for (int v = 0; v < U; ++v) {
-        const int cc = tx + 16 * v;
-        ev[u][v] = (rr < nr && cc < nc) ? V::load(B.E, (r0 + rr) * ld + c0 + cc) : V::zero();
-      }
-    }
-    if (pend) {
-      VT wa[U], er[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        wa[u] = ty + 16 * u < nr ? V::load(B.ew, r0 + ty + 16 * u) : V::zero();
-#pragma unroll
-      for (int v = 0; v < U; ++v)
-        er[v] = tx + 16 * v < nc ? V::load(B.erow, c0 + tx + 16 * v) : V::zero();
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int rr = ty + 16 * u;
-#pragma unroll
-        for (int v = 0; v < U; ++v) {
-          const int cc = tx + 16 * v;
-          if (rr < nr && cc < nc) {
-            ev[u][v] = V::step(wa[u], er[v], ev[u][v]);
-            V::store(B.E, (r0 + rr) * ld + c0 + cc, ev[u][v]);
-          }
-        }
-      }
-    }
-    __syncthreads();  // publishes the tile metadata
-  } else {
+  {
     // FP64: acc; mixed: the float-float pair (fh, fl), and E = A - T R is
     // formed in float-float too, so the mixed path leaves the FP64 pipe alone
     double acc[MIX == 0 ? U : 1][MIX == 0 ? U : 1];
@@ -1054,7 +1059,7 @@ __device__ __noinline__ void screen_tile_stored_t(const InstDev &in, int b, int 
       const int rr = ty + 16 * u;
       const int64_t a = r0 + rr;
       const bool arow = rr < nr && a < sr;
-      const VT wa = (pend && arow) ? V::load(B.ew, a) : V::zero();
+      const VT wa = (pend && arow) ? V::load(ew, a) : V::zero();
 #pragma unroll
       for (int v = 0; v < U; ++v) {
         const int cc = tx + 16 * v;
@@ -1066,7 +1071,7 @@ __device__ __noinline__ void screen_tile_stored_t(const InstDev &in, int b, int 
         VT e;
         if (arow && c < sc) {
           e = V::load(B.E, a * ld + c);
-          if (pend) e = V::step(wa, V::load(B.erow, c), e);
+          if (pend) e = V::step(wa, V::load(erow, c), e);
         } else if constexpr (MIX == 0) {
           const double A =
               HIL ? in.hilb[sm.srow[rr] + sm.scol[cc]] : tile_entry(in, sm, wl, wr, rr, cc);
@@ -1382,6 +1387,15 @@ __device__ void snap_ctrl(const Ctrl &cr, int nb, CtrlSnap &out) {
 // costly tile take fewer cheap ones.  The decide phase after the screen
 // clears the counter.
 
+// column-major linear index of superblock entry (a, c) of bond b
+__device__ __forceinline__ int64_t entry_lin(const InstDev &in, int b, int64_t a, int64_t c) {
+  const int64_t nb0 = in.n[b], nb1 = in.n[b + 1];
+  const int64_t p = a / nb0, i = a - p * nb0;
+  const int64_t q = c / nb1, j = c - q * nb1;
+  return left_set(in, b).lin[p] + i * in.stride[b] + j * in.stride[b + 1] +
+         right_set(in, b).lin[q];
+}
+
 // carried region of bond b: row tiles < tr0 and column tiles < tc0 lie in
 // the stored extent (its rows / columns are whole prefix / suffix blocks)
 __host__ __device__ __forceinline__ void carried_tiles(const InstDev &in, const TileGeo &g, int b,
@@ -1392,25 +1406,27 @@ __host__ __device__ __forceinline__ void carried_tiles(const InstDev &in, const 
 }
 
 // bookkeeping of a screen (one thread, from the CTA's staged geometry):
-// candidate slots per bond for the merge, and the statistics.  Stored form:
-// sr / sc / pend are the stored extents and pending steps, spt the slots per
-// tile; recompute form: sr = sc = null.
+// candidate slots per bond for the merge, and the statistics.  Stored form: sr /
+// sc are the stored extents, nfs the fresh items' slots, nca the carried
+// tiles' (the mixed forms; FP64 counts the candidates that it lists); the
+// carried tiles' FMAs and bytes are counted as they are brought up to date.
 __device__ void screen_bookkeeping(const InstDev &in, const int32_t *r, const TileGeo *geo,
-                                   const int32_t *sr, const int32_t *sc, const int32_t *pend,
-                                   int32_t spt) {
+                                   const int32_t *sr, const int32_t *sc, const int32_t *nfs,
+                                   const int32_t *nca) {
   Ctrl &cw = *in.ctrl;
   int64_t entries = 0, fmas = 0, fresh = 0, bytes = 0;
   for (int b = 0; b < in.nb; ++b) {
-    cw.ntiles[b] = geo[b].nrt * geo[b].nct * spt;
     const int64_t e = (int64_t)geo[b].rows * geo[b].cols;
     entries += e;
     if (sr) {
-      // carried entries cost one FMA when a rank-one step is pending
       const int64_t kept = (int64_t)sr[b] * sc[b];
       fresh += e - kept;
-      fmas += (e - kept) * r[b] + (pend[b] ? kept : 0);
-      bytes += 8 * e + (pend[b] ? 8 * kept : 0);
+      fmas += (e - kept) * r[b];
+      bytes += 8 * (e - kept);
+      cw.nfresh[b] = nfs[b];
+      if (in.prec != P_FP64) cw.ntiles[b] = nca[b];
     } else {
+      cw.ntiles[b] = geo[b].nrt * geo[b].nct;
       fresh += e;
       fmas += e * r[b];
     }
@@ -1418,154 +1434,450 @@ __device__ void screen_bookkeeping(const InstDev &in, const int32_t *r, const Ti
   cw.sweeps += 1;
   cw.entries += entries;
   cw.entries_fresh += fresh;
-  cw.stored_bytes += bytes;
-  cw.screen_fmas += fmas;
+  atomicAdd((unsigned long long *)&cw.stored_bytes, (unsigned long long)bytes);
+  atomicAdd((unsigned long long *)&cw.screen_fmas, (unsigned long long)fmas);
   cw.screened = 1;
 }
 
+// ---------------------------------------------------------------------------
+// Lazy carried tiles (FP64).  A carried tile takes part in a screen only
+// through its best |E|, and each pivot's rank-one step moves its entries by at
+// most max |ew| max |erow| over the tile.  So every carried tile keeps a bound
+// U on its |E| with every step so far, and its best entry with its exact value
+// (one step per pivot), and its entries are left as they are, with the pivot
+// index up to which their steps are applied, until U reaches L, the largest
+// value among the tiles' best entries: a tile with U < L does not hold the
+// argmax.  Then all pending steps are applied in order in one pass, the same
+// FMAs as sweep by sweep, so every stored value that is ever read is bit for
+// bit the eager one.  A screen brings up to date 58 % of the carried tiles of
+// the 6D n = 256 Hilbert cross, 42 % of a 6D Maxwellian's (n = 40) and 5 % of a
+// 2d2v run's, whose bonds reach their ranks early (counted on the oracle's
+// residuals).  It saves passes over memory, not steps, except in tiles that
+// never get that far: E's traffic goes from 241 to 44 GB and the screens from
+// 137 to 97 ms in the 6D Maxwellian at ranks 256, from 36 to 8.5 GB and 41 to
+// 37 ms in the 2d2v run, from 13.2 to 8.6 GB and 6.4 to 6.0 ms in the Hilbert
+// cross, whose screens are bound by the FP64 pipe.  The mixed forms' top-k
+// candidates need a bound on the k-th largest tile, and their steps run on a
+// pipe that is not the limit: there it cost more than it saved (5.9 against
+// 5.4 ms when it was tried), so they bring every tile up to date in every
+// screen.
+// phase_bound, before the screen, moves U and the best entries through the
+// newest step and leaves every CTA's largest best entry per bond; the update
+// phase reads single entries through their pending steps (stored_entry).
+
+// carried tiles of bond b that have a state: those carried by the last screen too
+__device__ __forceinline__ void stateful_tiles(const InstDev &in, const Ctrl &cr, const TileGeo &g,
+                                               int b, int32_t &tr, int32_t &tc) {
+  carried_tiles(in, g, b, ld_cg(cr.pv_rows[b]), ld_cg(cr.pv_cols[b]), tr, tc);
+}
+// column tiles at the run's rank caps: the stride of the states' rows; 0 if the
+// states would not fit their slots (then every carried tile is brought up to
+// date by every screen)
+__device__ __forceinline__ int32_t state_stride(const InstDev &in, const Ctrl &cr, const TileGeo &g,
+                                                int b) {
+  if (in.prec != P_FP64) return 0;
+  const int64_t capL = b == 0 ? 1 : cr.maxr[b - 1], capR = b == in.nb - 1 ? 1 : cr.maxr[b + 1];
+  const int64_t nr = g.pr > 0 ? capL * g.P.tpb : (capL * in.n[b] + g.te - 1) / g.te;
+  const int64_t nc = g.pc > 0 ? capR * g.Q.tpb : (capR * in.n[b + 1] + g.te - 1) / g.te;
+  return nr * nc <= in.bond[b].cand_cap ? (int32_t)nc : 0;
+}
+
+constexpr int LAZY_MAX = 24;  // pending steps a tile may have (a screen's pass applies them)
+
+// E(a, c) of bond b with every step up to pivot z1 applied, from its tile's state
+template <int MIX>
+__device__ __forceinline__ typename SV<MIX>::T stored_entry_t(const BondDev &B, int64_t a, int64_t c,
+                                                              int z0, int z1) {
+  using V = SV<MIX>;
+  typename V::T e = V::load(B.E, a * B.ldR + c);
+  int z = z0 + 1;
+  for (; z + 3 <= z1; z += 4) {
+    typename V::T w[4], r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      w[k] = V::load(B.ew, (z + k) * B.ldT + a);
+      r[k] = V::load(B.erow, (z + k) * B.ldR + c);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) e = V::step(w[k], r[k], e);
+  }
+  for (; z <= z1; ++z) e = V::step(V::load(B.ew, z * B.ldT + a), V::load(B.erow, z * B.ldR + c), e);
+  return e;
+}
+
+// what the update phase needs to find the state of an entry's tile
+struct LazyGeo {
+  TileGeo g;
+  int32_t tr, tc, stride;
+};
+__device__ __forceinline__ int lazy_z(const InstDev &in, const LazyGeo &q, int b, int64_t a, int64_t c,
+                                      int z1) {
+  if (q.stride == 0) return z1;
+  const int32_t tr = row_tile_of(in, q.g, b, (int32_t)a), tc = col_tile_of(in, q.g, b, (int32_t)c);
+  if (tr >= q.tr || tc >= q.tc) return z1;  // not carried by the last screen: up to date
+  return ld_cg(in.bond[b].tstate[(int64_t)tr * q.stride + tc].z);
+}
+// as a double (update phase; the mixed forms' entries are up to date)
+__device__ __forceinline__ double stored_entry(const InstDev &in, const LazyGeo &q, int b, int64_t a,
+                                               int64_t c, int z1) {
+  const BondDev &B = in.bond[b];
+  if (in.prec == P_FP64) return stored_entry_t<0>(B, a, c, lazy_z(in, q, b, a, c, z1), z1);
+  const float2 v = SV<2>::load(B.E, a * B.ldR + c);
+  return __dadd_rn((double)v.x, (double)v.y);
+}
+
+// phase: bound.  The states of the carried tiles through the newest step.
+template <int MIX>
+__device__ void bound_bond(const InstDev &in, int b, int32_t T, int32_t tc0, int32_t stride, bool pend,
+                           int z1, int64_t gt, int64_t NTOT, uint64_t &best) {
+  using V = SV<MIX>;
+  const BondDev &B = in.bond[b];
+  for (int64_t x = gt; x < T; x += NTOT) {
+    const int32_t tr = (int32_t)x / tc0, tc = (int32_t)x - tr * tc0;
+    TileState *ts = B.tstate + (int64_t)tr * stride + tc;
+    typename V::T v = V::unbits(ld_cg(ts->val));
+    if (pend) {
+      const float U = __ldcg(&ts->U);
+      const int32_t row = ld_cg(ts->row), col = ld_cg(ts->col);
+      const float dw = __uint_as_float(__ldcg(&B.wmax[tr])), de = __uint_as_float(__ldcg(&B.emax[tc]));
+      v = V::step(V::load(B.ew, (int64_t)z1 * B.ldT + row), V::load(B.erow, (int64_t)z1 * B.ldR + col), v);
+      ts->val = V::bits(v);
+      // every rounding up, and room for the rounding of the values themselves
+      ts->U = __fmul_ru(__fadd_ru(U, __fmul_ru(dw, de)), 1.000001f);
+    }
+    const uint64_t k = V::key(v);
+    best = best > k ? best : k;
+  }
+}
+
+__device__ void phase_bound(const RunArgs &ra) {
+  __shared__ CtrlSnap snap;
+  __shared__ int32_t s_tr[TTC_MAXB], s_tc[TTC_MAXB], s_str[TTC_MAXB], s_pend[TTC_MAXB];
+  __shared__ unsigned long long s_best[TTC_MAXB];
+  const int64_t NTOT = (int64_t)gridDim.x * NT;
+  const int64_t gt = (int64_t)blockIdx.x * NT + threadIdx.x;
+  for (int ii = 0; ii < ra.count; ++ii) {
+    const InstDev &in = inst(ra, ii);
+    if (!in.stored || in.prec != P_FP64) continue;
+    const Ctrl &cr = *in.ctrl;
+    snap_ctrl(cr, in.nb, snap);
+    if (snap.state != ST_SCREEN) continue;
+    if (threadIdx.x < in.nb) {
+      const int b = threadIdx.x;
+      const TileGeo g = planned_geo(in, cr, b);
+      int32_t tr, tc;
+      stateful_tiles(in, cr, g, b, tr, tc);
+      s_tr[b] = tr;
+      s_tc[b] = tc;
+      s_str[b] = state_stride(in, cr, g, b);
+      s_pend[b] = ld_cg(cr.e_pend[b]);
+      s_best[b] = 0ull;
+    }
+    __syncthreads();
+    for (int b = 0; b < in.nb; ++b) {
+      uint64_t best = 0;
+      const int32_t T = s_tr[b] * s_tc[b];
+      if (T > 0 && s_str[b] > 0) {
+        bound_bond<0>(in, b, T, s_tc[b], s_str[b], s_pend[b], snap.r[b] - 1, gt, NTOT, best);
+        for (int o = 16; o > 0; o >>= 1) {
+          const uint64_t k = __shfl_xor_sync(0xffffffffu, best, o);
+          best = best > k ? best : k;
+        }
+        if ((threadIdx.x & 31) == 0 && best) atomicMax(&s_best[b], (unsigned long long)best);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < in.nb) in.bond[threadIdx.x].low[blockIdx.x] = s_best[threadIdx.x];
+    __syncthreads();
+  }
+}
+
+// the largest of the CTAs' best keys of bond b (a warp)
+__device__ uint64_t low_key(const InstDev &in, int b) {
+  uint64_t best = 0;
+  for (int c = threadIdx.x & 31; c < (int)gridDim.x; c += 32) {
+    const uint64_t v = ld_cg(in.bond[b].low[c]);
+    best = best > v ? best : v;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t v = __shfl_xor_sync(0xffffffffu, best, o);
+    best = best > v ? best : v;
+  }
+  return best;
+}
+
 // A carried tile (TE = 32 or 64 wide) of bond b by one warp: lane l holds
-// columns l (and l + 32); rows go in rounds of 32 (TE = 32) or 8 (TE = 64),
+// columns l (and l + 32); rows go in rounds of 16 (TE = 32) or 8 (TE = 64),
 // every load of a round issued before its first use.  Then the pending
-// rank-one step E(a,c) = fma(ew[a], erow[c], E(a,c)) and its stores, and the
-// tile's best |E| (ties: lowest linear index).  The tile lies in one block
-// (p, q) of the superblock, where the linear index is
-// L.lin[p] + R.lin[q] + i stride_b + j stride_{b+1}: the ties need no loads.
-// Eight tiles per CTA are in flight instead of one.
+// rank-one steps z0 + 1..z1, E(a,c) = fma(ew_z[a], erow_z[c], E(a,c)) in
+// order, and the stores; the tile's best |E| (ties: lowest linear index) goes
+// to *out and, with the new state, to *ts (if any).  lin: the warp's shared
+// memory (mixed forms).
 template <int TE, int MIX>
 __device__ __noinline__ void screen_carried_warp(const InstDev &in, int b, int64_t r0, int nr,
-                                                 int64_t c0, int nc, int pend, Cand *out,
-                                                 int spt) {
+                                                 int64_t c0, int nc, int z0, int z1, int64_t *lin,
+                                                 Cand *out, TileState *ts) {
   using V = SV<MIX>;
   using VT = typename V::T;
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NC = TE / 32;                // columns per lane
-  constexpr int RR = TE == 32 ? 32 : (MIX == 0 ? 8 : 16);  // rows per round
+  constexpr int RR = TE == 32 ? 16 : 8;      // rows per round
   const BondDev &B = in.bond[b];
   const int lane = threadIdx.x & 31;
   const int64_t ld = B.ldR;
-  const int64_t nb0 = in.n[b], nb1 = in.n[b + 1];
-  const int64_t p = r0 / nb0, i0 = r0 - p * nb0;
-  const int64_t q = c0 / nb1, j0 = c0 - q * nb1;
-  const int64_t sb = in.stride[b], sb1 = in.stride[b + 1];
-  const int64_t lp = lane == 0 ? left_set(in, b).lin[p] : 0;
-  const int64_t rq = lane == 1 ? right_set(in, b).lin[q] : 0;
-  VT wa[NC], er[NC];
   bool cok[NC];
 #pragma unroll
-  for (int k = 0; k < NC; ++k) {
-    cok[k] = lane + 32 * k < nc;
-    wa[k] = (pend && lane + 32 * k < nr) ? V::load(B.ew, r0 + lane + 32 * k) : V::zero();
-    er[k] = (pend && cok[k]) ? V::load(B.erow, c0 + lane + 32 * k) : V::zero();
+  for (int k = 0; k < NC; ++k) cok[k] = lane + 32 * k < nc;
+  // mixed forms: the parts of the linear index, the rows' in shared memory
+  // (their 24-bit keys tie often; FP64 looks linear indices up after the
+  // rounds); the sets' parts are loaded here and used behind the first rows
+  int64_t lc[NC] = {}, lr[NC] = {};
+  uint32_t ci[NC] = {}, ri[NC] = {};
+  if constexpr (MIX != 0) {
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const uint32_t c = (uint32_t)(c0 + min(lane + 32 * k, nc - 1)), n1 = (uint32_t)in.n[b + 1], q = c / n1;
+      const uint32_t a = (uint32_t)(r0 + min(lane + 32 * k, nr - 1)), n0 = (uint32_t)in.n[b], p = a / n0;
+      ci[k] = c - q * n1;
+      ri[k] = a - p * n0;
+      lc[k] = right_set(in, b).lin[q];
+      lr[k] = left_set(in, b).lin[p];
+    }
   }
+  // the mixed forms have one pending step at most: its row and column values
+  // wait in registers, the row's by shuffle (FP64 loads them per round and step)
+  VT wa[NC], er1[NC];
+  if constexpr (MIX != 0) {
+    const double *ew = B.ew + (int64_t)z1 * B.ldT + r0, *er = B.erow + (int64_t)z1 * ld + c0;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      wa[k] = z1 > z0 ? V::load(ew, min(lane + 32 * k, nr - 1)) : V::zero();
+      er1[k] = z1 > z0 ? V::load(er, min(lane + 32 * k, nc - 1)) : V::zero();
+    }
+  }
+  // (row brr, column lane + 32 bkk) the lane's first best; tied (FP64): another
+  // of its entries has the same key (rare; the linear indices decide after the
+  // rounds, where they cost the loop no registers)
   uint64_t bk = 0;
-  int64_t bl = LLONG_MAX;
-  int brr = -1, bcc = 0;
-  // mixed forms: the rounds stay a loop; unrolled, their float-float steps
-  // make a body large enough to compete for the instruction cache with the
-  // fresh tiles of the SM's other CTA (the FP64 body is small)
-#pragma unroll(MIX == 0 ? TE / RR : 1)
-  for (int r1 = 0; r1 < TE; r1 += RR) {
+  int brr = -1, bkk = 0;
+  bool tied = false;
+  // the rounds stay a loop: unrolled, the body is large enough to compete for
+  // the instruction cache with the fresh tiles of the SM's other CTA
+  const int rl = nr - 1;
+  const int cl = min(lane, nc - 1), cl1 = min(lane + 32, nc - 1);  // columns, clamped
+#pragma unroll 1
+  for (int r1 = 0; r1 < nr; r1 += RR) {
     VT ev[RR][NC];
-#pragma unroll
-    for (int rr = 0; rr < RR; ++rr)
-#pragma unroll
-      for (int k = 0; k < NC; ++k)
-        ev[rr][k] = (cok[k] && r1 + rr < nr) ? V::load(B.E, (r0 + r1 + rr) * ld + c0 + lane + 32 * k)
-                                             : V::zero();
-    if (pend) {
+    {
+      // rows past the tile read its last row again
+      const double *E = B.E + (r0 + r1) * ld + c0;
 #pragma unroll
       for (int rr = 0; rr < RR; ++rr) {
-        const int row = r1 + rr;
-        VT w;
-        if constexpr (MIX == 0) {
-          w = __shfl_sync(FULL, wa[row >> 5], row & 31);
-        } else {
-          w.x = __shfl_sync(FULL, wa[row >> 5].x, row & 31);
-          w.y = __shfl_sync(FULL, wa[row >> 5].y, row & 31);
-        }
-#pragma unroll
-        for (int k = 0; k < NC; ++k)
-          if (row < nr && cok[k]) {
-            ev[rr][k] = V::step(w, er[k], ev[rr][k]);
-            V::store(B.E, (r0 + row) * ld + c0 + lane + 32 * k, ev[rr][k]);
-          }
+        ev[rr][0] = V::load(E, cl);
+        if (NC == 2) ev[rr][NC - 1] = V::load(E, cl1);
+        if (r1 + rr < rl) E += ld;
       }
     }
-    // the lane's best: rows in order, only a larger key replaces within a
-    // column (the earlier row has the lower linear index); across its
-    // columns the linear index decides
+    if constexpr (MIX != 0) {
+      if (r1 == 0) {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+          lc[k] += (int64_t)ci[k] * in.stride[b + 1];
+          lin[lane + 32 * k] = lr[k] + (int64_t)ri[k] * in.stride[b];
+        }
+        __syncwarp();
+      }
+    }
+    if constexpr (MIX != 0) {
+      if (z1 > z0) {
+#pragma unroll
+        for (int rr = 0; rr < RR; ++rr) {
+          const int row = r1 + rr;  // (the halves of wa: r1 is a multiple of RR <= 32)
+          VT w;
+          w.x = __shfl_sync(FULL, NC == 2 && r1 >= 32 ? wa[NC - 1].x : wa[0].x, row & 31);
+          w.y = __shfl_sync(FULL, NC == 2 && r1 >= 32 ? wa[NC - 1].y : wa[0].y, row & 31);
+#pragma unroll
+          for (int k = 0; k < NC; ++k) ev[rr][k] = V::step(w, er1[k], ev[rr][k]);
+        }
+      }
+    } else for (int z = z0 + 1; z <= z1; ++z) {
+      const double *ew = B.ew + (int64_t)z * B.ldT + r0 + r1;
+      const double *er = B.erow + (int64_t)z * ld + c0;
+      VT e[NC];
+      e[0] = V::load(er, cl);
+      if (NC == 2) e[NC - 1] = V::load(er, cl1);
+#pragma unroll
+      for (int rr = 0; rr < RR; ++rr) {
+        const VT w = V::load(ew, min(rr, rl - r1));
+#pragma unroll
+        for (int k = 0; k < NC; ++k) ev[rr][k] = V::step(w, e[k], ev[rr][k]);
+      }
+    }
+    if (z1 > z0) {
+      double *E = B.E + (r0 + r1) * ld + c0;
+#pragma unroll
+      for (int rr = 0; rr < RR; ++rr) {
+        if (r1 + rr <= rl) {
+          if (cok[0]) V::store(E, lane, ev[rr][0]);
+          if (NC == 2 && cok[NC - 1]) V::store(E, lane + 32, ev[rr][NC - 1]);
+        }
+        E += ld;
+      }
+    }
 #pragma unroll
     for (int rr = 0; rr < RR; ++rr)
 #pragma unroll
       for (int k = 0; k < NC; ++k) {
-        const int row = r1 + rr;
-        if (row < nr && cok[k]) {
-          const uint64_t key = V::key(ev[rr][k]);
-          if (brr < 0 || key >= bk) {
-            const int64_t l = (i0 + row) * sb + (j0 + lane + 32 * k) * sb1;
-            if (brr < 0 || key > bk || l < bl) {
-              bk = key;
-              bl = l;
-              brr = row;
-              bcc = lane + 32 * k;
-            }
-          }
+        if (r1 + rr > rl || !cok[k]) continue;
+        const uint64_t key = V::key(ev[rr][k]);
+        bool take = brr < 0 || key > bk;
+        if constexpr (MIX == 0)
+          tied = !take && (tied || key == bk);
+        else if (!take && key == bk)
+          take = lin[r1 + rr] + lc[k] < lin[brr] + lc[bkk];
+        if (take) {
+          bk = key;
+          brr = r1 + rr;
+          bkk = k;
         }
       }
   }
+  int bcc = lane + 32 * bkk;
+  int64_t bl = LLONG_MAX;
+  if (brr >= 0) bl = MIX == 0 ? entry_lin(in, b, r0 + brr, c0 + bcc) : lin[brr] + lc[bkk];
+  if (MIX == 0 && tied) {
+#pragma unroll 1
+    for (int row = brr; row < nr; ++row)
+#pragma unroll 1
+      for (int col = lane; col < nc; col += 32) {
+        if (V::key(V::load(B.E, (r0 + row) * ld + c0 + col)) != bk) continue;
+        const int64_t l = entry_lin(in, b, r0 + row, c0 + col);
+        if (l < bl) {
+          bl = l;
+          brr = row;
+          bcc = col;
+        }
+      }
+  }
+  const int mine = brr < 0 ? -1 : brr * 64 + bcc;
   for (int off = 16; off > 0; off >>= 1) {
     const uint64_t ok = __shfl_xor_sync(FULL, bk, off);
     const int64_t ol = __shfl_xor_sync(FULL, bl, off);
     const int orr = __shfl_xor_sync(FULL, brr, off);
     const int oc = __shfl_xor_sync(FULL, bcc, off);
-    if (orr >= 0 && (brr < 0 || ok > bk || (ok == bk && ol < bl))) {
+    if (orr >= 0 && (brr < 0 || kb_better(KeyBest{ok, ol, orr, oc}, KeyBest{bk, bl, brr, bcc}))) {
       bk = ok;
       bl = ol;
       brr = orr;
       bcc = oc;
     }
   }
-  const int64_t LP = __shfl_sync(FULL, lp, 0), RQ = __shfl_sync(FULL, rq, 1);
-  if (lane == 0) {
-    out->key = bk;
-    out->lin = LP + RQ + bl;
-    out->row = (int32_t)(r0 + brr);
-    out->col = (int32_t)(c0 + bcc);
-    for (int k = 1; k < spt; ++k) out[k] = Cand{0ull, LLONG_MAX, -2, -2};
+  if (lane == 0) *out = Cand{bk, bl, (int32_t)(r0 + brr), (int32_t)(c0 + bcc)};
+  if (ts && mine == brr * 64 + bcc) {  // the lane that holds (and stored) the best
+    const VT bv = V::load(B.E, (r0 + brr) * ld + c0 + bcc);
+    *ts = TileState{V::up(bv), z1, V::bits(bv), bl, (int32_t)(r0 + brr), (int32_t)(c0 + bcc)};
   }
+  __syncwarp();
 }
 
 __device__ __forceinline__ void carried_warp(const InstDev &in, int te, int b, int64_t r0, int nr,
-                                             int64_t c0, int nc, int pend, Cand *out, int spt) {
+                                             int64_t c0, int nc, int z0, int z1, int64_t *lin,
+                                             Cand *out, TileState *ts) {
   if (in.prec == P_FP64) {
     if (te == 32)
-      screen_carried_warp<32, 0>(in, b, r0, nr, c0, nc, pend, out, spt);
+      screen_carried_warp<32, 0>(in, b, r0, nr, c0, nc, z0, z1, lin, out, ts);
     else
-      screen_carried_warp<64, 0>(in, b, r0, nr, c0, nc, pend, out, spt);
+      screen_carried_warp<64, 0>(in, b, r0, nr, c0, nc, z0, z1, lin, out, ts);
   } else {
     if (te == 32)
-      screen_carried_warp<32, 2>(in, b, r0, nr, c0, nc, pend, out, spt);
+      screen_carried_warp<32, 2>(in, b, r0, nr, c0, nc, z0, z1, lin, out, ts);
     else
-      screen_carried_warp<64, 2>(in, b, r0, nr, c0, nc, pend, out, spt);
+      screen_carried_warp<64, 2>(in, b, r0, nr, c0, nc, z0, z1, lin, out, ts);
+  }
+}
+
+// carried tiles [t0, t1) of bond b by one warp (t1 - t0 <= 32; tc0 column tiles):
+// a lane per tile finds the pivot its entries are at and whether a candidate
+// may lie in it; those tiles are brought up to pivot cur.  low: the bond's L.
+// cand: the bond's slots after the fresh items'; FP64 lists its candidates
+// there (a place each from ntiles, one atomic per run), the mixed forms use a
+// slot per tile.
+__device__ __forceinline__ void carried_run(const InstDev &in, const TileGeo &g, int b, int32_t t0,
+                                            int32_t t1, int32_t tc0, int32_t cur, int32_t pend,
+                                            int32_t ptr, int32_t ptc, int32_t stride, uint64_t low,
+                                            int64_t *lin, Cand *cand, unsigned long long &fma,
+                                            unsigned long long &bytes) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const bool has = t0 + lane < t1;
+  int32_t zt = has ? (pend ? cur - 1 : cur) : -1;  // (first time: fresh in the last screen)
+  unsigned todo = __ballot_sync(FULL, has);
+  if (in.prec == P_FP64) {
+    bool asis = false;  // up to date as it stands, and its best entry is a candidate
+    uint64_t key = 0;
+    const TileState *ts = nullptr;
+    if (has) {
+      const int32_t tr = (t0 + lane) / tc0, tc = t0 + lane - tr * tc0;
+      if (tr < ptr && tc < ptc) {
+        ts = in.bond[b].tstate + (int64_t)tr * stride + tc;
+        const int32_t z = ld_cg(ts->z);
+        const float U = __ldcg(&ts->U);
+        key = SV<0>::key(ld_cg(ts->val));
+        const bool skip = (double)U < __longlong_as_double((long long)low);
+        asis = z == cur && key >= low;
+        zt = (z == cur || (skip && cur - z < LAZY_MAX)) ? -1 : z;
+      }
+    }
+    todo = __ballot_sync(FULL, zt >= 0);
+    const unsigned kept = __ballot_sync(FULL, asis);
+    if (!(todo | kept)) return;
+    int32_t at = 0;
+    if (lane == 0) at = atomicAdd(&in.ctrl->ntiles[b], __popc(todo) + __popc(kept));
+    cand += __shfl_sync(FULL, at, 0);
+    if (asis)
+      cand[__popc(todo) + __popc(kept & ((1u << lane) - 1))] =
+          Cand{key, ld_cg(ts->lin), ld_cg(ts->row), ld_cg(ts->col)};
+  } else {
+    cand += t0;
+  }
+  unsigned long long nf = 0, nb = 0;
+  for (; todo; todo &= todo - 1, ++cand) {
+    const int x = __ffs(todo) - 1;
+    const int z0 = __shfl_sync(FULL, zt, x);
+    const int32_t tr = (t0 + x) / tc0, tc = t0 + x - tr * tc0;
+    int64_t r0, c0;
+    int nr, nc;
+    tile_rows(in, g, b, tr, r0, nr);
+    tile_cols(in, g, b, tc, c0, nc);
+    carried_warp(in, g.te, b, r0, nr, c0, nc, z0, cur, lin, cand,
+                 stride > 0 ? in.bond[b].tstate + (int64_t)tr * stride + tc : nullptr);
+    const unsigned long long e = (unsigned long long)nr * nc;
+    nf += e * (unsigned long long)(cur - z0);
+    nb += (cur > z0 ? 16 : 8) * e;
+  }
+  if (lane == 0) {
+    atomicAdd(&fma, nf);
+    atomicAdd(&bytes, nb);
   }
 }
 
 // The stored screen of one instance.  Work items come from two queues:
 //   A: tiles new to a superblock (fresh: A - T R, r_k FMAs per entry, FP64
-//      pipe or FP32 pipe in the mixed forms), one tile (or quarter) per
-//      block item;
-//   B: carried tiles (one load, one FMA when a rank-one step is pending, one
-//      store per entry: memory-bound).  On bonds cut into subtensor pieces a
-//      carried tile lies in one block (p, q) and is screened by one warp, and
-//      an item is eight such tiles, one per warp; elsewhere an item is one
-//      tile screened by the whole CTA.
+//      pipe or FP32 pipe in the mixed forms), one tile (or quarter) per item;
+//   B: carried tiles, a run of them to a warp at a time: its lanes look up
+//      which of them a candidate may lie in, and the warp brings those up to
+//      date (one load, one FMA per pending step and one store per entry).
 // The CTAs of the first half of the SM-spread order (one per SM) start on A,
 // the others on B, so that every SM keeps its FP64 / FP32 pipe and its
 // memory path busy at once; a CTA whose queue runs dry moves to the other.
 // Place s takes the first item of its queue implicitly, later items come
 // from the queue's counter, fetched when an item starts so that the atomic's
-// round trip overlaps the tile.  The decide phase clears both counters.
-constexpr int CW = NT / 32;  // carried warp tiles per item
+// round trip overlaps it.  The decide phase clears both counters.  A run is a
+// sixth of a warp's even share (at most 32 tiles: its lanes; a warp's tile
+// takes 40 us beside seven others and a CTA on fresh tiles, so runs of eight
+// tiles per CTA left tails of half a sweep).
+// A bond's candidate slots are its fresh items' (nfresh), then its carried
+// tiles' (ntiles).
 
 __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, PhaseSmem &sm) {
   const Ctrl &cr = *in.ctrl;
@@ -1574,153 +1886,152 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
   __shared__ TileGeo s_geo[TTC_MAXB];
   __shared__ int32_t s_sr[TTC_MAXB], s_sc[TTC_MAXB], s_pend[TTC_MAXB];
   __shared__ int32_t s_tr0[TTC_MAXB], s_tc0[TTC_MAXB];
-  __shared__ int32_t s_warp[TTC_MAXB];  // carried tiles go to single warps
-  __shared__ int32_t s_item, s_q;
+  __shared__ int32_t s_ptr[TTC_MAXB], s_ptc[TTC_MAXB], s_str[TTC_MAXB];  // tiles with a state
+  __shared__ uint64_t s_low[TTC_MAXB];
+  __shared__ int32_t s_item;
+  __shared__ unsigned long long s_fma, s_byte;
   __syncthreads();
+  if (threadIdx.x == 0) s_fma = s_byte = 0ull;
   if (threadIdx.x < in.nb) {
     const int b = threadIdx.x;
     const TileGeo g = planned_geo(in, cr, b);
     const int32_t sr = ld_cg(cr.st_rows[b]);
     const int32_t sc = ld_cg(cr.st_cols[b]);
-    int32_t tr0, tc0;
+    int32_t tr0, tc0, ptr, ptc;
     carried_tiles(in, g, b, sr, sc, tr0, tc0);
+    stateful_tiles(in, cr, g, b, ptr, ptc);
     s_geo[b] = g;
     s_sr[b] = sr;
     s_sc[b] = sc;
     s_pend[b] = ld_cg(cr.e_pend[b]);
     s_tr0[b] = tr0;
     s_tc0[b] = tc0;
-    s_warp[b] = g.pr > 0 && g.pc > 0;
+    s_str[b] = state_stride(in, cr, g, b);
+    s_ptr[b] = s_str[b] > 0 ? ptr : 0;
+    s_ptc[b] = s_str[b] > 0 ? ptc : 0;
   }
   __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int b = warp; b < in.nb; b += NT / 32) {
+    const uint64_t k = s_ptr[b] * s_ptc[b] > 0 ? low_key(in, b) : 0;
+    if (lane == 0) s_low[b] = k;
+  }
   // with fewer fresh tiles than CTAs, fresh tiles go out as quarters
-  // (32 x 32) so that their work spreads over four times as many CTAs;
-  // candidate slots are then STORED_SLOTS per tile, else one
-  int32_t nf = 0, nB = 0;
+  // (32 x 32) so that their work spreads over four times as many CTAs
+  int32_t nf = 0, nc_all = 0;
   for (int b = 0; b < in.nb; ++b) {
     const int32_t nt = s_geo[b].nrt * s_geo[b].nct, nc = s_tr0[b] * s_tc0[b];
     nf += nt - nc;
-    nB += s_warp[b] ? (nc + CW - 1) / CW : nc;
+    nc_all += nc;
   }
-  const bool quarters = s_geo[0].te == 64 && nf < (int32_t)gridDim.x;
-  const int32_t spt = quarters ? STORED_SLOTS : 1;  // slots per tile
-  const int32_t nA = spt * nf;
   const int32_t G = gridDim.x;
+  const int32_t run = max(1, min(32, nc_all / (6 * G * (NT / 32))));  // tiles of a B item
+  int32_t nB = 0;
+  for (int b = 0; b < in.nb; ++b) nB += (s_tr0[b] * s_tc0[b] + run - 1) / run;
+  const bool quarters = s_geo[0].te == 64 && nf < (int32_t)gridDim.x;
+  const int32_t spt = quarters ? STORED_SLOTS : 1;  // items per tile
+  const int32_t nA = spt * nf;
   const int32_t qs = ld_cg(cr.qsplit);  // eighths of the CTAs that start on A (0: half)
   const int32_t HA = nA == 0 ? 0 : nB == 0 ? G : qs > 0 ? max(1, min(G - 1, G * qs / 8))
                                                          : (G + 1) / 2;
-  const int32_t N[2] = {nA, nB}, H[2] = {HA, G - HA};
-  if (blockIdx.x == 0 && threadIdx.x == 0) screen_bookkeeping(in, r, s_geo, s_sr, s_sc, s_pend, spt);
-  // thread 0 keeps the queue, whether it has switched, and the next item
-  int q0 = s_place < HA ? 0 : 1;
-  bool switched = false;
-  if (threadIdx.x == 0) {
-    int32_t j = q0 == 0 ? s_place : s_place - HA;
-    if (j >= N[q0]) {
-      switched = true;
-      q0 ^= 1;
-      j = H[q0] + atomicAdd(ctr[q0], 1);
-    }
-    s_q = q0;
-    s_item = j < N[q0] ? j : -1;
+  const int32_t HB = (G - HA) * (NT / 32);  // warps that start on B
+  __shared__ int32_t s_nf[TTC_MAXB], s_nc[TTC_MAXB];  // slots of the fresh items, carried tiles
+  if (threadIdx.x < in.nb) {
+    const int b = threadIdx.x, nc = s_tr0[b] * s_tc0[b];
+    s_nc[b] = nc;
+    s_nf[b] = (s_geo[b].nrt * s_geo[b].nct - nc) * spt;
   }
-  int32_t nxt = 0;
-  for (;;) {
-    __syncthreads();
-    const int qq = s_q;
-    int32_t j = s_item;
-    __syncthreads();
-    if (j < 0) break;
-    if (threadIdx.x == 0) nxt = H[qq] + atomicAdd(ctr[qq], 1);
-    if (qq == 0) {
-      // a fresh tile (or quarter q of it)
-      const int32_t qt = j % spt;
-      j /= spt;
-      for (int b = 0; b < in.nb; ++b) {
-        const TileGeo &g = s_geo[b];
-        const int32_t tr0 = s_tr0[b], tc0 = s_tc0[b];
-        const int32_t cnt = g.nrt * g.nct - tr0 * tc0;
-        if (j >= cnt) {
-          j -= cnt;
-          continue;
-        }
-        int32_t tr, tc;
-        if (j < tr0 * (g.nct - tc0)) {
-          // new columns of the stored rows
-          tr = j / (g.nct - tc0);
-          tc = tc0 + (j - tr * (g.nct - tc0));
-        } else {
-          // new rows, every column
-          const int32_t u = j - tr0 * (g.nct - tc0);
-          tr = tr0 + u / g.nct;
-          tc = u - (tr - tr0) * g.nct;
-        }
-        int64_t r0, c0;
-        int nr, nc;
-        tile_rows(in, g, b, tr, r0, nr);
-        tile_cols(in, g, b, tc, c0, nc);
-        Cand *slot = in.cand + in.bond[b].cand_base + (int64_t)(tr * g.nct + tc) * spt;
-        if (quarters) {
-          // quarter qt of the tile: rows / columns [32 qr, 32 qr + 32)
-          const int h = g.te / 2, qr = qt >> 1, qc = qt & 1;
-          const int nrq = min(h, nr - h * qr), ncq = min(h, nc - h * qc);
-          if (nrq > 0 && ncq > 0)
-            screen_tile_stored(in, b, r[b], r0 + h * qr, nrq, c0 + h * qc, ncq, h, s_sr[b],
-                               s_sc[b], s_pend[b], slot + qt, sm.s);
-          else if (threadIdx.x == 0)
-            slot[qt] = Cand{0ull, LLONG_MAX, -2, -2};  // an empty quarter
-        } else {
-          screen_tile_stored(in, b, r[b], r0, nr, c0, nc, g.te, s_sr[b], s_sc[b], s_pend[b],
-                             slot, sm.s);
-        }
-        break;
-      }
-    } else {
-      // carried tiles: eight warp tiles, or one block tile
-      for (int b = 0; b < in.nb; ++b) {
-        const TileGeo &g = s_geo[b];
-        const int32_t tc0 = s_tc0[b], nc_b = s_tr0[b] * tc0;
-        const int32_t cnt = s_warp[b] ? (nc_b + CW - 1) / CW : nc_b;
-        if (j >= cnt) {
-          j -= cnt;
-          continue;
-        }
-        const int32_t k = s_warp[b] ? j * CW + (int32_t)(threadIdx.x >> 5) : j;
-        if (k < nc_b) {
-          const int32_t tr = k / tc0, tc = k - tr * tc0;
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0) screen_bookkeeping(in, r, s_geo, s_sr, s_sc, s_nf, s_nc);
+  const bool a_first = s_place < HA;
+  for (int part = 0; part < 2; ++part) {
+    if ((part == 0) == a_first) {
+      // queue A, the CTA together
+      int32_t nxt = 0;
+      if (threadIdx.x == 0) s_item = a_first ? s_place : HA + atomicAdd(ctr[0], 1);
+      for (;;) {
+        __syncthreads();
+        int32_t j = s_item;
+        __syncthreads();
+        if (j >= nA) break;
+        if (threadIdx.x == 0) nxt = HA + atomicAdd(ctr[0], 1);
+        // a fresh tile (or quarter q of it)
+        const int32_t qt = j % spt;
+        j /= spt;
+        for (int b = 0; b < in.nb; ++b) {
+          const TileGeo &g = s_geo[b];
+          const int32_t tr0 = s_tr0[b], tc0 = s_tc0[b];
+          const int32_t cnt = g.nrt * g.nct - tr0 * tc0;
+          if (j >= cnt) {
+            j -= cnt;
+            continue;
+          }
+          int32_t tr, tc;
+          if (j < tr0 * (g.nct - tc0)) {
+            // new columns of the stored rows
+            tr = j / (g.nct - tc0);
+            tc = tc0 + (j - tr * (g.nct - tc0));
+          } else {
+            // new rows, every column
+            const int32_t u = j - tr0 * (g.nct - tc0);
+            tr = tr0 + u / g.nct;
+            tc = u - (tr - tr0) * g.nct;
+          }
+          Cand *slot = in.cand + in.bond[b].cand_base + j * spt + qt;
           int64_t r0, c0;
           int nr, nc;
           tile_rows(in, g, b, tr, r0, nr);
           tile_cols(in, g, b, tc, c0, nc);
-          Cand *slot = in.cand + in.bond[b].cand_base + (int64_t)(tr * g.nct + tc) * spt;
-          if (!s_warp[b]) {
-            screen_tile_stored(in, b, r[b], r0, nr, c0, nc, g.te, s_sr[b], s_sc[b], s_pend[b],
-                               slot, sm.s);
-            if (threadIdx.x == 0)
-              for (int x = 1; x < spt; ++x) slot[x] = Cand{0ull, LLONG_MAX, -2, -2};
-          } else {
-            carried_warp(in, g.te, b, r0, nr, c0, nc, s_pend[b], slot, spt);
+          int te = g.te;
+          if (quarters) {
+            // quarter qt of the tile: rows / columns [32 qr, 32 qr + 32)
+            const int h = te / 2, qr = qt >> 1, qc = qt & 1;
+            r0 += h * qr;
+            c0 += h * qc;
+            nr = min(h, nr - h * qr);
+            nc = min(h, nc - h * qc);
+            te = h;
           }
+          if (nr > 0 && nc > 0)
+            screen_tile_stored(in, b, r[b], r0, nr, c0, nc, te, s_sr[b], s_sc[b], s_pend[b], slot,
+                               sm.s);
+          else if (threadIdx.x == 0)
+            *slot = Cand{0ull, LLONG_MAX, -2, -2};  // an empty quarter
+          break;
         }
-        break;
+        if (threadIdx.x == 0) s_item = nxt;
+      }
+    } else {
+      // queue B, each warp on its own
+      int64_t *lin = reinterpret_cast<int64_t *>(&sm.s.op) + warp * BM;
+      int32_t item = a_first ? 0 : (s_place - HA) * (NT / 32) + warp;
+      if (a_first) {
+        if (lane == 0) item = HB + atomicAdd(ctr[1], 1);
+        item = __shfl_sync(0xffffffffu, item, 0);
+      }
+      while (item < nB) {
+        int32_t nxt = lane == 0 ? HB + atomicAdd(ctr[1], 1) : 0;
+        int32_t j = item;
+        for (int b = 0; b < in.nb; ++b) {
+          const int32_t tc0 = s_tc0[b], nc_b = s_tr0[b] * tc0;
+          const int32_t cnt = (nc_b + run - 1) / run;
+          if (j >= cnt) {
+            j -= cnt;
+            continue;
+          }
+          carried_run(in, s_geo[b], b, j * run, min(nc_b, (j + 1) * run), tc0, r[b] - 1, s_pend[b],
+                      s_ptr[b], s_ptc[b], s_str[b], s_low[b], lin,
+                      in.cand + in.bond[b].cand_base + s_nf[b], s_fma, s_byte);
+          break;
+        }
+        item = __shfl_sync(0xffffffffu, nxt, 0);
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      if (nxt >= N[qq]) {
-        nxt = -1;
-        if (!switched) {
-          switched = true;
-          q0 = qq ^ 1;
-          const int32_t t = H[q0] + atomicAdd(ctr[q0], 1);
-          nxt = t < N[q0] ? t : -1;
-        }
-      } else {
-        q0 = qq;
-      }
-      s_q = q0;
-      s_item = nxt;
-    }
+  }
+  if (threadIdx.x == 0 && s_byte) {
+    atomicAdd((unsigned long long *)&in.ctrl->screen_fmas, s_fma);
+    atomicAdd((unsigned long long *)&in.ctrl->stored_bytes, s_byte);
   }
 }
 
@@ -1731,15 +2042,6 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
 //   x = SplitMix64(seed) output 2i, x' = output 2i+1, i = (t nb + b) nl + j;
 // their argmax (lowest linear index on ties) is refined by whole-column and
 // whole-row scans (the while loop of Alg. 1) in the refinement phases.
-
-// column-major linear index of superblock entry (a, c) of bond b
-__device__ __forceinline__ int64_t entry_lin(const InstDev &in, int b, int64_t a, int64_t c) {
-  const int64_t nb0 = in.n[b], nb1 = in.n[b + 1];
-  const int64_t p = a / nb0, i = a - p * nb0;
-  const int64_t q = c / nb1, j = c - q * nb1;
-  return left_set(in, b).lin[p] + i * in.stride[b] + j * in.stride[b + 1] +
-         right_set(in, b).lin[q];
-}
 
 // E(a,c) = A(a,c) - chain(T(a,:), R(:,c)) with K terms: the contract's residual
 __device__ __forceinline__ double residual_at(const InstDev &in, int b, int K, int64_t a,
@@ -1825,7 +2127,7 @@ __device__ void phase_screen(const RunArgs &ra, PhaseSmem &sm) {
     if (threadIdx.x < in.nb) s_pg[threadIdx.x] = planned_geo(in, cr, threadIdx.x);
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0)
-      screen_bookkeeping(in, r, s_pg, nullptr, nullptr, nullptr, 1);
+      screen_bookkeeping(in, r, s_pg, nullptr, nullptr, nullptr, nullptr);
     for (int b = 0; b < in.nb; ++b) {
       const TileGeo &g = s_pg[b];
       const int32_t nt = g.nrt * g.nct;
@@ -2022,9 +2324,32 @@ __device__ void finalize_bond(const InstDev &in, Ctrl &cr, int b, DecideSmem &sm
                   ld_cg(cr.maxr[b]));
 }
 
+// stored forms, once a bond's candidates are merged (one thread): the screen
+// has stored every entry of the superblock; its list of candidates, item
+// counters and pending step are cleared for the next
+__device__ __forceinline__ void close_screen(Ctrl &cr, int b, const DecideSmem &sm) {
+  cr.pv_rows[b] = ld_cg(cr.st_rows[b]);
+  cr.pv_cols[b] = ld_cg(cr.st_cols[b]);
+  cr.st_rows[b] = sm.q_prow;
+  cr.st_cols[b] = sm.q_pcol;
+  cr.e_pend[b] = 0;
+  cr.ntiles[b] = 0;
+  if (b == 0) cr.steal = cr.steal2 = 0;  // item counters of the next screen
+}
+// the step maxima, cleared for the update phase's next step (block-wide); the
+// extents are the run's caps (ldT / ldR bound the tile counts)
+__device__ __forceinline__ void clear_maxima(const InstDev &in, int b) {
+  const BondDev &B = in.bond[b];
+  const Ctrl &cr = *in.ctrl;
+  const int32_t nr = ld_cg(cr.plan_nrt[b]), nc = ld_cg(cr.plan_nct[b]);
+  for (int x = threadIdx.x; x < nr; x += NT) B.wmax[x] = 0u;
+  for (int x = threadIdx.x; x < nc; x += NT) B.emax[x] = 0u;
+}
+
 // FP64 decide item of bond b: the control words it needs in one round of
 // parallel loads, the merge of the tile candidates (the Allgather of Alg. 3),
 // then the stop test on the merged best as it stands
+template <bool STORED>
 __device__ void decide_bond_fp64(const InstDev &in, Ctrl &cr, int b, DecideSmem &sm) {
   const int tid = threadIdx.x;
   if (tid == 0) sm.q_nt = ld_cg(cr.ntiles[b]);
@@ -2032,18 +2357,13 @@ __device__ void decide_bond_fp64(const InstDev &in, Ctrl &cr, int b, DecideSmem 
   if (tid == 2) sm.q_tau = ld_cg(cr.tau);
   if (tid == 3) sm.q_xrms = ld_cg(cr.xrms);
   if (tid == 4) sm.q_maxr = ld_cg(cr.maxr[b]);
-  if (tid == 5 && in.stored) sm.q_prow = ld_cg(cr.plan_rows[b]);
-  if (tid == 6 && in.stored) sm.q_pcol = ld_cg(cr.plan_cols[b]);
+  if (tid == 5 && STORED) sm.q_prow = ld_cg(cr.plan_rows[b]);
+  if (tid == 6 && STORED) sm.q_pcol = ld_cg(cr.plan_cols[b]);
+  if (tid == 7) sm.q_nf = STORED ? ld_cg(cr.nfresh[b]) : 0;
   __syncthreads();
-  if (in.stored && tid == 0) {
-    // the screen just stored every entry of the superblock and applied the
-    // pending rank-one step
-    cr.st_rows[b] = sm.q_prow;
-    cr.st_cols[b] = sm.q_pcol;
-    cr.e_pend[b] = 0;
-    if (b == 0) cr.steal = cr.steal2 = 0;  // item counters of the next screen
-  }
-  const int64_t nt = sm.q_nt;
+  const int64_t nt = sm.q_nt + sm.q_nf;
+  if (STORED && tid == 0) close_screen(cr, b, sm);
+  if (STORED) clear_maxima(in, b);
   KeyBest best{0ull, LLONG_MAX, -1, -1};
   const Cand *cand = in.cand + in.bond[b].cand_base;
   int bad = 0;
@@ -2059,16 +2379,16 @@ __device__ void decide_bond_fp64(const InstDev &in, Ctrl &cr, int b, DecideSmem 
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       bad += o[u].row == -1;  // -2 marks a slot left empty on purpose
-      kb_take(best, o[u]);
+      STORED ? kb_take_any(best, o[u]) : kb_take(best, o[u]);
     }
   }
   for (; t < nt; t += NT) {
     KeyBest o{cand[t].key, cand[t].lin, cand[t].row, cand[t].col};
     bad += o.row == -1;
-    kb_take(best, o);
+    STORED ? kb_take_any(best, o) : kb_take(best, o);
   }
   if (bad) atomicAdd((unsigned long long *)&cr.unscreened, (unsigned long long)bad);
-  best = block_best(best, sm.rk, sm.rl, sm.rr, sm.rc);
+  best = block_best<STORED>(best, sm.rk, sm.rl, sm.rr, sm.rc);
   if (tid == 0) {
     cr.best_key[b] = best.key;
     cr.best_lin[b] = best.lin;
@@ -2168,10 +2488,10 @@ __device__ void topk_of_slots(const Cand *src, int64_t t0, int64_t t1, int k, De
     bad += c.row == -1;
     if (c.row < 0) continue;
     // most slots lose to the list's last entry: one comparison
-    if (k == RS_K && loc[RS_K - 1].row >= 0 &&
-        !key_better(c.key, c.lin, loc[RS_K - 1].key, loc[RS_K - 1].lin))
-      continue;
     KeyBest o{c.key, c.lin, c.row, c.col};
+    if (k == RS_K && loc[RS_K - 1].row >= 0 &&
+        !key_better(o.key, o.lin, loc[RS_K - 1].key, loc[RS_K - 1].lin))
+      continue;
     // insertion into the sorted list loc[0..k-1]
 #pragma unroll
     for (int j = 0; j < RS_K; ++j) {
@@ -2235,8 +2555,9 @@ __device__ __noinline__ void decide_bond_rescore(const InstDev &in, Ctrl &cr, in
   if (tid == 4) sm.q_maxr = ld_cg(cr.maxr[b]);
   if (tid == 5) sm.q_prow = ld_cg(cr.plan_rows[b]);
   if (tid == 6) sm.q_pcol = ld_cg(cr.plan_cols[b]);
+  if (tid == 7) sm.q_nf = ld_cg(cr.nfresh[b]);
   __syncthreads();
-  const int64_t nt = sm.q_nt, L = (nt + P - 1) / P;
+  const int64_t nt = sm.q_nt + sm.q_nf, L = (nt + P - 1) / P;
   const int64_t t0 = min(nt, (int64_t)part * L), t1 = min(nt, t0 + L);
   const Cand *cand = in.cand + in.bond[b].cand_base;
   Cand *pb = in.refine_cand + in.bond[b].cand_base;  // the parts' results, [P][k]
@@ -2264,14 +2585,7 @@ __device__ __noinline__ void decide_bond_rescore(const InstDev &in, Ctrl &cr, in
     }
     topk_of_slots(pb, 0, (int64_t)P * k, k, sm, bad);
   }
-  if (tid == 0) {
-    // the screen just stored every entry of the superblock and applied the
-    // pending rank-one step
-    cr.st_rows[b] = sm.q_prow;
-    cr.st_cols[b] = sm.q_pcol;
-    cr.e_pend[b] = 0;
-    if (b == 0) cr.steal = cr.steal2 = 0;  // item counters of the next screen
-  }
+  if (tid == 0) close_screen(cr, b, sm);
   if (bad) atomicAdd((unsigned long long *)&cr.unscreened, (unsigned long long)bad);
   // FP64 re-score of the k candidates, a lane each of warp 0 (the chains run
   // side by side instead of queueing warps on the SM's FP64 units)
@@ -2538,7 +2852,10 @@ __device__ void phase_decide(const RunArgs &ra, PhaseSmem &sm) {
     } else if (in.nl > 0) {
       decide_bond_sampled(in, cr, b, sm.d);
     } else if (in.prec == P_FP64) {
-      decide_bond_fp64(in, cr, b, sm.d);
+      if (in.stored)
+        decide_bond_fp64<true>(in, cr, b, sm.d);
+      else
+        decide_bond_fp64<false>(in, cr, b, sm.d);
     } else if (in.stored) {
       decide_bond_rescore(in, cr, b, part, P, sm.d);
     } else {
@@ -3480,6 +3797,20 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
       for (int b = 0; b < in.nb; ++b)
         if (ad[b] && s_place == (cb0 + G - 1 - b % G) % G)
           border_inverse(in, b, ro[b], sm.d);
+      // where the stored entries' pending steps are found (the carried tiles of
+      // the last screen)
+      __shared__ LazyGeo s_lazy[TTC_MAXB];
+      const bool lazy = in.stored && in.prec == P_FP64;
+      if (lazy) __syncthreads();
+      if (lazy && threadIdx.x < in.nb) {
+        const int b = threadIdx.x;
+        LazyGeo q;
+        q.g = planned_geo(in, cr, b);
+        stateful_tiles(in, cr, q.g, b, q.tr, q.tc);
+        q.stride = state_stride(in, cr, q.g, b);
+        s_lazy[b] = q;
+      }
+      if (lazy) __syncthreads();
       auto item0 = [&](int64_t bs) -> int64_t {
         return idle ? LLONG_MAX : first_item(bs, gti, NTI);
       };
@@ -3497,16 +3828,36 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
           }
         }
         if (ad[b] && in.stored) {
-          // the pending rank-one step of the stored residual (from the
-          // sweep-start superblock, which E still holds)
+          // the rank-one step of the new pivot, from the residual of the
+          // sweep-start superblock (its entries through their pending steps),
+          // and its largest values per tile
+          const int z = ro[b];
           const int64_t rows = rows_of(in, ro, b), cols = cols_of(in, ro, b);
-          const int64_t ld = B.ldR, as = B.prow[ro[b]], cs = B.pcol[ro[b]];
-          for (int64_t x = item0(base); x < base + rows; x += NTI)
-            sv_put(in, B.ew, x - base,
-                   -(sv_get(in, B.E, (x - base) * ld + cs) / sv_get(in, B.E, as * ld + cs)));
+          const int64_t as = B.prow[z], cs = B.pcol[z];
+          const LazyGeo &lg = s_lazy[b];
+          double *ew = B.ew + (int64_t)z * B.ldT, *erow = B.erow + (int64_t)z * B.ldR;
+          if (item0(base) < base + rows) {
+            const double ep = stored_entry(in, lg, b, as, cs, z - 1);
+            for (int64_t x = item0(base); x < base + rows; x += NTI) {
+              const int64_t a = x - base;
+              const double w = -(stored_entry(in, lg, b, a, cs, z - 1) / ep);
+              sv_put(in, ew, a, w);
+              if (lazy)
+                atomicMax(&B.wmax[row_tile_of(in, lg.g, b, (int32_t)a)],
+                          __float_as_uint(__double2float_ru(fabs(w))));
+            }
+          }
           base += rows;
-          for (int64_t x = item0(base); x < base + cols; x += NTI)
-            B.erow[x - base] = B.E[as * ld + (x - base)];  // the same 8 bytes in either form
+          for (int64_t x = item0(base); x < base + cols; x += NTI) {
+            const int64_t c = x - base;
+            if (lazy) {
+              const double e = stored_entry_t<0>(B, as, c, lazy_z(in, lg, b, as, c, z - 1), z - 1);
+              erow[c] = e;
+              atomicMax(&B.emax[col_tile_of(in, lg.g, b, (int32_t)c)], __float_as_uint(SV<0>::up(e)));
+            } else {
+              erow[c] = B.E[as * B.ldR + c];  // a float-float pair, the same 8 bytes
+            }
+          }
           base += cols;
         }
         if (ad[b]) {
@@ -3694,6 +4045,12 @@ __device__ void phase_init3(const RunArgs &ra, PhaseSmem &sm) {
     const InstDev &in = inst(ra, ii);
     const Ctrl &cr = *in.ctrl;
     if (ld_cg(cr.state) == ST_DONE) continue;
+    if (in.stored)
+      for (int b = 0; b < in.nb; ++b) {
+        const BondDev &B = in.bond[b];
+        for (int64_t x = gt; x < B.ldT; x += NTOT) B.wmax[x] = 0u;
+        for (int64_t x = gt; x < B.ldR; x += NTOT) B.emax[x] = 0u;
+      }
     for (int b = 0; b < in.nb; ++b) {
       const BondDev &B = in.bond[b];
       const int64_t rows = in.n[b], cols = in.n[b + 1];
@@ -3870,6 +4227,10 @@ __global__ void __launch_bounds__(NT, 2) k_persistent(RunArgs ra) {
       if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&ra.bar->overrun, 1);
       break;
     }
+    if (ra.stored) {
+      phase_bound(ra);
+      if (!grid_barrier(ra, 14)) return;
+    }
     phase_screen(ra, sm);
     if (!grid_barrier(ra, 3)) return;
     clk.lap(ra, T_SCREEN);
@@ -3921,6 +4282,10 @@ __global__ void __launch_bounds__(NT, 2) k_init2(RunArgs ra) {
 __global__ void __launch_bounds__(NT, 2) k_init3(RunArgs ra) {
   cache_inst0(ra);
   phase_init3(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem));
+}
+__global__ void __launch_bounds__(NT, 2) k_bound(RunArgs ra) {
+  cache_inst0(ra);
+  phase_bound(ra);
 }
 __global__ void __launch_bounds__(NT, 2) k_screen(RunArgs ra) {
   cache_inst0(ra);
@@ -4103,6 +4468,7 @@ cudaError_t launch_phase(int phase, const RunArgs &ra, int grid, cudaStream_t s)
     case PH_INIT1: f = (const void *)k_init1; break;
     case PH_INIT2: f = (const void *)k_init2; break;
     case PH_INIT3: f = (const void *)k_init3; break;
+    case PH_BOUND: f = (const void *)k_bound; break;
     case PH_SCREEN: f = (const void *)k_screen; break;
     case PH_DECIDE: f = (const void *)k_decide; break;
     case PH_UPDATE: f = (const void *)k_update; break;
@@ -4230,7 +4596,7 @@ cudaError_t launch_rebuild_cores(const InstDev *d_inst, int nb, double *scratch,
 // rn x cn (rows, columns); its new entries are, in this order,
 //   rows ro..rn-1 x columns 0..cn-1, then rows 0..ro-1 x columns co..cn-1.
 // k_user_count sums them per bond (first: every entry of the rank-one
-// superblocks); k_user_gather writes their multi-indices, k_user_scatter
+// superblocks), and says whether the run is over or an error check is due; k_user_gather writes their multi-indices, k_user_scatter
 // puts the callback's values into the cache at (a, c).
 
 __device__ void user_extent(const InstDev &in, const Ctrl &cr, int b, int first, int64_t &ro,
@@ -4256,6 +4622,10 @@ __global__ void k_user_count(const InstDev *inp, int first, int64_t *counts) {
     if (cr.state != ST_DONE) tot += rn * cn - ro * co;
   }
   counts[in.nb] = tot;
+  int nadd = 0;
+  for (int b = 0; b < in.nb; ++b) nadd += cr.add[b];
+  counts[in.nb + 1] = cr.state == ST_DONE;
+  counts[in.nb + 2] = cr.state != ST_DONE && cr.screened && nadd == 0;
 }
 
 // entry x of the new entries of bond b -> superblock (a, c)
