@@ -334,11 +334,8 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
     CU(launch_phase(PH_SCREEN, ra, h0->grid, s));
     CU(launch_phase(PH_DECIDE, ra, h0->grid, s));
     if (ra.sampled) {
-      // refinement rounds: a phase pair per step (no-ops once every bond is done)
-      for (int k = 0; k < 2 * ra.max_rook; ++k) {
-        CU(launch_phase(PH_ROOK_SCAN, ra, h0->grid, s));
-        CU(launch_phase(PH_ROOK_DECIDE, ra, h0->grid, s));
-      }
+      // refinement rounds: a launch per step (no-ops once every bond is done)
+      for (int k = 0; k < 2 * ra.max_rook; ++k) CU(launch_phase(PH_ROOK_STEP, ra, h0->grid, s));
       CU(launch_phase(PH_FINALIZE, ra, h0->grid, s));
     }
     if (ra.mixed) {
@@ -612,6 +609,12 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
       B.J.idx = cv.take<int32_t>(cap * (d - 1 - b));
       B.J.lin = cv.take<int64_t>(cap);
       B.J.sum = cv.take<int32_t>(cap);
+      B.Tr = B.Rr = nullptr;
+      B.ldr = (cap + 15) / 16 * 16;
+      if (I.nl > 0) {
+        B.Tr = cv.take<double>(B.ldr * B.ldT);
+        B.Rr = cv.take<double>(B.ldr * B.ldR);
+      }
       B.Thi = B.Tlo = B.Rhi = B.Rlo = nullptr;
       if (I.prec != P_FP64) {
         B.Thi = cv.take<float>(cap * B.ldT);

@@ -49,6 +49,8 @@ struct BondDev {
   int64_t ldT, ldR;      // row / column capacity of the superblock
   double *T, *R, *U, *hpiv, *hc, *delta;
   float *Thi, *Tlo, *Rhi, *Rlo;
+  double *Tr, *Rr;       // sampled screen: T and R by superblock row / column,
+  int64_t ldr;           // [ldT][ldr] and [ldR][ldr] (null otherwise)
   int32_t *prow, *pcol;  // pivot superblock coordinates, insertion order
   // stored-residual form (null otherwise): the residual, and the rank-one steps
   // of the pivots z = 1, 2, ...: step z is row z of ew [cap][ldT] (the column
@@ -117,7 +119,8 @@ struct Ctrl {
   int64_t screen_t;          // sampled screen: screens run (the sample counter)
   int32_t dcount[TTC_MAXD];  // stored forms: parts of bond b's decide that have
                              // merged their share of the tile slots (the last
-                             // one finishes the bond and clears it)
+                             // one finishes the bond and clears it); sampled
+                             // screen: CTAs done with the refinement step
   int32_t dkind;             // work of the coming decide phases, fixed by the
                              // screen phase: DK_BONDS, DK_VERIFY or DK_NONE
   int32_t pad_dkind;

@@ -2061,24 +2061,96 @@ __device__ __forceinline__ void take_key(KeyBest &best, double e, int64_t lin, i
   }
 }
 
-// the CTA's best of its share of the samples of every bond, into the bond's
-// slot blockIdx.x (thread x of the grid takes samples x, x + G NT, ...)
+// CTAs that work on bond b in a sampled screen or a refinement step: every nb-th
+// one (each CTA has one bond, so one block reduction instead of nb in turn), or
+// all of them where a column or row is longer than 16 passes of such a share
+// (wide) or the grid has fewer CTAs than there are bonds; a CTA's candidate goes to slot `rank` of the bond.
+__device__ __forceinline__ int share_size(const InstDev &in, int b, bool wide) {
+  return wide || (int)gridDim.x < in.nb ? (int)gridDim.x : ((int)gridDim.x - b + in.nb - 1) / in.nb;
+}
+__device__ __forceinline__ int share_rank(const InstDev &in, int b, bool wide) {
+  if (wide || (int)gridDim.x < in.nb) return blockIdx.x;
+  return (int)blockIdx.x % in.nb == b ? (int)blockIdx.x / in.nb : -1;
+}
+__device__ __forceinline__ bool share_wide(const InstDev &in, const int32_t *r) {
+  int64_t longest = 0;
+  for (int b = 0; b < in.nb; ++b) longest = max(longest, max(rows_of(in, r, b), cols_of(in, r, b)));
+  return longest > (int64_t)16 * NT * max(1, (int)gridDim.x / in.nb);
+}
+
+// chain(row ra of A, row rb of Bm) over K terms for every lane of a warp, the rows
+// contiguous (lda, ldb entries apart): sixteen entries at a time, the warp loads
+// its 32 lanes' rows together, two rows per instruction, into shared memory
+// (32 x 17 doubles), and each lane runs the contract's chain on its own two (a
+// thread reading its own rows touches 32 lines per load).
+__device__ __forceinline__ double warp_chain_rows(const double *A, int64_t ra, int64_t lda,
+                                                  const double *Bm, int64_t rb, int64_t ldb, int K,
+                                                  double *buf) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, half = lane >> 4, el = lane & 15;
+  double acc = 0.0;
+  for (int c = 0; c < K; c += 16) {
+    const bool has = c + el < K;
+    double xv[16], yv[16];
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const double *tab = (side == 0 ? A : Bm) + c + el;
+      const int64_t o = side == 0 ? ra * lda : rb * ldb;
+      double v[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int64_t os = __shfl_sync(FULL, o, 2 * q + half);
+        v[q] = has ? tab[os] : 0.0;
+      }
+      __syncwarp();  // the previous rows are read
+#pragma unroll
+      for (int q = 0; q < 16; ++q) buf[(2 * q + half) * 17 + el] = v[q];
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < 16; ++t) {
+        if (side == 0)
+          xv[t] = buf[lane * 17 + t];
+        else
+          yv[t] = buf[lane * 17 + t];
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 16; ++t)
+      if (c + t < K) acc = __fma_rn(xv[t], yv[t], acc);
+  }
+  return acc;
+}
+
+// The CTA's best of its share of the samples of every bond, into the bond's
+// slot (thread x of the bond's share takes samples x, x + share NT, ...).  A
+// sample's row of T and column of R come from copies that keep them
+// contiguous: from the t-major factors every entry is a 32-byte sector of its
+// own (2 GB of L2 traffic a screen of 2^18 samples per bond at ranks 24).
 __device__ void screen_sampled_instance(const InstDev &in, const int32_t *r, int64_t t,
                                         PhaseSmem &sm) {
-  const int64_t NTOT = (int64_t)gridDim.x * NT;
-  const int64_t gt = (int64_t)blockIdx.x * NT + threadIdx.x;
+  double *buf = sm.sw.rows[threadIdx.x >> 5];
   for (int b = 0; b < in.nb; ++b) {
+    const int rank = share_rank(in, b, false);
+    if (rank < 0) continue;
+    const int64_t NTOT = (int64_t)share_size(in, b, false) * NT, gt = (int64_t)rank * NT + threadIdx.x;
+    __syncthreads();  // (the rows share memory with the reduction below)
+    const BondDev &B = in.bond[b];
     const int64_t rows = rows_of(in, r, b), cols = cols_of(in, r, b);
     KeyBest best{0ull, LLONG_MAX, -1, -1};
-    for (int64_t j = gt; j < in.nl; j += NTOT) {
-      const uint64_t i = (uint64_t)((t * in.nb + b) * in.nl + j);
+    for (int64_t j = gt;; j += NTOT) {
+      const bool valid = j < in.nl;
+      if (!__any_sync(0xffffffffu, valid)) break;
+      const uint64_t i = (uint64_t)((t * in.nb + b) * in.nl + (valid ? j : 0));
       const int64_t a = (int64_t)__umul64hi(splitmix64_at(in.lseed, 2 * i), (uint64_t)rows);
       const int64_t c = (int64_t)__umul64hi(splitmix64_at(in.lseed, 2 * i + 1), (uint64_t)cols);
-      take_key(best, residual_at(in, b, r[b], a, c), entry_lin(in, b, a, c), a, c);
+      const double acc = warp_chain_rows(B.Tr, a, B.ldr, B.Rr, c, B.ldr, r[b], buf);
+      if (!valid) continue;
+      const double e = __dsub_rn(sb_entry(in, b, a, c), acc);
+      if (best.row < 0 || abs_key(e) >= best.key) take_key(best, e, entry_lin(in, b, a, c), a, c);
     }
     best = block_best(best, sm.s.sk, sm.s.sl, sm.s.sr, sm.s.sc);
     if (threadIdx.x == 0) {
-      Cand *slot = in.cand + in.bond[b].cand_base + blockIdx.x;
+      Cand *slot = in.cand + in.bond[b].cand_base + rank;
       *slot = best.row >= 0 ? Cand{best.key, best.lin, best.row, best.col}
                             : Cand{0ull, LLONG_MAX, -2, -2};
     }
@@ -2793,7 +2865,7 @@ __device__ void verify_instance(const InstDev &in, Ctrl &cr, DecideSmem &sm) {
 // during the phase (state, screened, pending): a CTA that read them late
 // would number the items differently, and one bond would be decided twice.
 // item kinds of for_decide_items
-enum ItemMode { IM_DECIDE = 0, IM_PENDING = 1, IM_ROOK = 2, IM_FINALIZE = 3 };
+enum ItemMode { IM_DECIDE = 0, IM_PENDING = 1, IM_FINALIZE = 2 };
 
 // CTAs that share one bond's decide: the mixed stored form of a single
 // instance merges its tile slots' k best in DPARTS parts (the last part to
@@ -2831,7 +2903,6 @@ __device__ void for_decide_items(const RunArgs &ra, int mode, F &&f) {
         } else {
           take = kind == DK_BONDS && ld_cg(cr.state) != ST_DONE;
           if (mode == IM_PENDING) take = take && ld_cg(cr.pending[slot]);
-          if (mode == IM_ROOK) take = take && in.nl > 0 && ld_cg(cr.rook_stage[slot]) != 0;
           if (mode == IM_FINALIZE) take = take && in.nl > 0;
         }
         s_take = take ? 1 : 0;
@@ -2894,14 +2965,15 @@ __device__ void phase_decide2(const RunArgs &ra, PhaseSmem &sm) {
   });
 }
 
-// merge of the G candidate slots of bond b (block-wide; the best is valid
+// merge of the first nt candidate slots of bond b (block-wide; the best is valid
 // in every thread)
 __device__ KeyBest merge_slots(const InstDev &in, Ctrl &cr, int b, int64_t nt, DecideSmem &sm) {
   const Cand *cand = in.cand + in.bond[b].cand_base;
   KeyBest best{0ull, LLONG_MAX, -1, -1};
   int bad = 0;
   for (int64_t t = threadIdx.x; t < nt; t += NT) {
-    KeyBest o{cand[t].key, cand[t].lin, cand[t].row, cand[t].col};
+    const Cand c = ld_cand(cand + t);
+    const KeyBest o{c.key, c.lin, c.row, c.col};
     bad += o.row == -1;
     kb_take(best, o);
   }
@@ -2921,7 +2993,7 @@ __device__ KeyBest merge_slots(const InstDev &in, Ctrl &cr, int b, int64_t nt, D
 // sampled screen, decide item of bond b: the argmax over the samples becomes
 // the pivot candidate, and its refinement starts (column step first)
 __device__ void decide_bond_sampled(const InstDev &in, Ctrl &cr, int b, DecideSmem &sm) {
-  const KeyBest best = merge_slots(in, cr, b, gridDim.x, sm);
+  const KeyBest best = merge_slots(in, cr, b, share_size(in, b, false), sm);
   if (threadIdx.x == 0) {
     cr.best_key[b] = best.key;
     cr.best_lin[b] = best.lin;
@@ -2955,95 +3027,93 @@ __device__ bool any_rook(const RunArgs &ra) {
   return hit != 0;
 }
 
-// refinement scan: the pivot's column (step 1) or row (step 2) of every bond
-// in a refinement step, spread over the grid; each CTA's best of its share
-// goes to its slot
-__device__ void phase_rook_scan(const RunArgs &ra, PhaseSmem &sm) {
+// refinement step: the pivot's column (step 1) or row (step 2) of every bond in
+// a refinement step, each CTA's best of its share to its slot; the last CTA of a
+// bond's share to arrive merges them (no grid barrier and second phase in
+// between) and the pivot moves to a strictly larger |E|.  A round is step 1
+// then step 2, and the refinement ends after a round that moved nothing or
+// after max_rook rounds.  A CTA reads only the words of bonds it has a share
+// of, before it arrives.  A step is latency (a few thousand residuals of up to
+// 40 terms on the whole grid): as a scan of all bonds by every CTA, a barrier, a
+// merge of all slots and a second barrier it took about 20 us, so this form and
+// the row copies took the screen of Hilbert d=6, n=256, rank 40, 64 k samples, 8
+// rounds from 5.1-5.4 to 3.5 ms over 24 sweeps (4.8 with the copies alone).
+__device__ void phase_rook_step(const RunArgs &ra, PhaseSmem &sm) {
   __shared__ CtrlSnap snap;
-  __shared__ int32_t s_stage[TTC_MAXB], s_row[TTC_MAXB], s_col[TTC_MAXB];
-  const int64_t NTOT = (int64_t)gridDim.x * NT;
-  const int64_t gt = (int64_t)blockIdx.x * NT + threadIdx.x;
+  __shared__ int32_t s_stage, s_row, s_col, s_last;
   for (int ii = 0; ii < ra.count; ++ii) {
     const InstDev &in = inst(ra, ii);
     if (in.nl == 0) continue;
-    const Ctrl &cr = *in.ctrl;
+    Ctrl &cr = *in.ctrl;
     snap_ctrl(cr, in.nb, snap);
     if (snap.state == ST_DONE || ld_cg(cr.dkind) != DK_BONDS) continue;
-    if (threadIdx.x < in.nb) {
-      s_stage[threadIdx.x] = ld_cg(cr.rook_stage[threadIdx.x]);
-      s_row[threadIdx.x] = ld_cg(cr.best_row[threadIdx.x]);
-      s_col[threadIdx.x] = ld_cg(cr.best_col[threadIdx.x]);
-    }
-    __syncthreads();
     const int32_t *r = snap.r;  // the sweep-start ranks (no pivot added yet)
+    const bool wide = share_wide(in, r);
     for (int b = 0; b < in.nb; ++b) {
-      const int st = s_stage[b];
-      if (!st) continue;
+      const int rank = share_rank(in, b, wide);
+      if (rank < 0) continue;
+      if (threadIdx.x == 0) s_stage = ld_cg(cr.rook_stage[b]);
+      if (threadIdx.x == 1) s_row = ld_cg(cr.best_row[b]);
+      if (threadIdx.x == 2) s_col = ld_cg(cr.best_col[b]);
+      __syncthreads();
+      const int st = s_stage;
+      const int size = share_size(in, b, wide);
       const int64_t rows = rows_of(in, r, b), cols = cols_of(in, r, b);
-      KeyBest best{0ull, LLONG_MAX, -1, -1};
-      if (st == 1) {
-        const int64_t c = s_col[b];
-        for (int64_t a = gt; a < rows; a += NTOT)
+      const int64_t a0 = s_row, c0 = s_col, len = st == 1 ? rows : cols;
+      if (st) {
+        KeyBest best{0ull, LLONG_MAX, -1, -1};
+        for (int64_t x = (int64_t)rank * NT + threadIdx.x; x < len; x += (int64_t)size * NT) {
+          const int64_t a = st == 1 ? x : a0, c = st == 1 ? c0 : x;
           take_key(best, residual_at(in, b, r[b], a, c), entry_lin(in, b, a, c), a, c);
-      } else {
-        const int64_t a = s_row[b];
-        for (int64_t c = gt; c < cols; c += NTOT)
-          take_key(best, residual_at(in, b, r[b], a, c), entry_lin(in, b, a, c), a, c);
+        }
+        best = block_best(best, sm.s.sk, sm.s.sl, sm.s.sr, sm.s.sc);
+        if (threadIdx.x == 0) {
+          in.cand[in.bond[b].cand_base + rank] = best.row >= 0
+                                                     ? Cand{best.key, best.lin, best.row, best.col}
+                                                     : Cand{0ull, LLONG_MAX, -2, -2};
+          __threadfence();  // the slot before the arrival
+          s_last = atomicAdd(&cr.dcount[b], 1) == size - 1;
+          if (s_last) {
+            cr.dcount[b] = 0;
+            __threadfence();  // the other slots after theirs
+          }
+        }
+        __syncthreads();
+        if (s_last) {
+          const KeyBest line = merge_slots(in, cr, b, size, sm.d);
+          if (threadIdx.x == 0) {
+            const uint64_t cur = ld_cg(cr.best_key[b]);
+            int moved = ld_cg(cr.rook_moved[b]);
+            // several CTAs decide bonds of one instance at once: atomic counts
+            atomicAdd((unsigned long long *)&cr.entries, (unsigned long long)len);
+            atomicAdd((unsigned long long *)&cr.entries_fresh, (unsigned long long)len);
+            atomicAdd((unsigned long long *)&cr.screen_fmas, (unsigned long long)(len * r[b]));
+            if (line.row >= 0 && line.key > cur) {
+              cr.best_key[b] = line.key;
+              cr.best_lin[b] = line.lin;
+              if (st == 1)
+                cr.best_row[b] = line.row;
+              else
+                cr.best_col[b] = line.col;
+              moved = 1;
+            }
+            if (line.key > KEY_INF) cr.best_key[b] = line.key;  // a non-finite residual ends the bond
+            if (st == 1) {
+              cr.rook_stage[b] = 2;
+              cr.rook_moved[b] = moved;
+            } else {
+              const int round = ld_cg(cr.rook_round[b]) + 1;
+              cr.rook_round[b] = round;
+              const bool again = moved && round < in.max_rook && ld_cg(cr.best_key[b]) <= KEY_INF;
+              cr.rook_stage[b] = again ? 1 : 0;
+              cr.rook_moved[b] = 0;
+            }
+          }
+        }
       }
-      best = block_best(best, sm.s.sk, sm.s.sl, sm.s.sr, sm.s.sc);
-      if (threadIdx.x == 0) {
-        Cand *slot = in.cand + in.bond[b].cand_base + blockIdx.x;
-        *slot = best.row >= 0 ? Cand{best.key, best.lin, best.row, best.col}
-                              : Cand{0ull, LLONG_MAX, -2, -2};
-      }
+      __syncthreads();
     }
   }
-}
-
-// refinement decide: the pivot moves to a strictly larger |E| of its column
-// (step 1) or row (step 2); a round is step 1 then step 2, and the
-// refinement ends after a round that moved nothing or after max_rook rounds
-__device__ void phase_rook_decide(const RunArgs &ra, PhaseSmem &sm) {
-  for_decide_items(ra, IM_ROOK, [&](int ii, int b, int, int) {
-    const InstDev &in = inst(ra, ii);
-    Ctrl &cr = *in.ctrl;
-    const KeyBest line = merge_slots(in, cr, b, gridDim.x, sm.d);
-    if (threadIdx.x == 0) {
-      const int st = ld_cg(cr.rook_stage[b]);
-      const uint64_t cur = ld_cg(cr.best_key[b]);
-      int moved = ld_cg(cr.rook_moved[b]);
-      // ranks written by other CTAs' items: read through L2, not this SM's L1
-      const int32_t r_old = ld_cg(cr.r[b]);
-      const int64_t rows = (b == 0 ? 1 : ld_cg(cr.r[b - 1])) * in.n[b];
-      const int64_t cols = in.n[b + 1] * (b == in.nb - 1 ? 1 : ld_cg(cr.r[b + 1]));
-      // several CTAs decide bonds of one instance at once: atomic counts
-      const unsigned long long cnt = (unsigned long long)(st == 1 ? rows : cols);
-      atomicAdd((unsigned long long *)&cr.entries, cnt);
-      atomicAdd((unsigned long long *)&cr.entries_fresh, cnt);
-      atomicAdd((unsigned long long *)&cr.screen_fmas, cnt * (unsigned long long)r_old);
-      if (line.row >= 0 && line.key > cur) {
-        cr.best_key[b] = line.key;
-        cr.best_lin[b] = line.lin;
-        if (st == 1)
-          cr.best_row[b] = line.row;
-        else
-          cr.best_col[b] = line.col;
-        moved = 1;
-      }
-      if (line.key > KEY_INF) cr.best_key[b] = line.key;  // a non-finite residual ends the bond
-      if (st == 1) {
-        cr.rook_stage[b] = 2;
-        cr.rook_moved[b] = moved;
-      } else {
-        const int round = ld_cg(cr.rook_round[b]) + 1;
-        cr.rook_round[b] = round;
-        const bool again = moved && round < in.max_rook && ld_cg(cr.best_key[b]) <= KEY_INF;
-        cr.rook_stage[b] = again ? 1 : 0;
-        cr.rook_moved[b] = 0;
-      }
-    }
-    __syncthreads();
-  });
 }
 
 // sampled screen: the stop test and the pivot append of every bond, on the
@@ -3062,8 +3132,12 @@ __device__ void phase_finalize(const RunArgs &ra, PhaseSmem &sm) {
 //   B: new row z of R on the sweep-start columns              cols_old items
 //   D: new columns of R for the new suffix                    r_new * n_{b+1}
 // stores into T / R keep the FP32 (hi, lo) shadows of the mixed forms
-__device__ __forceinline__ void putT(const InstDev &in, const BondDev &B, int64_t o, double v) {
+// (and the copies by row / column of the sampled screen)
+__device__ __forceinline__ void putT(const InstDev &in, const BondDev &B, int64_t t, int64_t a,
+                                     double v) {
+  const int64_t o = t * B.ldT + a;
   B.T[o] = v;
+  if (B.Tr) B.Tr[a * B.ldr + t] = v;
   if (in.prec != P_FP64) {
     float hi, lo;
     split2(v, hi, lo);
@@ -3071,8 +3145,11 @@ __device__ __forceinline__ void putT(const InstDev &in, const BondDev &B, int64_
     B.Tlo[o] = lo;
   }
 }
-__device__ __forceinline__ void putR(const InstDev &in, const BondDev &B, int64_t o, double v) {
+__device__ __forceinline__ void putR(const InstDev &in, const BondDev &B, int64_t t, int64_t c,
+                                     double v) {
+  const int64_t o = t * B.ldR + c;
   B.R[o] = v;
+  if (B.Rr) B.Rr[c * B.ldr + t] = v;
   if (in.prec != P_FP64) {
     float hi, lo;
     split2(v, hi, lo);
@@ -3187,7 +3264,7 @@ __device__ __noinline__ void replay_row_warp(const InstDev &in, int b, int64_t a
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const int t = 32 * k + lane;
-    if (t < nz) putT(in, B, (int64_t)t * B.ldT + a, tr[k]);
+    if (t < nz) putT(in, B, t, a, tr[k]);
   }
 }
 
@@ -3278,7 +3355,7 @@ __device__ __noinline__ void replay_group(const InstDev &in, int b, int64_t a0, 
   // neighbouring rows are neighbours in T: lanes take rows first
   for (int x = lane; x < nz * RPW; x += 32) {
     const int rr = x % RPW, t = x / RPW;
-    if (rr < nrows) putT(in, B, (int64_t)t * B.ldT + a0 + rr, buf[rr * LD + t]);
+    if (rr < nrows) putT(in, B, t, a0 + rr, buf[rr * LD + t]);
   }
   __syncwarp();
 }
@@ -3310,8 +3387,12 @@ __device__ void update_row(const InstDev &in, int b, int64_t a, int z) {
   pivot_col_entries(in, b, a, z, z + 1, &ent);
   const double s = __dsub_rn(chain(T, ld, hc, 1, z), ent);
   const double w = __dmul_rn(B.delta[z], s);
-  for (int t = 0; t < z; ++t) putT(in, B, a + t * ld, __fma_rn(w, hp[t], T[t * ld]));
-  putT(in, B, a + (int64_t)z * ld, -w);
+  if (in.prec == P_FP64 && in.nl == 0) {
+    for (int t = 0; t < z; ++t) T[t * ld] = __fma_rn(w, hp[t], T[t * ld]);
+  } else {
+    for (int t = 0; t < z; ++t) putT(in, B, t, a, __fma_rn(w, hp[t], T[t * ld]));
+  }
+  putT(in, B, z, a, -w);
 }
 
 // first item >= base that thread gt of NTOT takes when items are dealt
@@ -3656,16 +3737,13 @@ __device__ double sample_residual(const InstDev &in, const int32_t *r, int pL, i
 
 // The error's samples when the prefix and suffix tables meet (pL + pR = d,
 // rows of len): lane l of a warp takes the l-th of 32 consecutive samples, as
-// in the thread dealing of the plain loop.  Sixteen entries at a time, the
-// warp loads the 32 samples' rows together, two rows per instruction, into
-// shared memory, and each lane runs the contract's chain on its own two rows
-// (a thread reading its own rows touches 32 lines per load).  The operations
-// and their order per thread are those of sample_residual.
+// in the thread dealing of the plain loop, and the warp loads their rows
+// together.  The operations and their order per thread are those of
+// sample_residual.
 __device__ __noinline__ double samples_joined(const InstDev &in, int pL, int pR, int len,
                                               int64_t base, int64_t ns, int64_t gs, int64_t NTOT,
                                               SampleSmem &sw) {
   constexpr unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31, half = lane >> 4, el = lane & 15;
   double *buf = sw.rows[threadIdx.x >> 5];
   const int d = in.d;
   double part = 0.0;
@@ -3684,38 +3762,7 @@ __device__ __noinline__ double samples_joined(const InstDev &in, int pL, int pR,
       eR += sample_coord(in, k, m) * st;
       st *= in.n[m];
     }
-    double acc = 0.0;
-    for (int c = 0; c < len; c += 16) {
-      const bool has = c + el < len;
-      double xv[16], yv[16];
-#pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        const double *tab = (side == 0 ? in.tabL : in.tabR) + c + el;
-        const int64_t e = side == 0 ? eL : eR;
-        double v[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const int sr = 2 * q + half;
-          const int64_t es = __shfl_sync(FULL, e, sr);
-          const int vs = __shfl_sync(FULL, valid, sr);
-          v[q] = (vs && has) ? tab[es * len] : 0.0;
-        }
-        __syncwarp();  // the previous rows are read
-#pragma unroll
-        for (int q = 0; q < 16; ++q) buf[(2 * q + half) * 17 + el] = v[q];
-        __syncwarp();
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-          if (side == 0)
-            xv[t] = buf[lane * 17 + t];
-          else
-            yv[t] = buf[lane * 17 + t];
-        }
-      }
-#pragma unroll
-      for (int t = 0; t < 16; ++t)
-        if (c + t < len) acc = __fma_rn(xv[t], yv[t], acc);
-    }
+    const double acc = warp_chain_rows(in.tabL, eL, len, in.tabR, eR, len, len, buf);
     if (valid) {
       const double e = __dsub_rn(xk, acc);
       part = __fma_rn(e, e, part);
@@ -3867,7 +3914,7 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
             update_row(in, b, x - base, z);
           base += rows;
           for (int64_t x = item0(base); x < base + cols; x += NTI)
-            putR(in, B, (int64_t)z * B.ldR + (x - base), sb_entry(in, b, B.prow[z], x - base));
+            putR(in, B, z, x - base, sb_entry(in, b, B.prow[z], x - base));
           base += cols;
         }
         if (b < in.nb - 1 && ad[b + 1]) {
@@ -3877,7 +3924,7 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
           for (int64_t x = item0(base); x < base + nit; x += NTI) {
             const int64_t l = x - base, t = l / nb1, jj = l - t * nb1;
             const int64_t c = q * nb1 + jj;
-            putR(in, B, t * B.ldR + c, sb_entry(in, b, B.prow[t], c));
+            putR(in, B, t, c, sb_entry(in, b, B.prow[t], c));
           }
           base += nit;
         }
@@ -4059,11 +4106,11 @@ __device__ void phase_init3(const RunArgs &ra, PhaseSmem &sm) {
       for (int64_t x = first_item(base, gt, NTOT); x < base + rows; x += NTOT) {
         const int64_t a = x - base;
         const double s = __dsub_rn(0.0, sb_entry(in, b, a, c0));
-        putT(in, B, a, -__dmul_rn(delta, s));
+        putT(in, B, 0, a, -__dmul_rn(delta, s));
       }
       base += rows;
       for (int64_t x = first_item(base, gt, NTOT); x < base + cols; x += NTOT)
-        putR(in, B, x - base, sb_entry(in, b, a0, x - base));
+        putR(in, B, 0, x - base, sb_entry(in, b, a0, x - base));
       base += cols;
     }
   }
@@ -4238,13 +4285,11 @@ __global__ void __launch_bounds__(NT, 2) k_persistent(RunArgs ra) {
     if (!grid_barrier(ra, 4)) return;
     clk.lap(ra, T_DECIDE);
     if (ra.sampled) {
-      // the refinement of Alg. 1: a scan and a decide per step, then the
-      // stop tests on the refined pivots
+      // the refinement of Alg. 1, step by step, then the stop tests on the
+      // refined pivots
       for (int k = 0; k < 2 * ra.max_rook && any_rook(ra); ++k) {
-        phase_rook_scan(ra, sm);
+        phase_rook_step(ra, sm);
         if (!grid_barrier(ra, 10)) return;
-        phase_rook_decide(ra, sm);
-        if (!grid_barrier(ra, 11)) return;
       }
       clk.lap(ra, T_SCREEN);
       phase_finalize(ra, sm);
@@ -4303,13 +4348,9 @@ __global__ void __launch_bounds__(NT, 2) k_decide2(RunArgs ra) {
   cache_inst0(ra);
   phase_decide2(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem));
 }
-__global__ void __launch_bounds__(NT, 2) k_rook_scan(RunArgs ra) {
+__global__ void __launch_bounds__(NT, 2) k_rook_step(RunArgs ra) {
   cache_inst0(ra);
-  phase_rook_scan(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem));
-}
-__global__ void __launch_bounds__(NT, 2) k_rook_decide(RunArgs ra) {
-  cache_inst0(ra);
-  phase_rook_decide(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem));
+  phase_rook_step(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem));
 }
 __global__ void __launch_bounds__(NT, 2) k_finalize(RunArgs ra) {
   cache_inst0(ra);
@@ -4475,8 +4516,7 @@ cudaError_t launch_phase(int phase, const RunArgs &ra, int grid, cudaStream_t s)
     case PH_REFINE: f = (const void *)k_refine; break;
     case PH_DECIDE2: f = (const void *)k_decide2; break;
     case PH_VERIFY: f = (const void *)k_verify; break;
-    case PH_ROOK_SCAN: f = (const void *)k_rook_scan; break;
-    case PH_ROOK_DECIDE: f = (const void *)k_rook_decide; break;
+    case PH_ROOK_STEP: f = (const void *)k_rook_step; break;
     case PH_FINALIZE: f = (const void *)k_finalize; break;
     default: return cudaErrorInvalidValue;
   }
@@ -4577,7 +4617,7 @@ __global__ void __launch_bounds__(NT, 2) k_rebuild_rows(const InstDev *inp) {
   const int64_t gt = (int64_t)blockIdx.x * NT + threadIdx.x, NTOT = (int64_t)gridDim.x * NT;
   for (int64_t x = gt; x < r * nn; x += NTOT) {
     const int64_t t = x / nn, c = x - t * nn;
-    putR(in, B, t * B.ldR + c, sb_entry(in, bl, B.prow[t], c));
+    putR(in, B, t, c, sb_entry(in, bl, B.prow[t], c));
   }
 }
 
