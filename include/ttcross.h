@@ -358,7 +358,7 @@ ttc_status ttcross_check_tiles(int d, const int64_t *n, const int32_t *r, const 
    The result is written to *err, a caller-owned device double, in stream
    order on `stream`; the call returns after enqueueing two kernels.
    Scratch: a static 64 KiB device array per GPU holds one partial sum per
-   chunk of 4096 samples, so nsamples is limited to 16,777,216 (larger
+   chunk (at most 4096 chunks of at most 4096 samples), so nsamples is limited to 16,777,216 (larger
    requests return TTC_ERR_INVALID_ARG).  The first call on a device looks up
    that array's address; make it before any stream capture.  Calls outside a
    capture look it up again, so a call after cudaDeviceReset (which reloads

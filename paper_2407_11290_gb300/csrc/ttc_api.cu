@@ -1,5 +1,6 @@
 // ttc_api.cu -- the C ABI of include/ttcross.h: argument checks, the device
 // memory of an instance (one pooled allocation), and the launches.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1101,18 +1102,9 @@ ttc_status ttcross_rebuild_cores(ttc_handle *h, void *stream) {
     CU(cudaEventCreate(&h->ev2));
     CU(cudaEventCreate(&h->ev3));
   }
-  // the factors go, so that the cores come from the pivot sets alone
-  for (int b = 0; b < h->nb; ++b) {
-    const BondDev &B = h->hi.bond[b];
-    CU(cudaMemsetAsync(B.T, 0, sizeof(double) * B.cap * B.ldT, st));
-    CU(cudaMemsetAsync(B.hc, 0, sizeof(double) * B.cap * B.cap, st));
-    CU(cudaMemsetAsync(B.hpiv, 0, sizeof(double) * B.cap * B.cap, st));
-    CU(cudaMemsetAsync(B.delta, 0, sizeof(double) * B.cap, st));
-  }
-  const BondDev &BL = h->hi.bond[h->nb - 1];
-  CU(cudaMemsetAsync(BL.R, 0, sizeof(double) * BL.cap * BL.ldR, st));
+  const int rmax = *std::max_element(h->h_ctrl.r, h->h_ctrl.r + h->nb);
   CU(cudaEventRecord(h->ev2, st));
-  CU(launch_rebuild_cores(h->d_inst, h->nb, h->rebuild_scratch, h->grid, st));
+  CU(launch_rebuild_cores(h->d_inst, h->nb, rmax, h->rebuild_scratch, h->grid, st));
   CU(cudaEventRecord(h->ev3, st));
   h->rebuilt = true;
   return TTC_OK;

@@ -120,7 +120,8 @@ struct SpreadSmem {
 constexpr int RB_WARPS = 2, RB_STAGES = 3;
 constexpr int RB_SMALL = 64;  // pivots up to which a warp rebuilds eight rows
 constexpr int RB_BUF = 2 * RCAP + RCAP + 2 * RB_STAGES * RCAP;
-static_assert(RB_BUF >= 2 * 8 * (RB_SMALL + 1) + RB_SMALL + 2 * RB_STAGES * RB_SMALL, "replay buffer");
+constexpr int RB_BUF_SMALL = 2 * 8 * (RB_SMALL + 1) + RB_SMALL + 2 * RB_STAGES * RB_SMALL;
+static_assert(RB_BUF >= RB_BUF_SMALL, "replay buffer");
 struct ReplaySmem {
   double red_pad[NT / 32];
   double buf[RB_WARPS][RB_BUF];
@@ -3175,99 +3176,6 @@ __device__ __forceinline__ void pivot_col_entries(const InstDev &in, int b, int6
   }
 }
 
-// Alg. 4 for row a of bond b (eq. aca_approx_T_sub for pivots 0..nz-1 in
-// insertion order) by one warp (core construction from the pivots): lane u
-// keeps T(a, 32k + u), k < K, in registers.  Step z runs the contract's chain
-// over t < z on every lane from broadcasts (the serial order is the
-// contract's), then each lane updates its own entries.  The next history row
-// loads during this step when PF.
-template <int K, bool PF>
-__device__ __noinline__ void replay_row_warp(const InstDev &in, int b, int64_t a, int nz) {
-  const BondDev &B = in.bond[b];
-  const int lane = threadIdx.x & 31;
-  const int64_t cap = B.cap;
-  constexpr unsigned FULL = 0xffffffffu;
-  const double *hcb = B.hc;
-  const double *hpb = B.hpiv;
-  const double *dlb = B.delta;
-  auto off = [&](int z) -> int64_t { return (int64_t)z * cap; };
-  double tr[K], en[K], hc[K], hp[K], hcn[K], hpn[K];
-  if (in.gen == 0) {
-    const int64_t nb0 = in.n[b];
-    const int64_t p = a / nb0, i = a - p * nb0;
-    const int32_t rs = left_set(in, b).sum[p] + (int32_t)i;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int t = 32 * k + lane;
-      en[k] = t < nz ? in.hilb[rs + B.J.sum[t]] : 0.0;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int t = 32 * k + lane;
-      en[k] = t < nz ? sb_entry(in, b, a, B.pcol[t]) : 0.0;
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    tr[k] = 0.0;
-    hcn[k] = 0.0;
-    hpn[k] = 0.0;
-  }
-  double dn = nz > 0 ? dlb[0] : 0.0;
-  for (int z = 0; z < nz; ++z) {
-    const double dz = dn;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int t = 32 * k + lane;
-      if (PF) {
-        hc[k] = hcn[k];
-        hp[k] = hpn[k];
-      } else {
-        hc[k] = t < z ? hcb[off(z) + t] : 0.0;
-        hp[k] = t < z ? hpb[off(z) + t] : 0.0;
-      }
-    }
-    if (z + 1 < nz) {
-      dn = dlb[z + 1];
-      if (PF) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          const int t = 32 * k + lane;
-          hcn[k] = t < z + 1 ? hcb[off(z + 1) + t] : 0.0;
-          hpn[k] = t < z + 1 ? hpb[off(z + 1) + t] : 0.0;
-        }
-      }
-    }
-    double acc = 0.0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      if (32 * k >= z) break;
-      const int lim = min(32, z - 32 * k);
-      for (int u = 0; u < lim; ++u)
-        acc = __fma_rn(__shfl_sync(FULL, tr[k], u), __shfl_sync(FULL, hc[k], u), acc);
-    }
-    double ez = 0.0;
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-      if (k == (z >> 5)) ez = __shfl_sync(FULL, en[k], z & 31);
-    const double w = __dmul_rn(dz, __dsub_rn(acc, ez));
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int t = 32 * k + lane;
-      if (t < z)
-        tr[k] = __fma_rn(w, hp[k], tr[k]);
-      else if (t == z)
-        tr[k] = -w;
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int t = 32 * k + lane;
-    if (t < nz) putT(in, B, t, a, tr[k]);
-  }
-}
-
 // Alg. 4 for up to 32 / LPR rows of bond b by one warp, LPR lanes a row: the
 // steps of update_row, the same FMAs in the same order.  The contract's chain
 // of step z is z dependent FMAs; its operands T(a, t) and c_z(t) come from
@@ -3283,12 +3191,11 @@ __device__ __noinline__ void replay_row_warp(const InstDev &in, int b, int64_t a
 // and in local memory), one row a warp (LPR 32) where they are long.  (With
 // the row in registers and two shuffles per chain element a row of 256 pivots
 // took 2.3 times its floor: 200 ms of update phases in the 6D Maxwellian.)
-template <int LPR>
+template <int LPR, int NZM>  // NZM: pivots at most
 __device__ __noinline__ void replay_group(const InstDev &in, int b, int64_t a0, int nrows, int nz,
                                           double *buf) {
   constexpr int RPW = 32 / LPR;                                // rows of the warp
-  constexpr int NZM = LPR == 32 ? RCAP : RB_SMALL;             // pivots at most
-  constexpr int LD = LPR == 32 ? RCAP : RB_SMALL + 1;          // row stride (bank spread)
+  constexpr int LD = LPR == 32 ? NZM : NZM + 1;                // row stride (bank spread)
   const BondDev &B = in.bond[b];
   const int lane = threadIdx.x & 31, s = lane % LPR, rI = min(lane / LPR, nrows - 1);
   const int64_t cap = B.cap, a = a0 + rI;
@@ -3371,9 +3278,9 @@ __device__ __forceinline__ int replay_warps(const InstDev &in, int b, int nz) {
 __device__ void replay_rows(const InstDev &in, int b, int64_t p, int nz, int g, double *buf) {
   const int64_t nit = in.n[b], i0 = (int64_t)g * replay_rows_per_warp(nz);
   if (nz <= RB_SMALL)
-    replay_group<4>(in, b, p * nit + i0, (int)min((int64_t)8, nit - i0), nz, buf);
+    replay_group<4, RB_SMALL>(in, b, p * nit + i0, (int)min((int64_t)8, nit - i0), nz, buf);
   else
-    replay_group<32>(in, b, p * nit + i0, 1, nz, buf);
+    replay_group<32, RCAP>(in, b, p * nit + i0, 1, nz, buf);
 }
 
 __device__ void update_row(const InstDev &in, int b, int64_t a, int z) {
@@ -4536,13 +4443,17 @@ cudaError_t launch_phase(int phase, const RunArgs &ra, int grid, cudaStream_t s)
 // Core construction from the pivot sets alone (Alg. 5, second loop; Sec.
 // 3.2.2 and eq. corereshape): the history of Alg. 4 is rebuilt for every
 // bond, then every superblock row of T_k is replayed from it, sliced over the
-// grid (a row per warp), and the last bond's R is formed from the entries.
+// grid (replay_group), and the last bond's R is formed from the entries.
 // By the arithmetic contract every value equals the one the sweeps kept.
 
-// history of bond blockIdx.x (one CTA per bond), step by step: before step
-// t every pivot row a_z (z >= t) holds T(a_z, :t); step t takes its column
-// c_t = R(:t, c_t) = A(a_u, c_t), its snapshot T(a_t, :t) and delta_t, then
-// applies itself to the later pivot rows (a thread per row)
+// history of bond blockIdx.x (one CTA per bond).  M starts as the entries
+// A(a_z, c_u) of the pivot rows and columns (k_rebuild_start); before step t
+// row z >= t holds T(a_z, :t) in its first t places.  Step t takes its column
+// c_t = A(a_u, c_t) (u < t), its snapshot T(a_t, :t) and delta_t, a thread per
+// row z >= t runs the chain over c_t (z = t gives the pivot), and the updates
+// of the later rows are dealt over the CTA.  Serial in t: a step is a chain of t
+// FMAs (63 cycles each), a divide and three CTA barriers, so M lies in
+// shared memory where it fits (up to RB_SMALL pivots).
 __global__ void __launch_bounds__(NT) k_rebuild_history(const InstDev *inp, double *scratch) {
   const InstDev &in = *inp;
   const int b = blockIdx.x;
@@ -4550,65 +4461,80 @@ __global__ void __launch_bounds__(NT) k_rebuild_history(const InstDev *inp, doub
   const BondDev &B = in.bond[b];
   const int r = in.ctrl->r[b];
   const int64_t cap = B.cap;
-  double *Tp = scratch + (int64_t)b * RCAP * RCAP;  // [z][u]: T(a_z, u) of pivot row z
-  __shared__ double s_hc[RCAP], s_hp[RCAP];
+  const bool small = r <= RB_SMALL;
+  const int64_t ld = small ? RB_SMALL + 1 : RCAP;
+  double *M = small ? reinterpret_cast<double *>(dyn_smem) : scratch + (int64_t)b * RCAP * RCAP;
+  __shared__ double s_hc[RCAP], s_hp[RCAP], s_w[RCAP];
   __shared__ double s_delta;
   __shared__ int s_ok;
-  for (int x = threadIdx.x; x < r * r; x += NT) Tp[x] = 0.0;
+  for (int x = threadIdx.x; small && x < r * r; x += NT) {
+    const int z = x / r, u = x - z * r;
+    M[z * ld + u] = scratch[((int64_t)b * RCAP + z) * RCAP + u];
+  }
   __syncthreads();
   for (int t = 0; t < r; ++t) {
     // c_t restricted to the earlier pivots, and row a_t's snapshot
     for (int u = threadIdx.x; u < t; u += NT) {
-      const double c = sb_entry(in, b, B.prow[u], B.pcol[t]);
-      s_hc[u] = c;
-      s_hp[u] = Tp[(int64_t)t * RCAP + u];
-      B.hc[(int64_t)t * cap + u] = c;
+      s_hc[u] = M[u * ld + t];
+      s_hp[u] = M[t * ld + u];
+      B.hc[(int64_t)t * cap + u] = s_hc[u];
       B.hpiv[(int64_t)t * cap + u] = s_hp[u];
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      const double piv = __dsub_rn(sb_entry(in, b, B.prow[t], B.pcol[t]), chain(s_hp, 1, s_hc, 1, t));
-      s_delta = 1.0 / piv;
-      s_ok = isfinite(s_delta) ? 1 : 0;
-      B.delta[t] = s_delta;
+    for (int z = t + threadIdx.x; z < r; z += NT) {
+      const double acc = chain(M + z * ld, 1, s_hc, 1, t), e = M[z * ld + t];
+      if (z == t) {
+        s_delta = 1.0 / __dsub_rn(e, acc);
+        s_ok = isfinite(s_delta) ? 1 : 0;
+        B.delta[t] = s_delta;
+      } else {
+        s_w[z] = __dsub_rn(acc, e);
+      }
     }
     __syncthreads();
     if (!s_ok) return;  // no such pivot was taken (the sweeps check the same value)
     const double dt = s_delta;
     // step t on the later pivot rows z > t
-    for (int z = t + 1 + threadIdx.x; z < r; z += NT) {
-      double *Tz = Tp + (int64_t)z * RCAP;
-      const double sv = __dsub_rn(chain(Tz, 1, s_hc, 1, t), sb_entry(in, b, B.prow[z], B.pcol[t]));
-      const double w = __dmul_rn(dt, sv);
-      for (int u = 0; u < t; ++u) Tz[u] = __fma_rn(w, s_hp[u], Tz[u]);
-      Tz[t] = -w;
+    for (int x = threadIdx.x; x < (r - t - 1) * (t + 1); x += NT) {
+      const int z = t + 1 + x / (t + 1), u = x % (t + 1);
+      const double w = __dmul_rn(dt, s_w[z]);
+      M[z * ld + u] = u < t ? __fma_rn(w, s_hp[u], M[z * ld + u]) : -w;
     }
     __syncthreads();
   }
 }
 
 // every superblock row of every bond replayed through its whole history
-// (Alg. 4), a row per warp, rows dealt over the grid; then R of the last
-// bond (its core) from the entries
-__global__ void __launch_bounds__(NT, 2) k_rebuild_rows(const InstDev *inp) {
+// (Alg. 4), groups of rows dealt over the grid; then R of the last bond (its
+// core) from the entries.  FP64 issue bounds it where rows are many: a warp's
+// instruction costs the same for one row as for eight, so up to RB_SMALL pivots
+// a warp takes eight rows (6D Hilbert n = 300, ranks 15..18, history and rows:
+// 0.34 -> 0.11 ms
+// with the clearing; a random TT of ranks 48: 22.5 -> 1.5 ms).  Rows that fill at most a quarter of the grid's warps (four
+// warps keep an SM's FP64 pipe busy) take a warp each, which is shorter.
+__global__ void __launch_bounds__(NT, 2) k_rebuild_rows(const InstDev *inp, int words) {
   const InstDev &in = *inp;
+  double *buf = reinterpret_cast<double *>(dyn_smem) + (threadIdx.x >> 5) * words;
   const int64_t nwarps = (int64_t)gridDim.x * (NT / 32);
-  const int64_t gw = (int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
+  // neighbouring groups on different CTAs: few groups still use every SM
+  const int64_t gw = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   int64_t base = 0;
   for (int b = 0; b < in.nb; ++b) {
     const int r = in.ctrl->r[b];
     const int64_t rows = (int64_t)(b == 0 ? 1 : in.ctrl->r[b - 1]) * in.n[b];
-    for (int64_t a = ((gw - base) % nwarps + nwarps) % nwarps; a < rows; a += nwarps) {
-      if (r <= 32)
-        replay_row_warp<1, true>(in, b, a, r);
-      else if (r <= 64)
-        replay_row_warp<2, true>(in, b, a, r);
-      else if (r <= 128)
-        replay_row_warp<4, true>(in, b, a, r);
+    const bool wide = r <= RB_SMALL && rows > nwarps / 4;
+    const int rpw = wide ? 8 : 1;
+    const int64_t groups = (rows + rpw - 1) / rpw;
+    for (int64_t g = ((gw - base) % nwarps + nwarps) % nwarps; g < groups; g += nwarps) {
+      const int64_t a0 = g * rpw;
+      if (wide)
+        replay_group<4, RB_SMALL>(in, b, a0, (int)min((int64_t)8, rows - a0), r, buf);
+      else if (r <= RB_SMALL)
+        replay_group<32, RB_SMALL>(in, b, a0, 1, r, buf);
       else
-        replay_row_warp<8, false>(in, b, a, r);
+        replay_group<32, RCAP>(in, b, a0, 1, r, buf);
     }
-    base += rows;
+    base += groups;
   }
   const int bl = in.nb - 1;
   const BondDev &B = in.bond[bl];
@@ -4621,12 +4547,48 @@ __global__ void __launch_bounds__(NT, 2) k_rebuild_rows(const InstDev *inp) {
   }
 }
 
-cudaError_t launch_rebuild_cores(const InstDev *d_inst, int nb, double *scratch, int grid,
-                                 cudaStream_t s) {
-  k_rebuild_history<<<nb, NT, 0, s>>>(d_inst, scratch);
-  cudaError_t e = cudaGetLastError();
+// the factors and histories go, so that the cores come from the pivot sets
+// alone (one launch; a memset per buffer was 4 per bond), and the entries of
+// the pivot rows and columns are formed over the whole grid
+__global__ void __launch_bounds__(NT) k_rebuild_start(const InstDev *inp, double *scratch) {
+  const InstDev &in = *inp;
+  const int64_t gt = (int64_t)blockIdx.x * NT + threadIdx.x, NTOT = (int64_t)gridDim.x * NT;
+  for (int b = 0; b < in.nb; ++b) {
+    const BondDev &B = in.bond[b];
+    const int64_t cap = B.cap;
+    for (int64_t x = gt; x < cap * B.ldT; x += NTOT) B.T[x] = 0.0;
+    for (int64_t x = gt; x < cap * cap; x += NTOT) {
+      B.hc[x] = 0.0;
+      B.hpiv[x] = 0.0;
+    }
+    for (int64_t x = gt; x < cap; x += NTOT) B.delta[x] = 0.0;
+    if (b == in.nb - 1)
+      for (int64_t x = gt; x < cap * B.ldR; x += NTOT) B.R[x] = 0.0;
+    const int r = in.ctrl->r[b];
+    for (int64_t x = gt; x < r * r; x += NTOT) {
+      const int z = (int)x / r, u = (int)x - z * r;
+      scratch[((int64_t)b * RCAP + z) * RCAP + u] = sb_entry(in, b, B.prow[z], B.pcol[u]);
+    }
+  }
+}
+
+// rmax: the largest rank (sizes the replay buffers: two CTAs a SM up to RB_SMALL)
+cudaError_t launch_rebuild_cores(const InstDev *d_inst, int nb, int rmax, double *scratch,
+                                 int grid, cudaStream_t s) {
+  const int words = rmax <= RB_SMALL ? RB_BUF_SMALL : RB_BUF;
+  const int bytes = words * (NT / 32) * (int)sizeof(double);
+  const int hist = RB_SMALL * (RB_SMALL + 1) * (int)sizeof(double);  // 33 KB
+  cudaError_t e = cudaFuncSetAttribute((const void *)k_rebuild_rows,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       RB_BUF * (NT / 32) * (int)sizeof(double));
   if (e != cudaSuccess) return e;
-  k_rebuild_rows<<<grid, NT, 0, s>>>(d_inst);
+  k_rebuild_start<<<grid, NT, 0, s>>>(d_inst, scratch);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_rebuild_history<<<nb, NT, hist, s>>>(d_inst, scratch);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_rebuild_rows<<<grid, NT, bytes, s>>>(d_inst, words);
   return cudaGetLastError();
 }
 
