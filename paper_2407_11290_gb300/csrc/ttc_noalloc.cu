@@ -9,11 +9,11 @@
 // sums it needs live in the file-scope array below, not in memory from
 // cudaMalloc.
 //
-// The array is a fixed 64 KiB per GPU: every device that loads the library
-// holds it until the process exits.  All calls share it, and each call
+// The arrays are a fixed 66 KiB per GPU: every device that loads the library
+// holds them until the process exits.  All calls share them, and each call
 // overwrites every slot it later reads, so nothing has to be cleared; but two
 // calls whose kernels overlap on the GPU (different streams, or different
-// host threads on one device) race on it and must be ordered by the caller.
+// host threads on one device) race on them and must be ordered by the caller.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -41,6 +41,8 @@ constexpr int kMaxDevices = 64;
 
 // (sum (X - X~)^2, sum X^2) of every chunk of samples
 static __device__ __align__(256) double g_chunk_sums[2 * kMaxChunks];
+// largest exponent of row k of middle core m (the tensor-core form)
+static __device__ int32_t g_row_exp[kMaxD][32];
 
 struct ErrArgs {
   int32_t d;
@@ -201,9 +203,14 @@ __global__ void __launch_bounds__(kThreads) k_chunk_sums(ErrArgs a, int64_t nchu
 // the samples by each middle index in turn and multiplies every run of up to
 // 16 samples of one index by that index's core slice, whose columns a warp
 // brings to fixed point itself.
+// Fixed point is as fine as its largest term, and a TT's bonds may be scaled at
+// will (a column of one core up, the row of the next down by as much).  So the
+// rows of a middle core are taken at their largest exponent, k_row_exp, and the
+// columns before them grow by it: both are exponents, no product is rounded.
 // A warp per sample in FP64 issued one FMA per core row with half its lanes
 // idle at size 16: 6.57 ms for 1e6 samples of a 6D n = 64 TT of ranks 16 (its
-// 1.04e9 FMAs take 1.7 ms at the FP64 pipe's rate).
+// 1.04e9 FMAs take 1.7 ms at the FP64 pipe's rate); this form takes 1.10 ms,
+// 0.09 ms of them for the rows' exponents.
 constexpr int kTcThreads = 512, kTcN = 256;
 
 template <int KP>
@@ -267,6 +274,34 @@ __device__ void tc_sort(const ErrArgs &a, int64_t k0, int ns, int m, TcSmem<KP> 
   __syncthreads();
 }
 
+// g_row_exp: a CTA per row of a middle core; 0 for a row of zeros
+__global__ void __launch_bounds__(kThreads) k_row_exp(ErrArgs a) {
+  const int m = (int)blockIdx.y + 1, k = (int)blockIdx.x;
+  if (k >= a.s[m]) return;
+  const int64_t len = a.n[m] * a.s[m + 1];
+  const double *G = a.core[m] + (int64_t)k * len;
+  int e = 0;
+  for (int64_t x = threadIdx.x; x < len; x += kThreads) {
+    const int v = ttc::tc_expo(G[x]);
+    if (v != 0x7ff) e = max(e, v);  // (the products find what is not finite)
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  __shared__ int red[kWarps];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < kWarps; ++i) e = max(e, red[i]);
+    g_row_exp[m][k] = e ? e - 1023 : 0;
+  }
+}
+
+// the unit's exponent of a row or column from its largest exponent (kNone: it
+// is zero) and whether an entry was not finite
+constexpr int32_t kNone = -(1 << 20);
+__device__ __forceinline__ int32_t tc_unit_of(int emax, bool bad) {
+  return bad ? ttc::TC_BAD : emax - 1084;
+}
+
 // one middle core: rows of the vectors times G_m(i), in place; the last one
 // meets the last core and leaves the residuals
 template <int KP>
@@ -279,6 +314,14 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
   const int K = a.s[m], N = a.s[m + 1];
   const bool last = m == a.d - 2;
   const int64_t ld = a.n[m] * N;
+  int32_t rx[KS][4];  // of the rows that the lane reads
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = ks * 16 + 2 * t + (q & 1) + 8 * (q >> 1);
+      rx[ks][q] = k < K ? g_row_exp[m][k] : 0;
+    }
   for (int x = warp; x < sm.ntiles; x += kTcThreads / 32) {
     const uint32_t tl = sm.tile[x];
     const int i = (int)(tl >> 16), at = (int)(tl >> 4) & 0xfff, rows = (int)(tl & 15) + 1;
@@ -312,7 +355,8 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
       // the lane's entries of column u, their largest exponent over the column
       const int u = 8 * c + g;
       double w[KS][4];
-      int emax = 0;
+      int emax = kNone;
+      bool inf = false;
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
@@ -323,10 +367,14 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) emax = max(emax, tc_expo(w[ks][q]));
+        for (int q = 0; q < 4; ++q) {
+          const int e = tc_expo(w[ks][q]);
+          inf |= e == 0x7ff;
+          if (e) emax = max(emax, e - rx[ks][q]);
+        }
       emax = max(emax, __shfl_xor_sync(FULL, emax, 1));
       emax = max(emax, __shfl_xor_sync(FULL, emax, 2));
-      const int32_t ge = tc_unit(emax);
+      const int32_t ge = tc_unit_of(emax, inf);
       ea[c] = __shfl_sync(FULL, ge, 8 * t);      // columns 2t, 2t + 1: lanes 4 (2t), 4 (2t + 1)
       eb[c] = __shfl_sync(FULL, ge, 8 * t + 4);
       bad |= ge == TC_BAD;
@@ -337,8 +385,8 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
         for (int q = 0; q < 4; ++q) acc[l][q] = TC_MAGIC;
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks) {
-        const uint4 z0 = tc_pack(tc_fix(w[ks][0], emax), tc_fix(w[ks][1], emax));
-        const uint4 z1 = tc_pack(tc_fix(w[ks][2], emax), tc_fix(w[ks][3], emax));
+        const uint4 z0 = tc_pack(tc_fix(w[ks][0], emax + rx[ks][0]), tc_fix(w[ks][1], emax + rx[ks][1]));
+        const uint4 z1 = tc_pack(tc_fix(w[ks][2], emax + rx[ks][2]), tc_fix(w[ks][3], emax + rx[ks][3]));
         uint32_t db[8][2];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -370,6 +418,10 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
         v1 = __fma_rn(tc_real(out[c][2], e1 + ea[c] + 88 - sh), ya1, v1);
         v1 = __fma_rn(tc_real(out[c][3], e1 + eb[c] + 88 - sh), yb1, v1);
       } else {
+        // from here on at the scale of the next core's rows
+        const int ua = 8 * c + 2 * t;
+        if (ua < N && ea[c] != TC_BAD) ea[c] += g_row_exp[m + 1][ua];
+        if (ua + 1 < N && eb[c] != TC_BAD) eb[c] += g_row_exp[m + 1][ua + 1];
         if (out[c][0]) top0 = max(top0, ea[c] + 64 - __clzll(llabs(out[c][0])));
         if (out[c][1]) top0 = max(top0, eb[c] + 64 - __clzll(llabs(out[c][1])));
         if (out[c][2]) top1 = max(top1, ea[c] + 64 - __clzll(llabs(out[c][2])));
@@ -433,12 +485,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_sums(ErrArgs a, int64_t ch
       for (int s = tid; s < ns; s += kTcThreads) {
         const int K = a.s[1];
         const double *G = a.core[0] + (int64_t)coord(a, k0 + s, 0) * K;
-        int emax = 0;
-        for (int k = 0; k < K; ++k) emax = max(emax, tc_expo(G[k]));
+        int emax = kNone;
+        bool inf = false;
+        for (int k = 0; k < K; ++k) {
+          const int e = tc_expo(G[k]);
+          inf |= e == 0x7ff;
+          if (e) emax = max(emax, e + g_row_exp[1][k]);
+        }
         for (int k = 0; k < KP; k += 2)
           *reinterpret_cast<uint4 *>(&sm.vec[s][k]) =
-              tc_pack(k < K ? tc_fix(G[k], emax) : TC_BIAS, k + 1 < K ? tc_fix(G[k + 1], emax) : TC_BIAS);
-        sm.unit[s] = tc_unit(emax);
+              tc_pack(k < K ? tc_fix(G[k], emax - g_row_exp[1][k]) : TC_BIAS,
+                      k + 1 < K ? tc_fix(G[k + 1], emax - g_row_exp[1][k + 1]) : TC_BIAS);
+        sm.unit[s] = tc_unit_of(emax, inf);
       }
       for (int m = 1; m < a.d - 1; ++m) {
         tc_sort<KP>(a, k0, ns, m, sm);
@@ -472,6 +530,9 @@ cudaError_t launch_tc(const ErrArgs &a, int64_t chunk, int64_t nchunks, int nsm,
   const void *f = (const void *)k_tc_sums<KP>;
   cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sizeof(TcSmem<KP>));
+  if (e != cudaSuccess) return e;
+  k_row_exp<<<dim3(32, (unsigned)(a.d - 2)), kThreads, 0, cs>>>(a);
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t grid = std::min<int64_t>(nchunks, nsm);
   k_tc_sums<KP><<<(unsigned)grid, kTcThreads, sizeof(TcSmem<KP>), cs>>>(a, chunk, nchunks, sums);
