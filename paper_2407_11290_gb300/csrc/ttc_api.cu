@@ -827,16 +827,17 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
   ttc_status s = ensure_cands(h, nullptr);
   if (s != TTC_OK) return cleanup(s);
   if (I.tc_perm) {
-    for (int m = 1; m < d - 1; ++m)
-      if (cudaMemset(const_cast<uint32_t *>(I.tc_tile[m]), 0xFF,
-                     sizeof(uint32_t) * (size_t)(I.tc_stride / TC_BLOCK * (TC_BLOCK / 16 + n[m]))) !=
-          cudaSuccess)
-        return cleanup(fail(TTC_ERR_CUDA, "cudaMemset of the sample tiles failed"));
+    // (the modes' tiles lie one after the other in the pool)
+    const uint32_t *t0 = I.tc_tile[1];
+    const uint32_t *t1 = I.tc_tile[d - 2] + I.tc_stride / TC_BLOCK * (TC_BLOCK / 16 + n[d - 2]);
+    if (cudaMemset(const_cast<uint32_t *>(t0), 0xFF, sizeof(uint32_t) * (size_t)(t1 - t0)) !=
+        cudaSuccess)
+      return cleanup(fail(TTC_ERR_CUDA, "cudaMemset of the sample tiles failed"));
     // (the tile arrays' pointers are part of the descriptor on the device)
     const size_t at = reinterpret_cast<char *>(&I.tc_tile[0]) - reinterpret_cast<char *>(&I);
     uint32_t *const *tiles = reinterpret_cast<uint32_t *const *>(reinterpret_cast<char *>(h->d_inst) + at);
-    if (launch_tc_perm(h->d_inst, d, I.tc_stride / TC_BLOCK, const_cast<uint16_t *>(I.tc_perm), tiles) !=
-        cudaSuccess)
+    if (launch_tc_perm(h->d_inst, d, *std::max_element(n + 1, n + d - 1), I.tc_stride / TC_BLOCK,
+                       const_cast<uint16_t *>(I.tc_perm), tiles) != cudaSuccess)
       return cleanup(fail(TTC_ERR_CUDA, "sorting the error samples failed"));
   }
   if (mxtab) {

@@ -4508,10 +4508,10 @@ __global__ void __launch_bounds__(NT) k_rebuild_history(const InstDev *inp, doub
 // (Alg. 4), groups of rows dealt over the grid; then R of the last bond (its
 // core) from the entries.  FP64 issue bounds it where rows are many: a warp's
 // instruction costs the same for one row as for eight, so up to RB_SMALL pivots
-// a warp takes eight rows (6D Hilbert n = 300, ranks 15..18, history and rows:
-// 0.34 -> 0.11 ms
-// with the clearing; a random TT of ranks 48: 22.5 -> 1.5 ms).  Rows that fill at most a quarter of the grid's warps (four
-// warps keep an SM's FP64 pipe busy) take a warp each, which is shorter.
+// a warp takes eight rows (6D Hilbert n = 300, ranks 15..18, history and rows
+// with the clearing: 0.34 -> 0.11 ms; a random TT of ranks 48: 22.5 -> 1.5 ms).
+// Rows that fill at most a quarter of the grid's warps (four warps keep an SM's
+// FP64 pipe busy) take a warp each, which is shorter.
 __global__ void __launch_bounds__(NT, 2) k_rebuild_rows(const InstDev *inp, int words) {
   const InstDev &in = *inp;
   double *buf = reinterpret_cast<double *>(dyn_smem) + (threadIdx.x >> 5) * words;
@@ -4724,21 +4724,23 @@ cudaError_t launch_user_samples(const InstDev *d_inst, int32_t *idx, cudaStream_
 
 // The samples of block blockIdx.x in the order of their index of mode
 // m = 1 + blockIdx.y (stable), and their tiles (create time; the tile slots
-// are all TC_NO_TILE before).  Eight warps take eighths of the block: each
+// are all TC_NO_TILE before).  PW warps take equal parts of the block: each
 // counts its samples per index, the counts (and the tiles they make) are
-// scanned over (index, warp), each warp places its samples.
-constexpr int TC_PW = 8;
-__global__ void __launch_bounds__(32 * TC_PW) k_tc_perm(const InstDev *inp, uint16_t *perm,
-                                                        uint32_t *const *tiles) {
+// scanned over (index, warp), each warp places its samples.  A warp's steps are
+// serial, so as many warps as the counts' shared memory has room for: 32 up to
+// 512 indices, 8 up to TC_NMAX.
+template <int PW, int NM>
+__global__ void __launch_bounds__(32 * PW) k_tc_perm(const InstDev *inp, uint16_t *perm,
+                                                     uint32_t *const *tiles) {
   constexpr unsigned FULL = 0xffffffffu;
-  constexpr int SEG = TC_BLOCK / TC_PW;
-  __shared__ uint16_t cnt[TC_PW][TC_NMAX];
-  __shared__ int32_t wsum[TC_PW], wtile[TC_PW];
+  constexpr int SEG = TC_BLOCK / PW;
+  __shared__ uint16_t cnt[PW][NM];
+  __shared__ int32_t wsum[PW], wtile[PW];
   const InstDev &in = *inp;
   const int m = 1 + blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int n = (int)in.n[m];
   const int64_t k0 = (int64_t)blockIdx.x * TC_BLOCK;
-  for (int x = threadIdx.x; x < TC_PW * n; x += blockDim.x) cnt[x / n][x % n] = 0;
+  for (int x = threadIdx.x; x < PW * n; x += blockDim.x) cnt[x / n][x % n] = 0;
   __syncthreads();
   for (int pass = 0; pass < 2; ++pass) {
     uint16_t *pm = perm + (int64_t)(m - 1) * in.tc_stride + k0;
@@ -4761,7 +4763,7 @@ __global__ void __launch_bounds__(32 * TC_PW) k_tc_perm(const InstDev *inp, uint
     int sum = 0, nti = 0;
     for (int i = i0; i < i1; ++i) {
       int v = 0;
-      for (int q = 0; q < TC_PW; ++q) v += cnt[q][i];
+      for (int q = 0; q < PW; ++q) v += cnt[q][i];
       sum += v;
       nti += (v + 15) / 16;
     }
@@ -4786,7 +4788,7 @@ __global__ void __launch_bounds__(32 * TC_PW) k_tc_perm(const InstDev *inp, uint
     uint32_t *tl = tiles[m] + (int64_t)blockIdx.x * (TC_BLOCK / 16 + n);
     for (int i = i0; i < i1; ++i) {
       const int first = at;
-      for (int q = 0; q < TC_PW; ++q) {
+      for (int q = 0; q < PW; ++q) {
         const int v = cnt[q][i];
         cnt[q][i] = (uint16_t)at;
         at += v;
@@ -4798,9 +4800,13 @@ __global__ void __launch_bounds__(32 * TC_PW) k_tc_perm(const InstDev *inp, uint
   }
 }
 
-cudaError_t launch_tc_perm(const InstDev *d_inst, int d, int64_t blocks, uint16_t *perm,
+cudaError_t launch_tc_perm(const InstDev *d_inst, int d, int64_t nmax, int64_t blocks, uint16_t *perm,
                            uint32_t *const *tiles) {
-  k_tc_perm<<<dim3((unsigned)blocks, (unsigned)(d - 2)), 32 * TC_PW>>>(d_inst, perm, tiles);
+  const dim3 g((unsigned)blocks, (unsigned)(d - 2));
+  if (nmax <= 512)
+    k_tc_perm<32, 512><<<g, 32 * 32>>>(d_inst, perm, tiles);
+  else
+    k_tc_perm<8, TC_NMAX><<<g, 32 * 8>>>(d_inst, perm, tiles);
   return cudaGetLastError();
 }
 

@@ -31,7 +31,7 @@ cudaError_t launch_user_samples(const InstDev *d_inst, int32_t *idx, cudaStream_
 // error check on the tensor cores: the samples sorted by every middle index
 // (perm and the device array of tile arrays, on the legacy stream), the bytes
 // of a plan
-cudaError_t launch_tc_perm(const InstDev *d_inst, int d, int64_t blocks, uint16_t *perm,
+cudaError_t launch_tc_perm(const InstDev *d_inst, int d, int64_t nmax, int64_t blocks, uint16_t *perm,
                            uint32_t *const *tiles);
 size_t tc_plan_bytes();
 cudaError_t launch_maxwellian_tables(const InstDev *d_inst, double *coef, double *nh, double *uv);
