@@ -294,7 +294,7 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
   ra.stored = 0;
   for (int i = 0; i < count; ++i)
     if (hs[i]->hi.stored && hs[i]->hi.prec == P_FP64) ra.stored = 1;
-  ra.max_rook = 0;
+  ra.max_rook = ra.rook_step = 0;
   for (int i = 0; i < count; ++i)
     if (hs[i]->hi.nl > 0) {
       ra.sampled = 1;
@@ -336,7 +336,8 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
     CU(launch_phase(PH_DECIDE, ra, h0->grid, s));
     if (ra.sampled) {
       // refinement rounds: a launch per step (no-ops once every bond is done)
-      for (int k = 0; k < 2 * ra.max_rook; ++k) CU(launch_phase(PH_ROOK_STEP, ra, h0->grid, s));
+      for (ra.rook_step = 0; ra.rook_step < 2 * ra.max_rook; ++ra.rook_step)
+        CU(launch_phase(PH_ROOK_STEP, ra, h0->grid, s));
       CU(launch_phase(PH_FINALIZE, ra, h0->grid, s));
     }
     if (ra.mixed) {

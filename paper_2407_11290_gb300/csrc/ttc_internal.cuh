@@ -113,9 +113,9 @@ struct Ctrl {
   int64_t entries_fresh;     // entries evaluated as A - T R (the rest carried)
   int64_t stored_bytes;      // bytes of E read and written by the screens
   // sampled screen: refinement step of each bond (0 none / done, 1 the
-  // column of the pivot next, 2 its row next), rounds run, whether the
-  // running round moved the pivot
-  int32_t rook_stage[TTC_MAXD], rook_round[TTC_MAXD], rook_moved[TTC_MAXD];
+  // column of the pivot next, 2 its row next; step k reads copy k mod 2 and
+  // writes the other), rounds run, whether the running round moved the pivot
+  int32_t rook_stage[2][TTC_MAXD], rook_round[TTC_MAXD], rook_moved[TTC_MAXD];
   int64_t screen_t;          // sampled screen: screens run (the sample counter)
   int32_t dcount[TTC_MAXD];  // stored forms: parts of bond b's decide that have
                              // merged their share of the tile slots (the last
@@ -242,6 +242,7 @@ struct RunArgs {
   int32_t sampled;       // some instance screens a random sample set (Alg. 1)
   int32_t stored;        // some instance keeps stored residuals
   int32_t max_rook;      // the largest refinement round count of the instances
+  int32_t rook_step;     // host-stepped runs: the refinement step of this launch
 };
 
 // ---------------------------------------------------------------------------

@@ -3001,7 +3001,7 @@ __device__ void decide_bond_sampled(const InstDev &in, Ctrl &cr, int b, DecideSm
     cr.best_row[b] = best.row;
     cr.best_col[b] = best.col;
     const bool go = in.max_rook > 0 && best.row >= 0 && best.key <= KEY_INF;
-    cr.rook_stage[b] = go ? 1 : 0;
+    cr.rook_stage[0][b] = go ? 1 : 0;  // (step 0 reads this copy)
     cr.rook_round[b] = 0;
     cr.rook_moved[b] = 0;
     if (b == 0) cr.screen_t = ld_cg(cr.screen_t) + 1;
@@ -3009,8 +3009,14 @@ __device__ void decide_bond_sampled(const InstDev &in, Ctrl &cr, int b, DecideSm
   __syncthreads();
 }
 
-// some bond of a sampled instance is in a refinement step
-__device__ bool any_rook(const RunArgs &ra) {
+// some bond of a sampled instance is in a refinement step k.  Step k reads the
+// stages' copy k mod 2 (here and in the step itself) and writes the other one,
+// for every bond.  That copy's readers were step k - 1's, and a CTA that writes
+// it has passed the grid barrier behind them; the copy read here is written
+// again by step k + 1, behind the barrier of step k, at which a CTA that is
+// still here has not arrived.  So every CTA reads the same stages and all of
+// them leave the loop after the same step.
+__device__ bool any_rook(const RunArgs &ra, int k) {
   __shared__ int hit;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -3021,7 +3027,7 @@ __device__ bool any_rook(const RunArgs &ra) {
       const Ctrl &cr = *in.ctrl;
       if (ld_cg(cr.state) == ST_DONE || ld_cg(cr.dkind) != DK_BONDS) continue;
       for (int b = 0; b < in.nb; ++b)
-        if (ld_cg(cr.rook_stage[b])) hit = 1;
+        if (ld_cg(cr.rook_stage[k & 1][b])) hit = 1;
     }
   }
   __syncthreads();
@@ -3033,13 +3039,13 @@ __device__ bool any_rook(const RunArgs &ra) {
 // bond's share to arrive merges them (no grid barrier and second phase in
 // between) and the pivot moves to a strictly larger |E|.  A round is step 1
 // then step 2, and the refinement ends after a round that moved nothing or
-// after max_rook rounds.  A CTA reads only the words of bonds it has a share
-// of, before it arrives.  A step is latency (a few thousand residuals of up to
+// after max_rook rounds.  A CTA reads a bond's best only if it has a share of
+// it, before it arrives; the stages have two copies (any_rook).  A step is latency (a few thousand residuals of up to
 // 40 terms on the whole grid): as a scan of all bonds by every CTA, a barrier, a
 // merge of all slots and a second barrier it took about 20 us, so this form and
 // the row copies took the screen of Hilbert d=6, n=256, rank 40, 64 k samples, 8
 // rounds from 5.1-5.4 to 3.5 ms over 24 sweeps (4.8 with the copies alone).
-__device__ void phase_rook_step(const RunArgs &ra, PhaseSmem &sm) {
+__device__ void phase_rook_step(const RunArgs &ra, PhaseSmem &sm, int k) {
   __shared__ CtrlSnap snap;
   __shared__ int32_t s_stage, s_row, s_col, s_last;
   for (int ii = 0; ii < ra.count; ++ii) {
@@ -3053,7 +3059,7 @@ __device__ void phase_rook_step(const RunArgs &ra, PhaseSmem &sm) {
     for (int b = 0; b < in.nb; ++b) {
       const int rank = share_rank(in, b, wide);
       if (rank < 0) continue;
-      if (threadIdx.x == 0) s_stage = ld_cg(cr.rook_stage[b]);
+      if (threadIdx.x == 0) s_stage = ld_cg(cr.rook_stage[k & 1][b]);
       if (threadIdx.x == 1) s_row = ld_cg(cr.best_row[b]);
       if (threadIdx.x == 2) s_col = ld_cg(cr.best_col[b]);
       __syncthreads();
@@ -3061,6 +3067,8 @@ __device__ void phase_rook_step(const RunArgs &ra, PhaseSmem &sm) {
       const int size = share_size(in, b, wide);
       const int64_t rows = rows_of(in, r, b), cols = cols_of(in, r, b);
       const int64_t a0 = s_row, c0 = s_col, len = st == 1 ? rows : cols;
+      int32_t *const next = &cr.rook_stage[(k + 1) & 1][b];
+      if (!st && rank == 0 && threadIdx.x == 0) *next = 0;
       if (st) {
         KeyBest best{0ull, LLONG_MAX, -1, -1};
         for (int64_t x = (int64_t)rank * NT + threadIdx.x; x < len; x += (int64_t)size * NT) {
@@ -3100,13 +3108,13 @@ __device__ void phase_rook_step(const RunArgs &ra, PhaseSmem &sm) {
             }
             if (line.key > KEY_INF) cr.best_key[b] = line.key;  // a non-finite residual ends the bond
             if (st == 1) {
-              cr.rook_stage[b] = 2;
+              *next = 2;
               cr.rook_moved[b] = moved;
             } else {
               const int round = ld_cg(cr.rook_round[b]) + 1;
               cr.rook_round[b] = round;
               const bool again = moved && round < in.max_rook && ld_cg(cr.best_key[b]) <= KEY_INF;
-              cr.rook_stage[b] = again ? 1 : 0;
+              *next = again ? 1 : 0;
               cr.rook_moved[b] = 0;
             }
           }
@@ -4194,8 +4202,8 @@ __global__ void __launch_bounds__(NT, 2) k_persistent(RunArgs ra) {
     if (ra.sampled) {
       // the refinement of Alg. 1, step by step, then the stop tests on the
       // refined pivots
-      for (int k = 0; k < 2 * ra.max_rook && any_rook(ra); ++k) {
-        phase_rook_step(ra, sm);
+      for (int k = 0; k < 2 * ra.max_rook && any_rook(ra, k); ++k) {
+        phase_rook_step(ra, sm, k);
         if (!grid_barrier(ra, 10)) return;
       }
       clk.lap(ra, T_SCREEN);
@@ -4257,7 +4265,7 @@ __global__ void __launch_bounds__(NT, 2) k_decide2(RunArgs ra) {
 }
 __global__ void __launch_bounds__(NT, 2) k_rook_step(RunArgs ra) {
   cache_inst0(ra);
-  phase_rook_step(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem));
+  phase_rook_step(ra, *reinterpret_cast<PhaseSmem *>(dyn_smem), ra.rook_step);
 }
 __global__ void __launch_bounds__(NT, 2) k_finalize(RunArgs ra) {
   cache_inst0(ra);
