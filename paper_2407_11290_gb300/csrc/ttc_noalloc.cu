@@ -274,7 +274,11 @@ __device__ void tc_sort(const ErrArgs &a, int64_t k0, int ns, int m, TcSmem<KP> 
   __syncthreads();
 }
 
-// g_row_exp: a CTA per row of a middle core; 0 for a row of zeros
+// no exponent: of a row or column of zeros
+constexpr int32_t kNone = -(1 << 20);
+
+// g_row_exp: a CTA per row of a middle core.  A row of zeros has none: the
+// column that meets it contributes nothing, so it must not set a unit.
 __global__ void __launch_bounds__(kThreads) k_row_exp(ErrArgs a) {
   const int m = (int)blockIdx.y + 1, k = (int)blockIdx.x;
   if (k >= a.s[m]) return;
@@ -291,13 +295,12 @@ __global__ void __launch_bounds__(kThreads) k_row_exp(ErrArgs a) {
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < kWarps; ++i) e = max(e, red[i]);
-    g_row_exp[m][k] = e ? e - 1023 : 0;
+    g_row_exp[m][k] = e ? e - 1023 : kNone;
   }
 }
 
 // the unit's exponent of a row or column from its largest exponent (kNone: it
 // is zero) and whether an entry was not finite
-constexpr int32_t kNone = -(1 << 20);
 __device__ __forceinline__ int32_t tc_unit_of(int emax, bool bad) {
   return bad ? ttc::TC_BAD : emax - 1084;
 }
@@ -420,8 +423,11 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
       } else {
         // from here on at the scale of the next core's rows
         const int ua = 8 * c + 2 * t;
-        if (ua < N && ea[c] != TC_BAD) ea[c] += g_row_exp[m + 1][ua];
-        if (ua + 1 < N && eb[c] != TC_BAD) eb[c] += g_row_exp[m + 1][ua + 1];
+        const int32_t xa = ua < N ? g_row_exp[m + 1][ua] : 0, xb = ua + 1 < N ? g_row_exp[m + 1][ua + 1] : 0;
+        if (xa == kNone) out[c][0] = out[c][2] = 0;
+        if (xb == kNone) out[c][1] = out[c][3] = 0;
+        if (ea[c] != TC_BAD) ea[c] += xa;
+        if (eb[c] != TC_BAD) eb[c] += xb;
         if (out[c][0]) top0 = max(top0, ea[c] + 64 - __clzll(llabs(out[c][0])));
         if (out[c][1]) top0 = max(top0, eb[c] + 64 - __clzll(llabs(out[c][1])));
         if (out[c][2]) top1 = max(top1, ea[c] + 64 - __clzll(llabs(out[c][2])));
@@ -490,12 +496,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_sums(ErrArgs a, int64_t ch
         for (int k = 0; k < K; ++k) {
           const int e = tc_expo(G[k]);
           inf |= e == 0x7ff;
-          if (e) emax = max(emax, e + g_row_exp[1][k]);
+          if (e && g_row_exp[1][k] != kNone) emax = max(emax, e + g_row_exp[1][k]);
         }
+        auto fix = [&](int k) {
+          return k < K && g_row_exp[1][k] != kNone ? tc_fix(G[k], emax - g_row_exp[1][k]) : TC_BIAS;
+        };
         for (int k = 0; k < KP; k += 2)
-          *reinterpret_cast<uint4 *>(&sm.vec[s][k]) =
-              tc_pack(k < K ? tc_fix(G[k], emax - g_row_exp[1][k]) : TC_BIAS,
-                      k + 1 < K ? tc_fix(G[k + 1], emax - g_row_exp[1][k + 1]) : TC_BIAS);
+          *reinterpret_cast<uint4 *>(&sm.vec[s][k]) = tc_pack(fix(k), fix(k + 1));
         sm.unit[s] = tc_unit_of(emax, inf);
       }
       for (int m = 1; m < a.d - 1; ++m) {
