@@ -207,22 +207,38 @@ __global__ void __launch_bounds__(kThreads) k_chunk_sums(ErrArgs a, int64_t nchu
 // will (a column of one core up, the row of the next down by as much).  So the
 // rows of a middle core are taken at their largest exponent, k_row_exp, and the
 // columns before them grow by it: both are exponents, no product is rounded.
+// That balances a dense bond only.  Where terms have scales of their own (sums of
+// TTs, CP forms, a peak beside a smooth part) the term that sets the unit need not
+// be one that counts, so every sample carries a bound of its error along:
+//   D_k = e_k 2^53 / (KP (d - 2)) - a_k   for entry k of its vector,
+// e_k a bound on the entry's error in fixed point and a_k the chain of absolute
+// values |G_1| ... |G_m|, of which an FP64 chain loses up to KP (d - 2) 2^-53.
+// Both go through a core as its absolute values do, so D does (one bf16 mma.sync
+// beside 36 f16 ones), and a core adds the error of its products: dropped digits of
+// up to 7 2^-62 a term, the operands' rounding, the sum's to 2^-57 (KP = 32; 2^-58),
+// relative to the largest entry of the row and of the column.  Where the sum of D
+// times the last core's |entries| is above zero the sample is computed again by
+// its FP64 chain, as are samples that met subnormal or non-finite entries or left
+// the range of doubles.  (None of the samples of exponential sums in a random
+// basis, 0.6 % of those of a 6D n = 64 Hilbert cross, 8 % of a 2+2D Maxwellian's.)
 // A warp per sample in FP64 issued one FMA per core row with half its lanes
 // idle at size 16: 6.57 ms for 1e6 samples of a 6D n = 64 TT of ranks 16 (its
-// 1.04e9 FMAs take 1.7 ms at the FP64 pipe's rate); this form takes 1.10 ms,
-// 0.09 ms of them for the rows' exponents.
+// 1.04e9 FMAs take 1.7 ms at the FP64 pipe's rate); this form takes 1.33 ms, 0.09 ms
+// of them for the rows' exponents and 0.21 ms for D (ranks 32: 5.70 ms, 4.50 without D).
 constexpr int kTcThreads = 512, kTcN = 256;
 
 template <int KP>
 struct TcSmem {
   static constexpr int S = 16384 / KP;
   uint64_t vec[S][KP];       // fixed-point rows (interleaved pairs)
-  int32_t unit[S];           // exponents of their units
-  double res[S];             // X - X~
+  uint16_t dif[S][KP];       // D of the rows' entries, bf16, largest entry 1
+  int32_t unit[S];           // exponents of their units; after the last core: whether
+                             // the sample goes to its FP64 chain
+  double res[S];             // X~
   uint16_t key[S], order[S];
   uint32_t tile[S / 16 + kTcN];
   int32_t cnt[kTcN];
-  int32_t ntiles;
+  int32_t ntiles, nagain;
   double red[kTcThreads / 32];
 };
 
@@ -304,9 +320,54 @@ __global__ void __launch_bounds__(kThreads) k_row_exp(ErrArgs a) {
 __device__ __forceinline__ int32_t tc_unit_of(int emax, bool bad) {
   return bad ? ttc::TC_BAD : emax - 1084;
 }
+// (the tests of doubles here are on their bits: a comparison would take the FP64 pipe)
+__device__ __forceinline__ bool tc_zero(double x) {
+  return ((uint32_t)__double2hiint(x) << 1 | (uint32_t)__double2loint(x)) == 0;
+}
+// entries that fixed point does not take: not finite, or subnormal
+__device__ __forceinline__ bool tc_odd(double x) {
+  return (uint32_t)(ttc::tc_expo(x) - 1) >= 0x7fe && !tc_zero(x);
+}
+
+// D in bf16 pairs, and its scale: |x| / 2^emax (emax in units of tc_expo, so below
+// 1) cut to bf16, a nonzero one to 2^-126 at least
+__device__ __forceinline__ uint32_t bf_pair(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+__device__ __forceinline__ float bf_lo(uint32_t p) { return __uint_as_float(p << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t p) { return __uint_as_float(p & 0xffff0000u); }
+__device__ __forceinline__ uint32_t bf_abs(double x, int emax) {
+  const int b = (__double2hiint(x) >> 13) & 0x3ffff;  // exponent field, seven bits of the mantissa
+  return b >= 0x80 ? (uint32_t)max(b - ((emax - 126) << 7), 0x80) : 0u;
+}
+__device__ __forceinline__ float exp2_clamped(int n) {
+  return __int_as_float((min(max(n, -126), 127) + 127) << 23);
+}
+// D 2^n of a float D as a double: next to zero below the range of doubles, NaN or
+// Inf above it and for those
+__device__ __forceinline__ double dif_real(float x, int n) {
+  const uint32_t b = __float_as_uint(x);
+  const int e = (int)(b >> 23 & 0xff);
+  const int f = e == 0xff ? 0x7ff : min(max(e + 896 + n, 0), 0x7ff);
+  const uint32_t hi = (b & 0x80000000u) | (uint32_t)f << 20 | (b & 0x7fffff) >> 3;
+  return x == 0.f ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
+}
+// bounds of the errors that D counts, in units of KP 2^-53 of one core
+constexpr float kDifVec = 0x1p-14f;   // an entry of the first vector: 2^-63, KP >= 16
+constexpr float kDifCore = 0.02f;     // 7 2^-62 + 2^-62 a term and 2^-58 (KP = 16) in all
+
+__device__ __forceinline__ void dif_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
 
 // one middle core: rows of the vectors times G_m(i), in place; the last one
-// meets the last core and leaves the residuals
+// meets the last core and leaves X~ and which samples need their FP64 chain
 template <int KP>
 __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
   using namespace ttc;
@@ -329,16 +390,7 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
     const uint32_t tl = sm.tile[x];
     const int i = (int)(tl >> 16), at = (int)(tl >> 4) & 0xfff, rows = (int)(tl & 15) + 1;
     const int sg = sm.order[at + min(g, rows - 1)], sg8 = sm.order[at + min(g + 8, rows - 1)];
-    uint4 A[KS][4];
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      A[ks][0] = *reinterpret_cast<const uint4 *>(&sm.vec[sg][ks * 16 + 2 * t]);
-      A[ks][1] = *reinterpret_cast<const uint4 *>(&sm.vec[sg8][ks * 16 + 2 * t]);
-      A[ks][2] = *reinterpret_cast<const uint4 *>(&sm.vec[sg][ks * 16 + 8 + 2 * t]);
-      A[ks][3] = *reinterpret_cast<const uint4 *>(&sm.vec[sg8][ks * 16 + 8 + 2 * t]);
-    }
     const int32_t e0 = sm.unit[sg], e1 = sm.unit[sg8];
-    __syncwarp();  // the rows are read
     const double *G = a.core[m] + (int64_t)i * N;
     const double *Y = a.core[a.d - 1];
     const int64_t yn = a.n[a.d - 1];
@@ -348,10 +400,12 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
       j1 = coord(a, k0 + sg8, a.d - 1);
     }
     int64_t out[CT][4];
+    uint32_t dif[CT][2];  // D of the outputs, bf16 (columns 2t, 2t + 1 of rows g, g + 8)
     int32_t ea[CT], eb[CT];
     int top0 = INT_MIN, top1 = INT_MIN;
     bool bad = e0 == TC_BAD || e1 == TC_BAD;
-    double v0 = 0.0, v1 = 0.0;
+    double v0 = 0.0, v1 = 0.0, d0 = 0.0, d1 = 0.0;
+    const float core = kDifCore / (float)(a.d - 2);
 #pragma unroll
     for (int c = 0; c < CT; ++c) {
       if (8 * c >= N) break;
@@ -359,7 +413,7 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
       const int u = 8 * c + g;
       double w[KS][4];
       int emax = kNone;
-      bool inf = false;
+      bool odd = false;
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
@@ -372,12 +426,22 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int e = tc_expo(w[ks][q]);
-          inf |= e == 0x7ff;
+          odd |= tc_odd(w[ks][q]);
           if (e) emax = max(emax, e - rx[ks][q]);
         }
       emax = max(emax, __shfl_xor_sync(FULL, emax, 1));
       emax = max(emax, __shfl_xor_sync(FULL, emax, 2));
-      const int32_t ge = tc_unit_of(emax, inf);
+      float dp[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) {
+        const uint16_t *x = &sm.dif[sg][ks * 16 + 2 * t], *y = &sm.dif[sg8][ks * 16 + 2 * t];
+        const uint32_t da[4] = {
+            *reinterpret_cast<const uint32_t *>(x), *reinterpret_cast<const uint32_t *>(y),
+            *reinterpret_cast<const uint32_t *>(x + 8), *reinterpret_cast<const uint32_t *>(y + 8)};
+        dif_mma(dp, da, bf_abs(w[ks][0], emax + rx[ks][0]) | bf_abs(w[ks][1], emax + rx[ks][1]) << 16,
+                bf_abs(w[ks][2], emax + rx[ks][2]) | bf_abs(w[ks][3], emax + rx[ks][3]) << 16);
+      }
+      const int32_t ge = tc_unit_of(emax, odd);
       ea[c] = __shfl_sync(FULL, ge, 8 * t);      // columns 2t, 2t + 1: lanes 4 (2t), 4 (2t + 1)
       eb[c] = __shfl_sync(FULL, ge, 8 * t + 4);
       bad |= ge == TC_BAD;
@@ -390,6 +454,9 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
       for (int ks = 0; ks < KS; ++ks) {
         const uint4 z0 = tc_pack(tc_fix(w[ks][0], emax + rx[ks][0]), tc_fix(w[ks][1], emax + rx[ks][1]));
         const uint4 z1 = tc_pack(tc_fix(w[ks][2], emax + rx[ks][2]), tc_fix(w[ks][3], emax + rx[ks][3]));
+        const uint64_t *x = &sm.vec[sg][ks * 16 + 2 * t], *y = &sm.vec[sg8][ks * 16 + 2 * t];
+        const uint4 x0 = *reinterpret_cast<const uint4 *>(x), x1 = *reinterpret_cast<const uint4 *>(x + 8);
+        const uint4 y0 = *reinterpret_cast<const uint4 *>(y), y1 = *reinterpret_cast<const uint4 *>(y + 8);
         uint32_t db[8][2];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -398,8 +465,7 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const uint32_t da[4] = {tc_digits(A[ks][0], k), tc_digits(A[ks][1], k),
-                                  tc_digits(A[ks][2], k), tc_digits(A[ks][3], k)};
+          const uint32_t da[4] = {tc_digits(x0, k), tc_digits(y0, k), tc_digits(x1, k), tc_digits(y1, k)};
 #pragma unroll
           for (int j = 0; k + j < 8; ++j) tc_mma(acc[k + j], da, db[j][0], db[j][1]);
         }
@@ -411,21 +477,40 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
         const int64_t lo = tc_join(tc_int(acc[4][q], true), tc_int(acc[5][q], true),
                                    tc_int(acc[6][q], true), tc_int(acc[7][q], true));
         out[c][q] = (hi << sh) + ((lo + (1ll << (31 - sh))) >> (32 - sh));
+        // (an output without a term, padding too, has no error)
+        if (dp[q] != 0.f) dp[q] += core;
       }
       if (last) {
         const int ua = 8 * c + 2 * t;
         const double ya0 = ua < N ? Y[ua * yn + j0] : 0.0, yb0 = ua + 1 < N ? Y[(ua + 1) * yn + j0] : 0.0;
         const double ya1 = ua < N ? Y[ua * yn + j1] : 0.0, yb1 = ua + 1 < N ? Y[(ua + 1) * yn + j1] : 0.0;
-        v0 = __fma_rn(tc_real(out[c][0], e0 + ea[c] + 88 - sh), ya0, v0);
-        v0 = __fma_rn(tc_real(out[c][1], e0 + eb[c] + 88 - sh), yb0, v0);
-        v1 = __fma_rn(tc_real(out[c][2], e1 + ea[c] + 88 - sh), ya1, v1);
-        v1 = __fma_rn(tc_real(out[c][3], e1 + eb[c] + 88 - sh), yb1, v1);
+        const double r0 = tc_real(out[c][0], e0 + ea[c] + 88 - sh), r1 = tc_real(out[c][1], e0 + eb[c] + 88 - sh);
+        const double r2 = tc_real(out[c][2], e1 + ea[c] + 88 - sh), r3 = tc_real(out[c][3], e1 + eb[c] + 88 - sh);
+        v0 = __fma_rn(r0, ya0, v0);
+        v0 = __fma_rn(r1, yb0, v0);
+        v1 = __fma_rn(r2, ya1, v1);
+        v1 = __fma_rn(r3, yb1, v1);
+        d0 = __fma_rn(dif_real(dp[0], e0 + ea[c] + 124), fabs(ya0), d0);
+        d0 = __fma_rn(dif_real(dp[1], e0 + eb[c] + 124), fabs(yb0), d0);
+        d1 = __fma_rn(dif_real(dp[2], e1 + ea[c] + 124), fabs(ya1), d1);
+        d1 = __fma_rn(dif_real(dp[3], e1 + eb[c] + 124), fabs(yb1), d1);
+        // (below the range of doubles)
+        bad |= (out[c][0] && tc_zero(r0)) || (out[c][1] && tc_zero(r1)) || (out[c][2] && tc_zero(r2)) ||
+               (out[c][3] && tc_zero(r3));
       } else {
         // from here on at the scale of the next core's rows
         const int ua = 8 * c + 2 * t;
         const int32_t xa = ua < N ? g_row_exp[m + 1][ua] : 0, xb = ua + 1 < N ? g_row_exp[m + 1][ua + 1] : 0;
-        if (xa == kNone) out[c][0] = out[c][2] = 0;
-        if (xb == kNone) out[c][1] = out[c][3] = 0;
+        if (xa == kNone) {
+          out[c][0] = out[c][2] = 0;
+          dp[0] = dp[2] = 0.f;
+        }
+        if (xb == kNone) {
+          out[c][1] = out[c][3] = 0;
+          dp[1] = dp[3] = 0.f;
+        }
+        dif[c][0] = bf_pair(dp[0], dp[1]);
+        dif[c][1] = bf_pair(dp[2], dp[3]);
         if (ea[c] != TC_BAD) ea[c] += xa;
         if (eb[c] != TC_BAD) eb[c] += xb;
         if (out[c][0]) top0 = max(top0, ea[c] + 64 - __clzll(llabs(out[c][0])));
@@ -435,14 +520,20 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
       }
     }
     bad = __any_sync(FULL, bad);
+    __syncwarp();  // the rows are read
     if (last) {
       for (int o = 1; o < 4; o <<= 1) {
         v0 = __dadd_rn(v0, __shfl_xor_sync(FULL, v0, o));
         v1 = __dadd_rn(v1, __shfl_xor_sync(FULL, v1, o));
+        d0 = __dadd_rn(d0, __shfl_xor_sync(FULL, d0, o));
+        d1 = __dadd_rn(d1, __shfl_xor_sync(FULL, d1, o));
       }
-      const double nan = __longlong_as_double(0x7FF8000000000000ll);
-      if (t == 0 && g < rows) sm.res[sg] = bad ? nan : v0;
-      if (t == 1 && g + 8 < rows) sm.res[sg8] = bad ? nan : v1;
+      // (a D that is Inf - Inf fails the comparison too)
+      const bool again = bad || !((t ? d1 : d0) <= 0.0) || tc_expo(t ? v1 : v0) == 0x7ff;
+      if (t < 2 && g + 8 * t < rows) {
+        sm.res[t ? sg8 : sg] = t ? v1 : v0;
+        sm.unit[t ? sg8 : sg] = again;
+      }
     } else {
       for (int o = 1; o < 4; o <<= 1) {
         top0 = max(top0, __shfl_xor_sync(FULL, top0, o));
@@ -456,10 +547,22 @@ __device__ void tc_core(const ErrArgs &a, int64_t k0, int m, TcSmem<KP> &sm) {
           if (g + 8 * h >= rows) continue;
           const int top = h ? top1 : top0;
           int64_t x0 = 0, x1 = 0;
-          if (8 * c < N && top != INT_MIN) {
-            x0 = tc_shift(out[c][2 * h], 62 - (top - ea[c]));
-            x1 = tc_shift(out[c][2 * h + 1], 62 - (top - eb[c]));
+          uint32_t dd = 0;
+          if (8 * c < N) {
+            // (a row of zeros that may not be one: D is whatever is above zero)
+            float da = bf_lo(dif[c][h]), db = bf_hi(dif[c][h]);
+            if (top != INT_MIN) {
+              x0 = tc_shift(out[c][2 * h], 62 - (top - ea[c]));
+              x1 = tc_shift(out[c][2 * h + 1], 62 - (top - eb[c]));
+              da *= exp2_clamped(36 + sh + ea[c] - top);
+              db *= exp2_clamped(36 + sh + eb[c] - top);
+            } else {
+              da = da != 0.f ? 0x1p100f : 0.f;
+              db = db != 0.f ? 0x1p100f : 0.f;
+            }
+            dd = bf_pair(da, db);
           }
+          *reinterpret_cast<uint32_t *>(&sm.dif[h ? sg8 : sg][8 * c + 2 * t]) = dd;
           *reinterpret_cast<uint4 *>(&sm.vec[h ? sg8 : sg][8 * c + 2 * t]) =
               tc_pack((uint64_t)x0 + TC_BIAS, (uint64_t)x1 + TC_BIAS);
         }
@@ -492,23 +595,41 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_sums(ErrArgs a, int64_t ch
         const int K = a.s[1];
         const double *G = a.core[0] + (int64_t)coord(a, k0 + s, 0) * K;
         int emax = kNone;
-        bool inf = false;
+        bool odd = false;
         for (int k = 0; k < K; ++k) {
           const int e = tc_expo(G[k]);
-          inf |= e == 0x7ff;
+          odd |= tc_odd(G[k]);
           if (e && g_row_exp[1][k] != kNone) emax = max(emax, e + g_row_exp[1][k]);
         }
         auto fix = [&](int k) {
           return k < K && g_row_exp[1][k] != kNone ? tc_fix(G[k], emax - g_row_exp[1][k]) : TC_BIAS;
         };
-        for (int k = 0; k < KP; k += 2)
+        const float vec = kDifVec / (float)(a.d - 2);
+        auto dif = [&](int k) {
+          if (k >= K || g_row_exp[1][k] == kNone || tc_zero(G[k])) return 0.f;
+          return vec - __uint_as_float(bf_abs(G[k], emax - g_row_exp[1][k]) << 16);
+        };
+        for (int k = 0; k < KP; k += 2) {
           *reinterpret_cast<uint4 *>(&sm.vec[s][k]) = tc_pack(fix(k), fix(k + 1));
-        sm.unit[s] = tc_unit_of(emax, inf);
+          *reinterpret_cast<uint32_t *>(&sm.dif[s][k]) = bf_pair(dif(k), dif(k + 1));
+        }
+        sm.unit[s] = tc_unit_of(emax, odd);
       }
+      if (tid == 0) sm.nagain = 0;
       for (int m = 1; m < a.d - 1; ++m) {
         tc_sort<KP>(a, k0, ns, m, sm);
         tc_core<KP>(a, k0, m, sm);
       }
+      // the samples that fixed point is not exact enough for
+      for (int s = tid; s < ns; s += kTcThreads)
+        if (sm.unit[s]) sm.order[atomicAdd(&sm.nagain, 1)] = (uint16_t)s;
+      __syncthreads();
+      for (int x = warp; x < sm.nagain; x += kTcThreads / 32) {
+        const int s = sm.order[x];
+        const double xt = tt_value_warp<1>(a, k0 + s);
+        if (lane == 0) sm.res[s] = xt;
+      }
+      __syncthreads();
       for (int s = tid; s < ns; s += kTcThreads) {
         const double x = entry(a, k0 + s), e = __dsub_rn(x, sm.res[s]);
         num = __fma_rn(e, e, num);
