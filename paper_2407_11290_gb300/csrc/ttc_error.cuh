@@ -18,8 +18,12 @@
 // within 2^24 and every FP32 sum is exact.  (This is the splitting of Ozaki,
 // Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication
 // by using fast routines of matrix multiplication", 2012, with digits in fixed
-// point.)  What is dropped lies 2^-61 below the largest product and below, so
-// X~ is at least as exact as the FP64 chains' (each of which rounds K times).
+// point.)  What is dropped lies 2^-61 below the largest product of a sum and below:
+// X~ is as exact as the FP64 chains' (each of which rounds K times) as long as
+// its terms are not far smaller than the largest ones of T and R.  An entry 2^-40
+// of its row's largest keeps 22 bits where FP64 kept 53.  In a cross T's entries
+// are about one and R's as large as the pivots, so what counts is the largest
+// pivot against rms(X) (TC_PEAK): beyond it the chains do the check.
 //
 // The same products extend the prefix / suffix tables by their last mode where
 // its rows are fewer than the samples (n^3 rows for 1e6 samples at n = 64).
@@ -201,7 +205,8 @@ __device__ float tc_tables(const InstDev &in, const int32_t *r, int pL, int pR, 
 // of every sample here (the extra phases cost about 20 us, 1.2e7).
 __device__ void tc_plan(const InstDev &in, const int32_t *r, TcPlan &p) {
   const int d = in.d;
-  if (!in.tc_perm) {
+  const double peak = __longlong_as_double((long long)ld_cg(in.ctrl->piv_max));
+  if (!in.tc_perm || !(peak <= TC_PEAK * ld_cg(in.ctrl->xrms))) {
     p.on = p.nst = p.tl = p.tr = 0;
     choose_split(in, r, p.pL, p.pR);
     return;

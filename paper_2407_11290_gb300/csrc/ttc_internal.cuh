@@ -32,6 +32,13 @@ constexpr int GRID_CAP = 4096;    // largest persistent grid (partial-sum slots)
 constexpr int TC_BLOCK = 32768;   // error samples sorted together by a middle index
 constexpr int TC_NMAX = 2048;     // largest middle mode size of the sorted samples
 constexpr uint32_t TC_NO_TILE = 0xffffffffu;  // an unused tile slot
+// The check's fixed point is 2^-62 of the largest entries of T and R.  T's are
+// about one (a pivot is the largest residual of its column), R's as large as
+// the pivots: where one lies this far above rms(X), the FP64 chains check.
+// At 2^9.6 (6D n = 256 Hilbert) the fixed point's error was a fifth of the chains'; it
+// grows with the ratio, theirs with the terms at hand.  X at 1e6 samples that
+// represent the tensor stays below 2^10 rms(X).
+constexpr double TC_PEAK = 4096.0;
 constexpr int64_t TC_TABLE_MAX = 1 << 20;  // prefix / suffix table rows of the tensor-core plan
 
 enum State : int32_t { ST_SCREEN = 0, ST_UPDATE = 1, ST_VERIFY = 2, ST_DONE = 3 };
@@ -80,6 +87,7 @@ struct Ctrl {
   int64_t best_lin[TTC_MAXD];
   int32_t best_row[TTC_MAXD], best_col[TTC_MAXD];
   double eps, tau, xrms, den, err;
+  uint64_t piv_max;          // bits of the largest |residual| at a pivot (the start's |X| too)
   int64_t sweeps, entries, refinements, tiles_refined;
   int64_t unscreened;        // candidate slots read by a merge that no screen wrote
   // tile schedule of the next screen (written by the instance's owner CTA

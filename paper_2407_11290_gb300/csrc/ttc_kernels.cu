@@ -2280,6 +2280,8 @@ __device__ bool append_pivot(const InstDev &in, Ctrl &cr, int b, int64_t as, int
     // (or its reciprocal overflows), so the screened value was rounding
     // noise and the bond takes no pivot; -1: not finite
     sm.flag = isfinite(delta) ? 1 : isfinite(piv) ? 0 : -1;
+    // (several CTAs append pivots of one instance at once)
+    if (sm.flag == 1) atomicMax((unsigned long long *)&cr.piv_max, (unsigned long long)abs_key(piv));
     B.delta[z] = delta;
   }
   __syncthreads();
@@ -3983,6 +3985,7 @@ __device__ void phase_init2(const RunArgs &ra, PhaseSmem &sm) {
       if (cr.state != ST_DONE) {
         // the pivot entry of every superblock is X(start)
         const double delta = 1.0 / __dsub_rn(xs0, 0.0);
+        cr.piv_max = abs_key(xs0);
         if (!isfinite(delta)) {
           cr.status = 4;
           cr.state = ST_DONE;
