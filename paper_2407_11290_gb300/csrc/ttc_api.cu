@@ -247,15 +247,16 @@ ttc_status user_stage(ttc_handle *h, int64_t cnt, cudaStream_t s) {
 
 // user generator: the entries that entered the superblocks in the last
 // decision (first: every entry of the rank-one superblocks) through the
-// callback into the cache, in stream order; *done and *verify: the run is over,
-// an error check is due (read with the count: one wait per sweep)
-ttc_status user_fill(ttc_handle *h, int first, cudaStream_t s, bool *done, bool *verify) {
+// callback into the cache, in stream order; *done and *verify: the run is over (2
+// and more: its last pivots' inverses are to be bordered), an error check is
+// due (read with the count: one wait per sweep)
+ttc_status user_fill(ttc_handle *h, int first, cudaStream_t s, int *done, bool *verify) {
   CU(launch_user_count(h->d_inst, first, h->ucounts, s));
   int64_t got[3] = {};
   CU(cudaMemcpyAsync(got, h->ucounts + h->nb, sizeof got, cudaMemcpyDeviceToHost, s));
   CU(cudaStreamSynchronize(s));
   const int64_t tot = got[0];
-  *done = got[1] != 0;
+  *done = (int)got[1];
   *verify = got[2] != 0;
   if (tot == 0) return TTC_OK;
   ttc_status st = user_stage(h, tot, s);
@@ -319,16 +320,17 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
   if (user && (us = user_samples(h0, s))) return us;
   CU(launch_phase(PH_INIT1, ra, h0->grid, s));
   CU(launch_phase(PH_INIT2, ra, h0->grid, s));
-  bool done = false, verify = true;
+  int done = 0;
+  bool verify = true;
   if (user && (us = user_fill(h0, 1, s, &done, &verify))) return us;
   CU(launch_phase(PH_INIT3, ra, h0->grid, s));
   for (int64_t it = 0; it <= ra.max_iters; ++it) {
-    if (!user) done = true;
+    if (!user) done = 1;
     for (int i = 0; i < count && !user; ++i) {
       int32_t st = 0;
       CU(cudaMemcpyAsync(&st, &hs[i]->d_ctrl->state, sizeof st, cudaMemcpyDeviceToHost, s));
       CU(cudaStreamSynchronize(s));
-      if (st != ST_DONE) done = false;
+      if (st != ST_DONE) done = 0;
     }
     if (done) return TTC_OK;
     if (ra.stored) CU(launch_phase(PH_BOUND, ra, h0->grid, s));
@@ -346,7 +348,7 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
     }
     if (user) {
       if ((us = user_fill(h0, 0, s, &done, &verify))) return us;
-      if (done) return TTC_OK;
+      if (done == 1) return TTC_OK;
     }
     if (verify) CU(launch_phase(PH_VERIFY, ra, h0->grid, s));
     CU(launch_phase(PH_UPDATE, ra, h0->grid, s));

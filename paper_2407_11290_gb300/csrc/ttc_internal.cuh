@@ -81,6 +81,7 @@ struct Ctrl {
   int32_t r[TTC_MAXD];     // current ranks (bond b)
   int32_t r_old[TTC_MAXD]; // ranks before the last pivot step
   int32_t add[TTC_MAXD];   // bond added a pivot in the last decision
+  int32_t u_rank[TTC_MAXD];// rank of its inverse U (r until the update borders it)
   int32_t maxr[TTC_MAXD];  // rank caps of this run
   int32_t ntiles[TTC_MAXD];// tiles screened for bond b in the last screen
   uint64_t best_key[TTC_MAXD];

@@ -2332,7 +2332,10 @@ __device__ __noinline__ void border_inverse(const InstDev &in, int b, int z, Dec
     U[(int64_t)t * cap + z] = -__dmul_rn(delta, sm.ua[t]);
     U[(int64_t)z * cap + t] = -__dmul_rn(delta, sm.bu[t]);
   }
-  if (tid == 0) U[(int64_t)z * cap + z] = delta;
+  if (tid == 0) {
+    U[(int64_t)z * cap + z] = delta;
+    in.ctrl->u_rank[b] = z + 1;
+  }
   __syncthreads();
 }
 
@@ -3704,8 +3707,16 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
     // the state word is rewritten by the owner CTA during this phase)
     snap_ctrl(cr, in.nb, snap);
     const int st = snap.state;
-    if (st == ST_DONE) continue;
     const int32_t *ro = snap.old_r, *rn = snap.r, *ad = snap.add;
+    if (st == ST_DONE) {
+      // a bond whose residual is not finite ends the run; the inverses of the
+      // bonds that took a pivot in that decision are bordered all the same (not
+      // every bond's flag is of that decision, so the inverses' ranks tell)
+      for (int b = 0; b < in.nb; ++b)
+        if (s_place == b % (int)gridDim.x && ld_cg(cr.u_rank[b]) < rn[b])
+          border_inverse(in, b, rn[b] - 1, sm.d);
+      continue;
+    }
     int nadd = 0;
     for (int b = 0; b < in.nb; ++b) nadd += ad[b];
     const bool screened = snap.screened != 0;
@@ -3993,6 +4004,7 @@ __device__ void phase_init2(const RunArgs &ra, PhaseSmem &sm) {
         for (int b = 0; b < in.nb; ++b) {
           in.bond[b].delta[0] = delta;
           in.bond[b].U[0] = delta;
+          cr.u_rank[b] = 1;
         }
       }
     }
@@ -4637,7 +4649,9 @@ __global__ void k_user_count(const InstDev *inp, int first, int64_t *counts) {
   counts[in.nb] = tot;
   int nadd = 0;
   for (int b = 0; b < in.nb; ++b) nadd += cr.add[b];
-  counts[in.nb + 1] = cr.state == ST_DONE;
+  int nu = 0;  // inverses to be bordered yet
+  for (int b = 0; b < in.nb; ++b) nu += cr.u_rank[b] < cr.r[b];
+  counts[in.nb + 1] = cr.state == ST_DONE ? 1 + nu : 0;
   counts[in.nb + 2] = cr.state != ST_DONE && cr.screened && nadd == 0;
 }
 
