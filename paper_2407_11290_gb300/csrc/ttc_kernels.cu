@@ -377,10 +377,23 @@ __host__ __device__ TileGeo tile_geo_e(const InstDev &in, const Ctrl &cr, const 
 // stays faster (measured on the 6D Hilbert workloads).  Entries from TT cores
 // cost hundreds of FMAs each: 32 x 32 tiles below four waves of 64 x 64.
 // the tile plan of the next screen at ranks r, computed by one warp of the
-// owner CTA (lane b handles bond b)
+// owner CTA (lane b handles bond b).  The stored forms keep the edge of the
+// run's first plan: their tile states and candidate lists are numbered by it,
+// and the update phase reads it beside this writer (planned_cut).
 __device__ void write_plan_warp(const InstDev &in, Ctrl &cr, const int32_t *r, int grid) {
   const int lane = threadIdx.x & 31;
   const bool act = lane < in.nb;
+  const int32_t kept = in.stored ? ld_cg(cr.plan_te) : 0;  // (zero before the first plan)
+  if (kept) {
+    if (act) {
+      const TileGeo g = tile_geo_e(in, cr, r, lane, kept);
+      cr.plan_rows[lane] = g.rows;
+      cr.plan_cols[lane] = g.cols;
+      cr.plan_nrt[lane] = g.nrt;
+      cr.plan_nct[lane] = g.nct;
+    }
+    return;
+  }
   TileGeo g64;
   int64_t t64 = 0;
   int kmax = 0;
@@ -415,8 +428,10 @@ __device__ void write_plan_warp(const InstDev &in, Ctrl &cr, const int32_t *r, i
     TileGeo g32;
     int ok = 1;
     if (act) {
+      // (the stored forms', at the run's rank caps: an edge for the whole run)
+      const TileGeo gc = tile_geo_e(in, cr, in.stored ? cr.maxr : r, lane, 32);
       g32 = tile_geo_e(in, cr, r, lane, 32);
-      ok = (int64_t)g32.nrt * g32.nct <= in.bond[lane].cand_cap;
+      ok = (int64_t)gc.nrt * gc.nct <= in.bond[lane].cand_cap;
     }
     fok = __all_sync(0xffffffffu, ok);
     if (fok) {
@@ -452,18 +467,25 @@ __device__ void write_plan_warp(const InstDev &in, Ctrl &cr, const int32_t *r, i
   if (lane == 0) cr.plan_te = te;
 }
 
-// geometry of bond b as planned (cheap: no tile counting)
-__device__ __forceinline__ TileGeo planned_geo(const InstDev &in, const Ctrl &cr, int b) {
-  TileGeo g;
+// how the planned tiles of bond b cut its blocks: the edge and the pieces, none
+// of which a stored form's later plans change (rows, columns and counts stay
+// unset)
+__device__ __forceinline__ TileGeo planned_cut(const InstDev &in, const Ctrl &cr, int b) {
+  TileGeo g = {};
   g.te = ld_cg(cr.plan_te);
-  g.rows = ld_cg(cr.plan_rows[b]);
-  g.cols = ld_cg(cr.plan_cols[b]);
-  g.nrt = ld_cg(cr.plan_nrt[b]);
-  g.nct = ld_cg(cr.plan_nct[b]);
   g.pr = cr.grid[b];
   g.pc = cr.grid[b + 1];
   if (g.pr > 0) g.P = make_pieces((int32_t)in.n[b], g.pr, g.te);
   if (g.pc > 0) g.Q = make_pieces((int32_t)in.n[b + 1], g.pc, g.te);
+  return g;
+}
+// geometry of bond b as planned (cheap: no tile counting)
+__device__ __forceinline__ TileGeo planned_geo(const InstDev &in, const Ctrl &cr, int b) {
+  TileGeo g = planned_cut(in, cr, b);
+  g.rows = ld_cg(cr.plan_rows[b]);
+  g.cols = ld_cg(cr.plan_cols[b]);
+  g.nrt = ld_cg(cr.plan_nrt[b]);
+  g.nct = ld_cg(cr.plan_nct[b]);
   return g;
 }
 
@@ -3779,8 +3801,9 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
       if (lazy) __syncthreads();
       if (lazy && threadIdx.x < in.nb) {
         const int b = threadIdx.x;
+        // (the owner CTA writes the next plan's rows, columns and counts meanwhile)
         LazyGeo q;
-        q.g = planned_geo(in, cr, b);
+        q.g = planned_cut(in, cr, b);
         stateful_tiles(in, cr, q.g, b, q.tr, q.tc);
         q.stride = state_stride(in, cr, q.g, b);
         s_lazy[b] = q;
