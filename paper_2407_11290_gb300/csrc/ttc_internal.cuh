@@ -29,6 +29,16 @@ constexpr int TT_SMALL = 16;      // ranks up to which a tile's rows share their
 constexpr int BM = 64, BN = 64;   // screen tile (superblock rows x columns)
 constexpr int RCAP = 256;         // largest rank capacity the kernels accept
 constexpr int GRID_CAP = 4096;    // largest persistent grid (partial-sum slots)
+// Bytes of E from which on a screen's carried tiles are lazy (lazy_at).  What laziness
+// saves is E's passes over HBM, for a phase and a grid barrier a sweep, and E this
+// small stays in the L2 (129 MB on two dies) beside the factors.  Measured (ms; lazy
+// throughout, from 32, 48, 64 and 129 MB on): 6D n = 64 Hilbert, 23 MB: 1.56, 1.41
+// from any line; 6D n = 100, 61 MB: 2.21, 2.12, 2.10, 2.07, 2.06; 6D n = 128, 114 MB: 2.85,
+// 2.78, 2.74, 2.68, 2.63; 4D n = 96 Maxwellian, 30 MB: 8.07, 6.60, 6.59, 6.60, 6.57; 6D
+// n = 256, 808 MB: 8.03, 7.95, 7.95, 7.93, 7.91; but 2d2v n = 200, 134 MB: 4.08, 4.09, 4.11,
+// 4.15, 4.40.  An instance counts alone: batches gain more from fewer phases (8 x 6D
+// n = 64: 8.00 lazy, 6.77 with each below the line; 7.12 where their sum counts).
+constexpr float LAZY_BYTES = 48e6f;
 constexpr int TC_BLOCK = 32768;   // error samples sorted together by a middle index
 constexpr int TC_NMAX = 2048;     // largest middle mode size of the sorted samples
 constexpr uint32_t TC_NO_TILE = 0xffffffffu;  // an unused tile slot
@@ -95,10 +105,10 @@ struct Ctrl {
   // whenever its ranks change, read by every CTA): tile edge, and per bond
   // the superblock rows / columns and row / column tile counts
   int32_t plan_te;
+  int32_t lazy;              // stored FP64: its carried tiles wait for their steps (lazy_at)
   int32_t plan_rows[TTC_MAXD], plan_cols[TTC_MAXD];
   int32_t plan_nrt[TTC_MAXD], plan_nct[TTC_MAXD];
   int32_t screened;          // screened in this sweep (set by the screen, cleared by decide)
-  int32_t pad2;
   int32_t pending[TTC_MAXD]; // mixed forms: bond merged, waiting for the refinement
   int32_t nrefine_bond[TTC_MAXD];
   int64_t screen_fmas, error_fmas;  // algorithmic FMAs of the screens / errors
@@ -249,7 +259,7 @@ struct RunArgs {
   int32_t max_iters;     // sweep cap of the launch (sum of rank caps + refinements)
   int32_t *smid;         // [grid] the SM each CTA of a persistent launch runs on
   int32_t sampled;       // some instance screens a random sample set (Alg. 1)
-  int32_t stored;        // some instance keeps stored residuals
+  int32_t stored;        // some instance keeps FP64 stored residuals (host-stepped: bound phases)
   int32_t max_rook;      // the largest refinement round count of the instances
   int32_t rook_step;     // host-stepped runs: the refinement step of this launch
 };

@@ -376,6 +376,15 @@ __host__ __device__ TileGeo tile_geo_e(const InstDev &in, const Ctrl &cr, const 
 // CTAs to work.  At small ranks the per-tile overhead dominates and 64 x 64
 // stays faster (measured on the 6D Hilbert workloads).  Entries from TT cores
 // cost hundreds of FMAs each: 32 x 32 tiles below four waves of 64 x 64.
+// Whether the carried tiles of a screen at ranks r wait for their steps ("lazy
+// carried tiles" below).
+__device__ bool lazy_at(const InstDev &in, const int32_t *r) {
+  if (!in.stored || in.prec != P_FP64) return false;
+  float e = 0.f;
+  for (int b = 0; b < in.nb; ++b) e += (float)rows_of(in, r, b) * (float)cols_of(in, r, b);
+  return 8.f * e >= LAZY_BYTES;
+}
+
 // the tile plan of the next screen at ranks r, computed by one warp of the
 // owner CTA (lane b handles bond b).  The stored forms keep the edge of the
 // run's first plan: their tile states and candidate lists are numbered by it,
@@ -383,6 +392,7 @@ __host__ __device__ TileGeo tile_geo_e(const InstDev &in, const Ctrl &cr, const 
 __device__ void write_plan_warp(const InstDev &in, Ctrl &cr, const int32_t *r, int grid) {
   const int lane = threadIdx.x & 31;
   const bool act = lane < in.nb;
+  if (lane == 0) cr.lazy = lazy_at(in, r);
   const int32_t kept = in.stored ? ld_cg(cr.plan_te) : 0;  // (zero before the first plan)
   if (kept) {
     if (act) {
@@ -1484,7 +1494,9 @@ __device__ void screen_bookkeeping(const InstDev &in, const int32_t *r, const Ti
 // pipe that is not the limit: there it cost more than it saved (5.9 against
 // 5.4 ms when it was tried), so they bring every tile up to date in every
 // screen.
-// phase_bound, before the screen, moves U and the best entries through the
+// Below LAZY_BYTES of E every carried tile is brought up to date by every screen,
+// which then leaves its state as well, so that the first lazy screen finds one.
+// phase_bound, before a lazy screen, moves U and the best entries through the
 // newest step and leaves every CTA's largest best entry per bond; the update
 // phase reads single entries through their pending steps (stored_entry).
 
@@ -1581,8 +1593,8 @@ __device__ void phase_bound(const RunArgs &ra) {
   const int64_t gt = (int64_t)blockIdx.x * NT + threadIdx.x;
   for (int ii = 0; ii < ra.count; ++ii) {
     const InstDev &in = inst(ra, ii);
-    if (!in.stored || in.prec != P_FP64) continue;
     const Ctrl &cr = *in.ctrl;
+    if (!ld_cg(cr.lazy)) continue;
     snap_ctrl(cr, in.nb, snap);
     if (snap.state != ST_SCREEN) continue;
     if (threadIdx.x < in.nb) {
@@ -1930,8 +1942,9 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
     s_tr0[b] = tr0;
     s_tc0[b] = tc0;
     s_str[b] = state_stride(in, cr, g, b);
-    s_ptr[b] = s_str[b] > 0 ? ptr : 0;
-    s_ptc[b] = s_str[b] > 0 ? ptc : 0;
+    const bool waits = s_str[b] > 0 && ld_cg(cr.lazy);
+    s_ptr[b] = waits ? ptr : 0;
+    s_ptc[b] = waits ? ptc : 0;
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -3795,10 +3808,14 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
         if (ad[b] && s_place == (cb0 + G - 1 - b % G) % G)
           border_inverse(in, b, ro[b], sm.d);
       // where the stored entries' pending steps are found (the carried tiles of
-      // the last screen)
+      // the last screen; only a lazy screen leaves steps pending, and only for a
+      // lazy one are the new step's maxima formed)
       __shared__ LazyGeo s_lazy[TTC_MAXB];
+      __shared__ bool s_waits, s_bounds;
       const bool lazy = in.stored && in.prec == P_FP64;
       if (lazy) __syncthreads();
+      if (lazy && threadIdx.x == NT - 1) s_waits = lazy_at(in, ro);
+      if (lazy && threadIdx.x == NT - 2) s_bounds = lazy_at(in, rn);
       if (lazy && threadIdx.x < in.nb) {
         const int b = threadIdx.x;
         // (the owner CTA writes the next plan's rows, columns and counts meanwhile)
@@ -3832,7 +3849,9 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
           const int z = ro[b];
           const int64_t rows = rows_of(in, ro, b), cols = cols_of(in, ro, b);
           const int64_t as = B.prow[z], cs = B.pcol[z];
-          const LazyGeo &lg = s_lazy[b];
+          LazyGeo lg = s_lazy[b];
+          const bool bounds = lazy && s_bounds;
+          if (!lazy || !s_waits) lg.stride = 0;
           double *ew = B.ew + (int64_t)z * B.ldT, *erow = B.erow + (int64_t)z * B.ldR;
           if (item0(base) < base + rows) {
             const double ep = stored_entry(in, lg, b, as, cs, z - 1);
@@ -3840,7 +3859,7 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
               const int64_t a = x - base;
               const double w = -(stored_entry(in, lg, b, a, cs, z - 1) / ep);
               sv_put(in, ew, a, w);
-              if (lazy)
+              if (bounds)
                 atomicMax(&B.wmax[row_tile_of(in, lg.g, b, (int32_t)a)],
                           __float_as_uint(__double2float_ru(fabs(w))));
             }
@@ -3851,7 +3870,7 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
             if (lazy) {
               const double e = stored_entry_t<0>(B, as, c, lazy_z(in, lg, b, as, c, z - 1), z - 1);
               erow[c] = e;
-              atomicMax(&B.emax[col_tile_of(in, lg.g, b, (int32_t)c)], __float_as_uint(SV<0>::up(e)));
+              if (bounds) atomicMax(&B.emax[col_tile_of(in, lg.g, b, (int32_t)c)], __float_as_uint(SV<0>::up(e)));
             } else {
               erow[c] = B.E[as * B.ldR + c];  // a float-float pair, the same 8 bytes
             }
@@ -4101,16 +4120,21 @@ __device__ void phase_refine(const RunArgs &ra, PhaseSmem &sm) {
   }
 }
 
-__device__ bool all_done(const RunArgs &ra) {
-  __shared__ int done;
+// what the coming sweep is: 0 none (every instance is done), 1 one without, 2 one
+// with tiles that wait for their steps
+__device__ int sweep_kind(const RunArgs &ra) {
+  __shared__ int kind;
   __syncthreads();
   if (threadIdx.x == 0) {
-    done = 1;
-    for (int ii = 0; ii < ra.count; ++ii)
-      if (ld_cg(inst(ra, ii).ctrl->state) != ST_DONE) done = 0;
+    kind = 0;
+    for (int ii = 0; ii < ra.count; ++ii) {
+      const Ctrl &cr = *inst(ra, ii).ctrl;
+      const int32_t state = ld_cg(cr.state), lazy = ld_cg(cr.lazy);
+      if (state != ST_DONE) kind = max(kind, lazy ? 2 : 1);
+    }
   }
   __syncthreads();
-  return done != 0;
+  return kind;
 }
 
 // ---------------------------------------------------------------------------
@@ -4222,12 +4246,13 @@ __global__ void __launch_bounds__(NT, 2) k_persistent(RunArgs ra) {
   if (!grid_barrier(ra, 6)) return;
   clk.lap(ra, T_INIT);
   for (int it = 0;; ++it) {
-    if (all_done(ra)) break;
+    const int kind = sweep_kind(ra);
+    if (kind == 0) break;
     if (it >= ra.max_iters) {
       if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&ra.bar->overrun, 1);
       break;
     }
-    if (ra.stored) {
+    if (kind == 2) {
       phase_bound(ra);
       if (!grid_barrier(ra, 14)) return;
     }
