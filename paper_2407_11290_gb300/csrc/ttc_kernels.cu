@@ -1440,11 +1440,14 @@ __host__ __device__ __forceinline__ void carried_tiles(const InstDev &in, const 
 
 // bookkeeping of a screen (one thread, from the CTA's staged geometry):
 // candidate slots per bond for the merge, and the statistics.  Stored form: sr /
-// sc are the stored extents, nfs the fresh items' slots, nca the carried
-// tiles' (the mixed forms; FP64 counts the candidates that it lists); the
-// carried tiles' FMAs and bytes are counted as they are brought up to date.
+// sc are the stored extents, tr0 / tc0 the carried tiles', pend whether a step is
+// pending, nfs the fresh items' slots, nca the carried tiles' (the mixed forms;
+// FP64 counts the candidates that it lists); the carried tiles' FMAs and bytes
+// are counted as they are brought up to date, those of stored entries in tiles
+// that reach beyond them here.
 __device__ void screen_bookkeeping(const InstDev &in, const int32_t *r, const TileGeo *geo,
-                                   const int32_t *sr, const int32_t *sc, const int32_t *nfs,
+                                   const int32_t *sr, const int32_t *sc, const int32_t *tr0,
+                                   const int32_t *tc0, const int32_t *pend, const int32_t *nfs,
                                    const int32_t *nca) {
   Ctrl &cw = *in.ctrl;
   int64_t entries = 0, fmas = 0, fresh = 0, bytes = 0;
@@ -1454,8 +1457,10 @@ __device__ void screen_bookkeeping(const InstDev &in, const int32_t *r, const Ti
     if (sr) {
       const int64_t kept = (int64_t)sr[b] * sc[b];
       fresh += e - kept;
-      fmas += (e - kept) * r[b];
-      bytes += 8 * (e - kept);
+      const int64_t cr = geo[b].pr > 0 ? sr[b] : tr0[b] * geo[b].te;  // of the carried tiles
+      const int64_t cc = geo[b].pc > 0 ? sc[b] : tc0[b] * geo[b].te;
+      fmas += (e - kept) * r[b] + (pend[b] ? kept - cr * cc : 0);
+      bytes += 8 * (e - kept) + 16 * (kept - cr * cc);
       cw.nfresh[b] = nfs[b];
       if (in.prec != P_FP64) cw.ntiles[b] = nca[b];
     } else {
@@ -1978,7 +1983,8 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
     s_nf[b] = (s_geo[b].nrt * s_geo[b].nct - nc) * spt;
   }
   __syncthreads();
-  if (blockIdx.x == 0 && threadIdx.x == 0) screen_bookkeeping(in, r, s_geo, s_sr, s_sc, s_nf, s_nc);
+  if (blockIdx.x == 0 && threadIdx.x == 0)
+    screen_bookkeeping(in, r, s_geo, s_sr, s_sc, s_tr0, s_tc0, s_pend, s_nf, s_nc);
   const bool a_first = s_place < HA;
   for (int part = 0; part < 2; ++part) {
     if ((part == 0) == a_first) {
@@ -2235,7 +2241,7 @@ __device__ void phase_screen(const RunArgs &ra, PhaseSmem &sm) {
     if (threadIdx.x < in.nb) s_pg[threadIdx.x] = planned_geo(in, cr, threadIdx.x);
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0)
-      screen_bookkeeping(in, r, s_pg, nullptr, nullptr, nullptr, nullptr);
+      screen_bookkeeping(in, r, s_pg, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
     for (int b = 0; b < in.nb; ++b) {
       const TileGeo &g = s_pg[b];
       const int32_t nt = g.nrt * g.nct;
