@@ -172,8 +172,8 @@ ttc_status ensure_cands(ttc_handle *h, const int32_t *grid) {
     h->cand = nullptr;
   }
   // one allocation: FP64 candidates, mixed candidates, refinement list and results
-  // (stored form: the carried tiles' states, one per slot)
-  const size_t tbytes = h->hi.stored ? sizeof(TileState) : 0;
+  // (lazy tiles: their states, one per slot)
+  const size_t tbytes = h->hi.lazy ? sizeof(TileState) : 0;
   const size_t bytes = (sizeof(Cand) + sizeof(MCand) + 2 * sizeof(int32_t) + sizeof(Cand) + tbytes) *
                        (size_t)total;
   CU(cudaMalloc(&h->cand, bytes));
@@ -193,7 +193,7 @@ ttc_status ensure_cands(ttc_handle *h, const int32_t *grid) {
     h->bond_cand_cap[b] = need[b];
     h->hi.bond[b].cand_base = off;
     h->hi.bond[b].cand_cap = need[b];
-    h->hi.bond[b].tstate = h->hi.stored ? ts + off : nullptr;
+    h->hi.bond[b].tstate = h->hi.lazy ? ts + off : nullptr;
     off += need[b];
   }
   h->hi.cand = h->cand;
@@ -292,9 +292,9 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
   ra.persistent = (h0->opt.host_loop || user) ? 0 : 1;
   ra.mixed = 0;
   ra.sampled = 0;
-  ra.stored = 0;
+  ra.lazy = 0;
   for (int i = 0; i < count; ++i)
-    if (hs[i]->hi.stored && hs[i]->hi.prec == P_FP64) ra.stored = 1;
+    if (hs[i]->hi.lazy) ra.lazy = 1;
   ra.max_rook = ra.rook_step = 0;
   for (int i = 0; i < count; ++i)
     if (hs[i]->hi.nl > 0) {
@@ -333,7 +333,7 @@ ttc_status launch_run(ttc_handle *const *hs, int count, InstDev *const *d_list, 
       if (st != ST_DONE) done = 0;
     }
     if (done) return TTC_OK;
-    if (ra.stored) CU(launch_phase(PH_BOUND, ra, h0->grid, s));
+    if (ra.lazy) CU(launch_phase(PH_BOUND, ra, h0->grid, s));
     CU(launch_phase(PH_SCREEN, ra, h0->grid, s));
     CU(launch_phase(PH_DECIDE, ra, h0->grid, s));
     if (ra.sampled) {
@@ -745,9 +745,11 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     return s;
   };
   if (o.residual == TTC_RESIDUAL_STORED) {
-    // E [ldT][ldR], the steps ew [cap][ldT] and erow [cap][ldR], the step maxima
-    // and the CTAs' best keys per bond, in one allocation of its own (E dominates
-    // the footprint: 8 B per superblock entry at the rank caps)
+    // E [ldT][ldR], the newest step ew [ldT] and erow [ldR] (lazy tiles: every
+    // step, the newest one's maxima and the CTAs' best keys) per bond, in one
+    // allocation of its own (E dominates the footprint: 8 B per superblock entry
+    // at the rank caps)
+    I.lazy = I.prec == P_FP64;
     Carver ev;
     for (int pass = 0; pass < 2; ++pass) {
       ev.base = static_cast<char *>(h->estore);
@@ -755,15 +757,18 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
       for (int b = 0; b < d - 1; ++b) {
         BondDev &B = I.bond[b];
         double *E = ev.take<double>((size_t)(B.ldT * B.ldR));
-        double *ew = ev.take<double>((size_t)(B.cap * B.ldT));
-        double *er = ev.take<double>((size_t)(B.cap * B.ldR));
-        uint32_t *wm = ev.take<uint32_t>((size_t)B.ldT);
-        uint32_t *em = ev.take<uint32_t>((size_t)B.ldR);
-        uint64_t *low = ev.take<uint64_t>(GRID_CAP);
+        const size_t steps = I.lazy ? B.cap : 1;
+        double *ew = ev.take<double>(steps * (size_t)B.ldT);
+        double *er = ev.take<double>(steps * (size_t)B.ldR);
+        uint32_t *wm = I.lazy ? ev.take<uint32_t>((size_t)B.ldT) : nullptr;
+        uint32_t *em = I.lazy ? ev.take<uint32_t>((size_t)B.ldR) : nullptr;
+        uint64_t *low = I.lazy ? ev.take<uint64_t>(GRID_CAP) : nullptr;
         if (pass == 1) {
           B.E = E;
           B.ew = ew;
           B.erow = er;
+          B.ldw = I.lazy ? B.ldT : 0;
+          B.lde = I.lazy ? B.ldR : 0;
           B.wmax = wm;
           B.emax = em;
           B.low = low;

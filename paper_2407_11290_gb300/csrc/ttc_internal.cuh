@@ -70,11 +70,13 @@ struct BondDev {
   int64_t ldr;           // [ldT][ldr] and [ldR][ldr] (null otherwise)
   int32_t *prow, *pcol;  // pivot superblock coordinates, insertion order
   // stored-residual form (null otherwise): the residual, and the rank-one steps
-  // of the pivots z = 1, 2, ...: step z is row z of ew [cap][ldT] (the column
-  // -E(a,c*) / E(a*,c*)) and of erow [cap][ldR] (E(a*, :)); the largest |ew| /
-  // |erow| of the newest step per row / column tile of the carried tiles (float
-  // bits, rounded up)
+  // of the pivots z = 1, 2, ...: step z is row z of ew (the column -E(a,c*) /
+  // E(a*,c*)) and of erow (E(a*, :)), rows ldw = ldT and lde = ldR apart; where no
+  // tile waits for its steps (InstDev::lazy 0) one row each, ldw = lde = 0
   double *E, *ew, *erow;
+  int64_t ldw, lde;
+  // lazy tiles (null otherwise): the largest |ew| / |erow| of the newest step per row /
+  // column tile of the carried tiles (float bits, rounded up)
   uint32_t *wmax, *emax;
   struct TileState *tstate;  // carried tiles, [row tile][column tile at the rank caps]
   uint64_t *low;         // [GRID_CAP] each CTA's largest key among the carried tiles' entries
@@ -169,6 +171,7 @@ struct InstDev {
   int32_t prec;
   int32_t topk;
   int32_t stored;                    // stored-residual screen
+  int32_t lazy;                      // its carried tiles may wait for their steps (FP64)
   // Alg. 1 with a random sample set: samples per bond and screen (0: the
   // whole superblock), their SplitMix64 seed, refinement rounds
   int64_t nl;
@@ -220,7 +223,7 @@ struct MCand {
 struct TileState {
   float U;
   int32_t z;
-  double val;            // FP64, or a float-float pair
+  double val;
   int64_t lin;
   int32_t row, col;
 };
@@ -259,7 +262,7 @@ struct RunArgs {
   int32_t max_iters;     // sweep cap of the launch (sum of rank caps + refinements)
   int32_t *smid;         // [grid] the SM each CTA of a persistent launch runs on
   int32_t sampled;       // some instance screens a random sample set (Alg. 1)
-  int32_t stored;        // some instance keeps FP64 stored residuals (host-stepped: bound phases)
+  int32_t lazy;          // some instance's tiles may wait (host-stepped: bound phases)
   int32_t max_rook;      // the largest refinement round count of the instances
   int32_t rook_step;     // host-stepped runs: the refinement step of this launch
 };

@@ -379,7 +379,7 @@ __host__ __device__ TileGeo tile_geo_e(const InstDev &in, const Ctrl &cr, const 
 // Whether the carried tiles of a screen at ranks r wait for their steps ("lazy
 // carried tiles" below).
 __device__ bool lazy_at(const InstDev &in, const int32_t *r) {
-  if (!in.stored || in.prec != P_FP64) return false;
+  if (!in.lazy) return false;
   float e = 0.f;
   for (int b = 0; b < in.nb; ++b) e += (float)rows_of(in, r, b) * (float)cols_of(in, r, b);
   return 8.f * e >= LAZY_BYTES;
@@ -997,9 +997,6 @@ struct SV<0> {
   static __device__ __forceinline__ T step(T w, T e, T a) { return __fma_rn(w, e, a); }
   static __device__ __forceinline__ T from(double x) { return x; }
   static __device__ __forceinline__ uint64_t key(T v) { return abs_key(v); }
-  static __device__ __forceinline__ float up(T v) { return __double2float_ru(fabs(v)); }
-  static __device__ __forceinline__ double bits(T v) { return v; }
-  static __device__ __forceinline__ T unbits(double x) { return x; }
 };
 struct SVff {
   using T = float2;
@@ -1030,18 +1027,14 @@ struct SVff {
   static __device__ __forceinline__ uint64_t key(T v) {
     return (uint64_t)(__float_as_uint(v.x) & 0x7FFFFFFFu);
   }
-  static __device__ __forceinline__ float up(T v) { return fabsf(v.x); }
-  static __device__ __forceinline__ double bits(T v) {
-    return __hiloint2double(__float_as_int(v.y), __float_as_int(v.x));
-  }
-  static __device__ __forceinline__ T unbits(double x) {
-    return make_float2(__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x)));
-  }
 };
 template <>
 struct SV<1> : SVff {};
 template <>
 struct SV<2> : SVff {};
+
+// |x| as a float, rounded up
+__device__ __forceinline__ float abs_up(double x) { return __double2float_ru(fabs(x)); }
 
 // a double into stored form (update phase)
 __device__ __forceinline__ void sv_put(const InstDev &in, double *E, int64_t i, double x) {
@@ -1074,8 +1067,8 @@ __device__ __noinline__ void screen_tile_stored_t(const InstDev &in, int b, int 
   const int64_t ld = B.ldR;
   __syncthreads();
   stage_meta(in, b, r0, nr, c0, nc, sm);
-  const double *const ew = B.ew + (int64_t)(K - 1) * B.ldT;      // the newest step (pend)
-  const double *const erow = B.erow + (int64_t)(K - 1) * B.ldR;
+  const double *const ew = B.ew + (int64_t)(K - 1) * B.ldw;      // the newest step (pend)
+  const double *const erow = B.erow + (int64_t)(K - 1) * B.lde;
   VT ev[U][U];
   {
     // FP64: acc; mixed: the float-float pair (fh, fl), and E = A - T R is
@@ -1511,11 +1504,11 @@ __device__ __forceinline__ void stateful_tiles(const InstDev &in, const Ctrl &cr
   carried_tiles(in, g, b, ld_cg(cr.pv_rows[b]), ld_cg(cr.pv_cols[b]), tr, tc);
 }
 // column tiles at the run's rank caps: the stride of the states' rows; 0 if the
-// states would not fit their slots (then every carried tile is brought up to
-// date by every screen)
+// instance has none or they would not fit their slots (then every carried tile
+// is brought up to date by every screen)
 __device__ __forceinline__ int32_t state_stride(const InstDev &in, const Ctrl &cr, const TileGeo &g,
                                                 int b) {
-  if (in.prec != P_FP64) return 0;
+  if (!in.lazy) return 0;
   const int64_t capL = b == 0 ? 1 : cr.maxr[b - 1], capR = b == in.nb - 1 ? 1 : cr.maxr[b + 1];
   const int64_t nr = g.pr > 0 ? capL * g.P.tpb : (capL * in.n[b] + g.te - 1) / g.te;
   const int64_t nc = g.pc > 0 ? capR * g.Q.tpb : (capR * in.n[b + 1] + g.te - 1) / g.te;
@@ -1524,24 +1517,21 @@ __device__ __forceinline__ int32_t state_stride(const InstDev &in, const Ctrl &c
 
 constexpr int LAZY_MAX = 24;  // pending steps a tile may have (a screen's pass applies them)
 
-// E(a, c) of bond b with every step up to pivot z1 applied, from its tile's state
-template <int MIX>
-__device__ __forceinline__ typename SV<MIX>::T stored_entry_t(const BondDev &B, int64_t a, int64_t c,
-                                                              int z0, int z1) {
-  using V = SV<MIX>;
-  typename V::T e = V::load(B.E, a * B.ldR + c);
+// E(a, c) of bond b (FP64) with every step up to pivot z1 applied, from its tile's state
+__device__ __forceinline__ double stepped_entry(const BondDev &B, int64_t a, int64_t c, int z0, int z1) {
+  double e = B.E[a * B.ldR + c];
   int z = z0 + 1;
   for (; z + 3 <= z1; z += 4) {
-    typename V::T w[4], r[4];
+    double w[4], r[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      w[k] = V::load(B.ew, (z + k) * B.ldT + a);
-      r[k] = V::load(B.erow, (z + k) * B.ldR + c);
+      w[k] = B.ew[(z + k) * B.ldw + a];
+      r[k] = B.erow[(z + k) * B.lde + c];
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) e = V::step(w[k], r[k], e);
+    for (int k = 0; k < 4; ++k) e = __fma_rn(w[k], r[k], e);
   }
-  for (; z <= z1; ++z) e = V::step(V::load(B.ew, z * B.ldT + a), V::load(B.erow, z * B.ldR + c), e);
+  for (; z <= z1; ++z) e = __fma_rn(B.ew[z * B.ldw + a], B.erow[z * B.lde + c], e);
   return e;
 }
 
@@ -1561,31 +1551,29 @@ __device__ __forceinline__ int lazy_z(const InstDev &in, const LazyGeo &q, int b
 __device__ __forceinline__ double stored_entry(const InstDev &in, const LazyGeo &q, int b, int64_t a,
                                                int64_t c, int z1) {
   const BondDev &B = in.bond[b];
-  if (in.prec == P_FP64) return stored_entry_t<0>(B, a, c, lazy_z(in, q, b, a, c, z1), z1);
+  if (in.prec == P_FP64) return stepped_entry(B, a, c, lazy_z(in, q, b, a, c, z1), z1);
   const float2 v = SV<2>::load(B.E, a * B.ldR + c);
   return __dadd_rn((double)v.x, (double)v.y);
 }
 
 // phase: bound.  The states of the carried tiles through the newest step.
-template <int MIX>
 __device__ void bound_bond(const InstDev &in, int b, int32_t T, int32_t tc0, int32_t stride, bool pend,
                            int z1, int64_t gt, int64_t NTOT, uint64_t &best) {
-  using V = SV<MIX>;
   const BondDev &B = in.bond[b];
   for (int64_t x = gt; x < T; x += NTOT) {
     const int32_t tr = (int32_t)x / tc0, tc = (int32_t)x - tr * tc0;
     TileState *ts = B.tstate + (int64_t)tr * stride + tc;
-    typename V::T v = V::unbits(ld_cg(ts->val));
+    double v = ld_cg(ts->val);
     if (pend) {
       const float U = __ldcg(&ts->U);
       const int32_t row = ld_cg(ts->row), col = ld_cg(ts->col);
       const float dw = __uint_as_float(__ldcg(&B.wmax[tr])), de = __uint_as_float(__ldcg(&B.emax[tc]));
-      v = V::step(V::load(B.ew, (int64_t)z1 * B.ldT + row), V::load(B.erow, (int64_t)z1 * B.ldR + col), v);
-      ts->val = V::bits(v);
+      v = __fma_rn(B.ew[(int64_t)z1 * B.ldw + row], B.erow[(int64_t)z1 * B.lde + col], v);
+      ts->val = v;
       // every rounding up, and room for the rounding of the values themselves
       ts->U = __fmul_ru(__fadd_ru(U, __fmul_ru(dw, de)), 1.000001f);
     }
-    const uint64_t k = V::key(v);
+    const uint64_t k = abs_key(v);
     best = best > k ? best : k;
   }
 }
@@ -1618,7 +1606,7 @@ __device__ void phase_bound(const RunArgs &ra) {
       uint64_t best = 0;
       const int32_t T = s_tr[b] * s_tc[b];
       if (T > 0 && s_str[b] > 0) {
-        bound_bond<0>(in, b, T, s_tc[b], s_str[b], s_pend[b], snap.r[b] - 1, gt, NTOT, best);
+        bound_bond(in, b, T, s_tc[b], s_str[b], s_pend[b], snap.r[b] - 1, gt, NTOT, best);
         for (int o = 16; o > 0; o >>= 1) {
           const uint64_t k = __shfl_xor_sync(0xffffffffu, best, o);
           best = best > k ? best : k;
@@ -1688,7 +1676,7 @@ __device__ __noinline__ void screen_carried_warp(const InstDev &in, int b, int64
   // wait in registers, the row's by shuffle (FP64 loads them per round and step)
   VT wa[NC], er1[NC];
   if constexpr (MIX != 0) {
-    const double *ew = B.ew + (int64_t)z1 * B.ldT + r0, *er = B.erow + (int64_t)z1 * ld + c0;
+    const double *ew = B.ew + (int64_t)z1 * B.ldw + r0, *er = B.erow + (int64_t)z1 * B.lde + c0;
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
       wa[k] = z1 > z0 ? V::load(ew, min(lane + 32 * k, nr - 1)) : V::zero();
@@ -1741,8 +1729,8 @@ __device__ __noinline__ void screen_carried_warp(const InstDev &in, int b, int64
         }
       }
     } else for (int z = z0 + 1; z <= z1; ++z) {
-      const double *ew = B.ew + (int64_t)z * B.ldT + r0 + r1;
-      const double *er = B.erow + (int64_t)z * ld + c0;
+      const double *ew = B.ew + (int64_t)z * B.ldw + r0 + r1;
+      const double *er = B.erow + (int64_t)z * B.lde + c0;
       VT e[NC];
       e[0] = V::load(er, cl);
       if (NC == 2) e[NC - 1] = V::load(er, cl1);
@@ -1813,10 +1801,11 @@ __device__ __noinline__ void screen_carried_warp(const InstDev &in, int b, int64
     }
   }
   if (lane == 0) *out = Cand{bk, bl, (int32_t)(r0 + brr), (int32_t)(c0 + bcc)};
-  if (ts && mine == brr * 64 + bcc) {  // the lane that holds (and stored) the best
-    const VT bv = V::load(B.E, (r0 + brr) * ld + c0 + bcc);
-    *ts = TileState{V::up(bv), z1, V::bits(bv), bl, (int32_t)(r0 + brr), (int32_t)(c0 + bcc)};
-  }
+  if constexpr (MIX == 0)
+    if (ts && mine == brr * 64 + bcc) {  // the lane that holds (and stored) the best
+      const double bv = B.E[(r0 + brr) * ld + c0 + bcc];
+      *ts = TileState{abs_up(bv), z1, bv, bl, (int32_t)(r0 + brr), (int32_t)(c0 + bcc)};
+    }
   __syncwarp();
 }
 
@@ -1862,7 +1851,7 @@ __device__ __forceinline__ void carried_run(const InstDev &in, const TileGeo &g,
         ts = in.bond[b].tstate + (int64_t)tr * stride + tc;
         const int32_t z = ld_cg(ts->z);
         const float U = __ldcg(&ts->U);
-        key = SV<0>::key(ld_cg(ts->val));
+        key = abs_key(ld_cg(ts->val));
         const bool skip = (double)U < __longlong_as_double((long long)low);
         asis = z == cur && key >= low;
         zt = (z == cur || (skip && cur - z < LAZY_MAX)) ? -1 : z;
@@ -2200,10 +2189,7 @@ __device__ void screen_sampled_instance(const InstDev &in, const int32_t *r, int
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     Ctrl &cw = *in.ctrl;
     int64_t fmas = 0;
-    for (int b = 0; b < in.nb; ++b) {
-      cw.ntiles[b] = gridDim.x;
-      fmas += in.nl * r[b];
-    }
+    for (int b = 0; b < in.nb; ++b) fmas += in.nl * r[b];
     cw.sweeps += 1;
     cw.entries += in.nl * in.nb;
     cw.entries_fresh += in.nl * in.nb;
@@ -2482,7 +2468,7 @@ __device__ void decide_bond_fp64(const InstDev &in, Ctrl &cr, int b, DecideSmem 
   __syncthreads();
   const int64_t nt = sm.q_nt + sm.q_nf;
   if (STORED && tid == 0) close_screen(cr, b, sm);
-  if (STORED) clear_maxima(in, b);
+  if (STORED && in.lazy) clear_maxima(in, b);
   KeyBest best{0ull, LLONG_MAX, -1, -1};
   const Cand *cand = in.cand + in.bond[b].cand_base;
   int bad = 0;
@@ -3818,7 +3804,7 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
       // lazy one are the new step's maxima formed)
       __shared__ LazyGeo s_lazy[TTC_MAXB];
       __shared__ bool s_waits, s_bounds;
-      const bool lazy = in.stored && in.prec == P_FP64;
+      const bool lazy = in.lazy != 0;
       if (lazy) __syncthreads();
       if (lazy && threadIdx.x == NT - 1) s_waits = lazy_at(in, ro);
       if (lazy && threadIdx.x == NT - 2) s_bounds = lazy_at(in, rn);
@@ -3858,7 +3844,7 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
           LazyGeo lg = s_lazy[b];
           const bool bounds = lazy && s_bounds;
           if (!lazy || !s_waits) lg.stride = 0;
-          double *ew = B.ew + (int64_t)z * B.ldT, *erow = B.erow + (int64_t)z * B.ldR;
+          double *ew = B.ew + (int64_t)z * B.ldw, *erow = B.erow + (int64_t)z * B.lde;
           if (item0(base) < base + rows) {
             const double ep = stored_entry(in, lg, b, as, cs, z - 1);
             for (int64_t x = item0(base); x < base + rows; x += NTI) {
@@ -3867,18 +3853,19 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
               sv_put(in, ew, a, w);
               if (bounds)
                 atomicMax(&B.wmax[row_tile_of(in, lg.g, b, (int32_t)a)],
-                          __float_as_uint(__double2float_ru(fabs(w))));
+                          __float_as_uint(abs_up(w)));
             }
           }
           base += rows;
           for (int64_t x = item0(base); x < base + cols; x += NTI) {
             const int64_t c = x - base;
             if (lazy) {
-              const double e = stored_entry_t<0>(B, as, c, lazy_z(in, lg, b, as, c, z - 1), z - 1);
+              const double e = stepped_entry(B, as, c, lazy_z(in, lg, b, as, c, z - 1), z - 1);
               erow[c] = e;
-              if (bounds) atomicMax(&B.emax[col_tile_of(in, lg.g, b, (int32_t)c)], __float_as_uint(SV<0>::up(e)));
+              if (bounds)
+                atomicMax(&B.emax[col_tile_of(in, lg.g, b, (int32_t)c)], __float_as_uint(abs_up(e)));
             } else {
-              erow[c] = B.E[as * B.ldR + c];  // a float-float pair, the same 8 bytes
+              erow[c] = B.E[as * B.ldR + c];  // as it is, a float-float pair too
             }
           }
           base += cols;
@@ -4070,7 +4057,7 @@ __device__ void phase_init3(const RunArgs &ra, PhaseSmem &sm) {
     const InstDev &in = inst(ra, ii);
     const Ctrl &cr = *in.ctrl;
     if (ld_cg(cr.state) == ST_DONE) continue;
-    if (in.stored)
+    if (in.lazy)
       for (int b = 0; b < in.nb; ++b) {
         const BondDev &B = in.bond[b];
         for (int64_t x = gt; x < B.ldT; x += NTOT) B.wmax[x] = 0u;
