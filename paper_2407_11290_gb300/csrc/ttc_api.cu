@@ -171,32 +171,38 @@ ttc_status ensure_cands(ttc_handle *h, const int32_t *grid) {
     CU(cudaFree(h->cand));
     h->cand = nullptr;
   }
-  // one allocation: FP64 candidates, mixed candidates, refinement list and results
-  // (lazy tiles: their states, one per slot)
-  const size_t tbytes = h->hi.lazy ? sizeof(TileState) : 0;
-  const size_t bytes = (sizeof(Cand) + sizeof(MCand) + 2 * sizeof(int32_t) + sizeof(Cand) + tbytes) *
-                       (size_t)total;
-  CU(cudaMalloc(&h->cand, bytes));
-  // all bits set: an unwritten slot reads as row -1 with a NaN key, which the
-  // merges count (ttc_stats.unscreened_slots) instead of trusting
-  CU(cudaMemset(h->cand, 0xFF, bytes));
+  // one allocation, per slot: the candidates; mixed recompute form: the tiles'
+  // candidates and the refinement list; mixed forms: the results of the refinement
+  // or of the decide's parts; lazy tiles: their states
+  const bool mixed = h->hi.prec != P_FP64, tiles = mixed && !h->hi.stored;
+  Carver cv;
+  for (int pass = 0; pass < 2; ++pass) {
+    cv.off = 0;
+    h->hi.cand = cv.take<Cand>((size_t)total);
+    h->hi.mcand = tiles ? cv.take<MCand>((size_t)total) : nullptr;
+    const size_t checked = cv.off;
+    h->hi.refine_list = tiles ? cv.take<int32_t>(2 * (size_t)total) : nullptr;
+    h->hi.refine_cand = mixed ? cv.take<Cand>((size_t)total) : nullptr;
+    TileState *ts = h->hi.lazy ? cv.take<TileState>((size_t)total) : nullptr;
+    for (int64_t b = 0, at = 0; b < h->nb; at += need[b++])
+      h->hi.bond[b].tstate = ts ? ts + at : nullptr;
+    if (pass == 0) {
+      CU(cudaMalloc(&h->cand, cv.off));
+      cv.base = reinterpret_cast<char *>(h->cand);
+      // all bits set: an unwritten slot reads as row -1 with a NaN key, which the
+      // merges count (ttc_stats.unscreened_slots) instead of trusting; the other
+      // arrays are written before they are read
+      CU(cudaMemset(h->cand, 0xFF, checked));
+    }
+  }
   h->cand_cap = total;
-  char *base = reinterpret_cast<char *>(h->cand);
-  h->hi.mcand = reinterpret_cast<MCand *>(base + sizeof(Cand) * total);
-  h->hi.refine_cand = reinterpret_cast<Cand *>(base + (sizeof(Cand) + sizeof(MCand)) * total);
-  h->hi.refine_list =
-      reinterpret_cast<int32_t *>(base + (2 * sizeof(Cand) + sizeof(MCand)) * total);
-  TileState *ts = reinterpret_cast<TileState *>(
-      base + (2 * sizeof(Cand) + sizeof(MCand) + 2 * sizeof(int32_t)) * total);
   int64_t off = 0;
   for (int b = 0; b < h->nb; ++b) {
     h->bond_cand_cap[b] = need[b];
     h->hi.bond[b].cand_base = off;
     h->hi.bond[b].cand_cap = need[b];
-    h->hi.bond[b].tstate = h->hi.lazy ? ts + off : nullptr;
     off += need[b];
   }
-  h->hi.cand = h->cand;
   CU(cudaMemcpy(h->d_inst, &h->hi, sizeof(InstDev), cudaMemcpyHostToDevice));
   // the memset and the copy ran on the legacy stream, which does not order
   // against the caller's (possibly non-blocking) stream, and a pageable copy
@@ -567,6 +573,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
   }
   const bool mxtab = gen->kind == TTC_GEN_MAXWELLIAN || xv;
   int64_t core_cap = 0;
+  size_t clear_bytes = 0;  // of the pool
   for (int pass = 0; pass < 2; ++pass) {
     Carver cv;
     cv.base = static_cast<char *>(h->pool);
@@ -683,6 +690,8 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
       // beside the tables: the rows before their last mode, the cores' columns
       if (tc) ews = std::max(ews + (tl + trr) / 8 + (int64_t)cols + 4096, (int64_t)words);
     }
+    // (the rest is not cleared: it is written before it is read)
+    if (pass == 0) clear_bytes = cv.off;
     double *tabL = cv.take<double>(ews);
     double *tabR = tabL + tl_up;
     uint16_t *tcperm = tc ? cv.take<uint16_t>((size_t)((d - 2) * tc_blocks * TC_BLOCK)) : nullptr;
@@ -806,7 +815,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     h->user_fn = gen->user_fn;
     h->user = gen->user;
   }
-  if (cudaMemset(h->pool, 0, h->pool_bytes) != cudaSuccess)
+  if (cudaMemset(h->pool, 0, clear_bytes) != cudaSuccess)
     return cleanup(fail(TTC_ERR_CUDA, "cudaMemset failed"));
   if (gen->kind == TTC_GEN_HILBERT) {
     std::vector<double> tab(hlen);

@@ -4794,75 +4794,87 @@ cudaError_t launch_user_samples(const InstDev *d_inst, int32_t *idx, cudaStream_
 // counts its samples per index, the counts (and the tiles they make) are
 // scanned over (index, warp), each warp places its samples.  A warp's steps are
 // serial, so as many warps as the counts' shared memory has room for: 32 up to
-// 512 indices, 8 up to TC_NMAX.
+// 512 indices, 8 up to TC_NMAX; the second pass takes the indices and the places
+// among the warp's equal ones from registers (1e6 samples, four middle modes of
+// 64: 63 us, 71 with them formed again; two of 1024: 141 and 158; a ballot per bit in
+// place of the match was slower).
 template <int PW, int NM>
-__global__ void __launch_bounds__(32 * PW) k_tc_perm(const InstDev *inp, uint16_t *perm,
+__global__ void __launch_bounds__(32 * PW, 1) k_tc_perm(const InstDev *inp, uint16_t *perm,
                                                      uint32_t *const *tiles) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int SEG = TC_BLOCK / PW;
+  constexpr uint32_t NONE = 0xffffffffu;
   __shared__ uint16_t cnt[PW][NM];
   __shared__ int32_t wsum[PW], wtile[PW];
   const InstDev &in = *inp;
   const int m = 1 + blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int n = (int)in.n[m];
   const int64_t k0 = (int64_t)blockIdx.x * TC_BLOCK;
+  uint32_t held[SEG / 32];  // index, whether the last of its lanes, place among them
   for (int x = threadIdx.x; x < PW * n; x += blockDim.x) cnt[x / n][x % n] = 0;
   __syncthreads();
-  for (int pass = 0; pass < 2; ++pass) {
-    uint16_t *pm = perm + (int64_t)(m - 1) * in.tc_stride + k0;
-    for (int s = 0; s < SEG; s += 32) {
-      const int id = w * SEG + s + lane;
-      const bool ok = k0 + id < in.nsamples;
-      const int key = ok ? sample_coord(in, k0 + id, m) : n;
-      const unsigned peers = __match_any_sync(FULL, key);
-      const int rank = __popc(peers & ((1u << lane) - 1));
-      if (pass == 1 && ok) pm[cnt[w][key] + rank] = (uint16_t)id;
-      __syncwarp();
-      if (ok && rank == 0) cnt[w][key] += (uint16_t)__popc(peers);
-      __syncwarp();
+#pragma unroll
+  for (int s = 0; s < SEG / 32; ++s) {
+    const int id = w * SEG + s * 32 + lane;
+    const bool ok = k0 + id < in.nsamples;
+    const int key = ok ? sample_coord(in, k0 + id, m) : n;
+    const unsigned peers = __match_any_sync(FULL, key);
+    const int rank = __popc(peers & ((1u << lane) - 1)), many = __popc(peers);
+    held[s] = ok ? (uint32_t)(key << 16 | (rank + 1 == many) << 8 | rank) : NONE;
+    if (ok && rank == 0) cnt[w][key] += (uint16_t)many;
+    __syncwarp();
+  }
+  __syncthreads();
+  // exclusive scan in (index, warp) order: thread x takes indices [x c, (x + 1) c)
+  const int c = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int i0 = min(n, (int)threadIdx.x * c), i1 = min(n, i0 + c);
+  int sum = 0, nti = 0;
+  for (int i = i0; i < i1; ++i) {
+    int v = 0;
+    for (int q = 0; q < PW; ++q) v += cnt[q][i];
+    sum += v;
+    nti += (v + 15) / 16;
+  }
+  int inc = sum, tinc = nti;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(FULL, inc, o), u = __shfl_up_sync(FULL, tinc, o);
+    if (lane >= o) {
+      inc += v;
+      tinc += u;
     }
-    __syncthreads();
-    if (pass == 1) return;
-    // exclusive scan in (index, warp) order: thread x takes indices [x c, (x + 1) c)
-    const int c = (n + (int)blockDim.x - 1) / (int)blockDim.x;
-    const int i0 = min(n, (int)threadIdx.x * c), i1 = min(n, i0 + c);
-    int sum = 0, nti = 0;
-    for (int i = i0; i < i1; ++i) {
-      int v = 0;
-      for (int q = 0; q < PW; ++q) v += cnt[q][i];
-      sum += v;
-      nti += (v + 15) / 16;
+  }
+  if (lane == 31) {
+    wsum[w] = inc;
+    wtile[w] = tinc;
+  }
+  __syncthreads();
+  int at = inc - sum, ta = tinc - nti;
+  for (int q = 0; q < w; ++q) {
+    at += wsum[q];
+    ta += wtile[q];
+  }
+  uint32_t *tl = tiles[m] + (int64_t)blockIdx.x * (TC_BLOCK / 16 + n);
+  for (int i = i0; i < i1; ++i) {
+    const int first = at;
+    for (int q = 0; q < PW; ++q) {
+      const int v = cnt[q][i];
+      cnt[q][i] = (uint16_t)at;
+      at += v;
     }
-    int inc = sum, tinc = nti;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(FULL, inc, o), u = __shfl_up_sync(FULL, tinc, o);
-      if (lane >= o) {
-        inc += v;
-        tinc += u;
-      }
-    }
-    if (lane == 31) {
-      wsum[w] = inc;
-      wtile[w] = tinc;
-    }
-    __syncthreads();
-    int at = inc - sum, ta = tinc - nti;
-    for (int q = 0; q < w; ++q) {
-      at += wsum[q];
-      ta += wtile[q];
-    }
-    uint32_t *tl = tiles[m] + (int64_t)blockIdx.x * (TC_BLOCK / 16 + n);
-    for (int i = i0; i < i1; ++i) {
-      const int first = at;
-      for (int q = 0; q < PW; ++q) {
-        const int v = cnt[q][i];
-        cnt[q][i] = (uint16_t)at;
-        at += v;
-      }
-      for (int o = first; o < at; o += 16)
-        tl[ta++] = ((uint32_t)i << 19) | ((uint32_t)o << 4) | (uint32_t)(min(16, at - o) - 1);
-    }
-    __syncthreads();
+    for (int o = first; o < at; o += 16)
+      tl[ta++] = ((uint32_t)i << 19) | ((uint32_t)o << 4) | (uint32_t)(min(16, at - o) - 1);
+  }
+  __syncthreads();
+  uint16_t *pm = perm + (int64_t)(m - 1) * in.tc_stride + k0;
+#pragma unroll
+  for (int s = 0; s < SEG / 32; ++s) {
+    const uint32_t h = held[s];
+    const int key = h >> 16, rank = h & 0xff;
+    const int to = h == NONE ? 0 : cnt[w][key] + rank;
+    if (h != NONE) pm[to] = (uint16_t)(w * SEG + s * 32 + lane);
+    __syncwarp();
+    if (h != NONE && (h >> 8 & 1)) cnt[w][key] = (uint16_t)(to + 1);
+    __syncwarp();
   }
 }
 
