@@ -212,8 +212,10 @@ ttc_status ttcross_default_options(ttc_options *opt);
 /* Creates a TT-cross instance for a d-way tensor (2 <= d <= 16) with mode
    sizes n[0..d-1] >= 1 and the entry generator *gen.  opt may be NULL
    (defaults).  Allocates all device memory for rank capacity opt->max_rank on
-   the current CUDA device.  Errors: INVALID_ARG (shape/generator/options),
-   OOM, CUDA.  On success *out owns the instance. */
+   the current CUDA device; where that does not fit, without the parts that only
+   make runs faster (the results are the same, the error value within the
+   rounding of its sums).  Errors: INVALID_ARG (shape/generator/options), OOM,
+   CUDA.  On success *out owns the instance. */
 ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen,
                           const ttc_options *opt, ttc_handle **out);
 

@@ -388,8 +388,10 @@ ttc_status ttcross_default_options(ttc_options *opt) {
 
 const char *ttcross_last_error_string(void) { return g_err.c_str(); }
 
-ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, const ttc_options *opt,
-                          ttc_handle **out) {
+// lean: without what only makes runs faster (the error check on the tensor cores, its
+// larger tables, lazy tiles, the sampled screen's row copies)
+static ttc_status create_instance(int d, const int64_t *n, const ttc_generator *gen,
+                                  const ttc_options *opt, bool lean, ttc_handle **out) {
   g_err.clear();
   if (!out) return fail(TTC_ERR_INVALID_ARG, "null output handle");
   *out = nullptr;
@@ -622,7 +624,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
       B.J.sum = cv.take<int32_t>(cap);
       B.Tr = B.Rr = nullptr;
       B.ldr = (cap + 15) / 16 * 16;
-      if (I.nl > 0) {
+      if (I.nl > 0 && !lean) {
         B.Tr = cv.take<double>(B.ldr * B.ldT);
         B.Rr = cv.take<double>(B.ldr * B.ldR);
       }
@@ -643,7 +645,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     {
       // (an eighth of the stored residuals where those are larger)
       double estore = 0.0;
-      if (o.residual == TTC_RESIDUAL_STORED)
+      if (o.residual == TTC_RESIDUAL_STORED && !lean)
         for (int b = 0; b < d - 1; ++b) estore += 8.0 * (double)I.bond[b].ldT * (double)I.bond[b].ldR;
       const int64_t lim = std::max<int64_t>(ns, 4096);
       const int64_t bytes = std::max((int64_t)128 << 20, (int64_t)std::min(estore / 8.0, 1e18));
@@ -668,7 +670,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     // samples' results (at most 1 GiB, else the FP64 chains do every check)
     const int64_t tl_up = (tl + 31) / 32 * 32, tr_up = (trr + 31) / 32 * 32;
     const int64_t tc_blocks = (ns + TC_BLOCK - 1) / TC_BLOCK;
-    bool tc = d >= 3 && ns >= 2 * TC_BLOCK && ns <= (1 << 24);
+    bool tc = !lean && d >= 3 && ns >= 2 * TC_BLOCK && ns <= (1 << 24);
     int64_t ews = tl_up + tr_up;
     if (tc) {
       auto up16 = [](int64_t v) { return (v + 15) / 16 * 16; };
@@ -758,7 +760,7 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
     // step, the newest one's maxima and the CTAs' best keys) per bond, in one
     // allocation of its own (E dominates the footprint: 8 B per superblock entry
     // at the rank caps)
-    I.lazy = I.prec == P_FP64;
+    I.lazy = I.prec == P_FP64 && !lean;
     Carver ev;
     for (int pass = 0; pass < 2; ++pass) {
       ev.base = static_cast<char *>(h->estore);
@@ -876,6 +878,17 @@ ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, con
   }
   *out = h;
   return TTC_OK;
+}
+
+ttc_status ttcross_create(int d, const int64_t *n, const ttc_generator *gen, const ttc_options *opt,
+                          ttc_handle **out) {
+  ttc_status s = create_instance(d, n, gen, opt, false, out);
+  if (s == TTC_ERR_OOM) {
+    cudaGetLastError();  // the failed allocation's, which later launches would report
+    s = create_instance(d, n, gen, opt, true, out);
+    if (s == TTC_ERR_OOM) cudaGetLastError();
+  }
+  return s;
 }
 
 ttc_status ttcross_run(ttc_handle *h, double eps, int max_rank, const int32_t *subtensor_grid,

@@ -2156,7 +2156,8 @@ __device__ __forceinline__ double warp_chain_rows(const double *A, int64_t ra, i
 // slot (thread x of the bond's share takes samples x, x + share NT, ...).  A
 // sample's row of T and column of R come from copies that keep them
 // contiguous: from the t-major factors every entry is a 32-byte sector of its
-// own (2 GB of L2 traffic a screen of 2^18 samples per bond at ranks 24).
+// own (2 GB of L2 traffic a screen of 2^18 samples per bond at ranks 24).  An
+// instance that had no memory for the copies reads the factors.
 __device__ void screen_sampled_instance(const InstDev &in, const int32_t *r, int64_t t,
                                         PhaseSmem &sm) {
   double *buf = sm.sw.rows[threadIdx.x >> 5];
@@ -2174,7 +2175,8 @@ __device__ void screen_sampled_instance(const InstDev &in, const int32_t *r, int
       const uint64_t i = (uint64_t)((t * in.nb + b) * in.nl + (valid ? j : 0));
       const int64_t a = (int64_t)__umul64hi(splitmix64_at(in.lseed, 2 * i), (uint64_t)rows);
       const int64_t c = (int64_t)__umul64hi(splitmix64_at(in.lseed, 2 * i + 1), (uint64_t)cols);
-      const double acc = warp_chain_rows(B.Tr, a, B.ldr, B.Rr, c, B.ldr, r[b], buf);
+      const double acc = B.Tr ? warp_chain_rows(B.Tr, a, B.ldr, B.Rr, c, B.ldr, r[b], buf)
+                              : chain(B.T + a, B.ldT, B.R + c, B.ldR, r[b]);
       if (!valid) continue;
       const double e = __dsub_rn(sb_entry(in, b, a, c), acc);
       if (best.row < 0 || abs_key(e) >= best.key) take_key(best, e, entry_lin(in, b, a, c), a, c);
