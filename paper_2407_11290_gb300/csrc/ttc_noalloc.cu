@@ -687,9 +687,25 @@ ttc_status bad(ttc_status s, const char *msg) {
 std::mutex g_mu;
 double *g_sums[kMaxDevices] = {};
 
+// Every kernel of this file on the current device: a kernel is loaded, which takes
+// device memory, when it is first asked for
+cudaError_t load_kernels() {
+  const void *all[] = {(const void *)k_chunk_sums<1>, (const void *)k_chunk_sums<2>,
+                       (const void *)k_chunk_sums<4>, (const void *)k_chunk_sums<8>,
+                       (const void *)k_row_exp,       (const void *)k_tc_sums<16>,
+                       (const void *)k_tc_sums<32>,   (const void *)k_finish};
+  for (const void *f : all) {
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, f);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // Device address of g_chunk_sums on device dev (the current device).  The
 // first call on a device looks it up and keeps it, so that a later call made
-// while the stream is being captured needs no lookup.  Calls outside a
+// while the stream is being captured needs no lookup, and loads the kernels of
+// all sizes, so that no later call does.  Calls outside a
 // capture look it up again: after cudaDeviceReset the module is loaded anew
 // and the array may sit elsewhere.
 ttc_status scratch_on(int dev, bool capturing, double **out) {
@@ -701,6 +717,7 @@ ttc_status scratch_on(int dev, bool capturing, double **out) {
       if (capturing) return bad(TTC_ERR_CUDA, "scratch address unknown: make a first call before capture");
       return bad(TTC_ERR_CUDA, "cudaGetSymbolAddress of the scratch failed");
     }
+    if (!g_sums[dev] && load_kernels() != cudaSuccess) return bad(TTC_ERR_CUDA, "loading the kernels failed");
     g_sums[dev] = static_cast<double *>(p);
   }
   *out = g_sums[dev];
