@@ -1509,10 +1509,11 @@ __device__ __forceinline__ void stateful_tiles(const InstDev &in, const Ctrl &cr
 __device__ __forceinline__ int32_t state_stride(const InstDev &in, const Ctrl &cr, const TileGeo &g,
                                                 int b) {
   if (!in.lazy) return 0;
-  const int64_t capL = b == 0 ? 1 : cr.maxr[b - 1], capR = b == in.nb - 1 ? 1 : cr.maxr[b + 1];
-  const int64_t nr = g.pr > 0 ? capL * g.P.tpb : (capL * in.n[b] + g.te - 1) / g.te;
-  const int64_t nc = g.pc > 0 ? capR * g.Q.tpb : (capR * in.n[b + 1] + g.te - 1) / g.te;
-  return nr * nc <= in.bond[b].cand_cap ? (int32_t)nc : 0;
+  // (superblock extents stay below 2^31)
+  const int32_t capL = b == 0 ? 1 : cr.maxr[b - 1], capR = b == in.nb - 1 ? 1 : cr.maxr[b + 1];
+  const int32_t nr = g.pr > 0 ? capL * g.P.tpb : (capL * (int32_t)in.n[b] - 1) / g.te + 1;
+  const int32_t nc = g.pc > 0 ? capR * g.Q.tpb : (capR * (int32_t)in.n[b + 1] - 1) / g.te + 1;
+  return (int64_t)nr * nc <= in.bond[b].cand_cap ? nc : 0;
 }
 
 constexpr int LAZY_MAX = 24;  // pending steps a tile may have (a screen's pass applies them)
@@ -1542,7 +1543,7 @@ struct LazyGeo {
 };
 __device__ __forceinline__ int lazy_z(const InstDev &in, const LazyGeo &q, int b, int64_t a, int64_t c,
                                       int z1) {
-  if (q.stride == 0) return z1;
+  if (!in.lazy || q.stride == 0) return z1;
   const int32_t tr = row_tile_of(in, q.g, b, (int32_t)a), tc = col_tile_of(in, q.g, b, (int32_t)c);
   if (tr >= q.tr || tc >= q.tc) return z1;  // not carried by the last screen: up to date
   return ld_cg(in.bond[b].tstate[(int64_t)tr * q.stride + tc].z);
@@ -1890,6 +1891,70 @@ __device__ __forceinline__ void carried_run(const InstDev &in, const TileGeo &g,
   }
 }
 
+// A carried tile of bond b by the whole CTA, from pivot z0 to cur: an eighth of its rows
+// to each warp.  Its best entry goes to the bond's next listed slot (FP64) or
+// to the tile's own (mixed forms), and to its state.
+__device__ __forceinline__ void carried_cta(const InstDev &in, const TileGeo &g, int b, int32_t t, int32_t tc0,
+                            int32_t z0, int32_t cur, int32_t stride, int64_t *lin, Cand *cand,
+                            unsigned long long &fma, unsigned long long &bytes) {
+  __shared__ Cand s_cand[NT / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t tr = t / tc0, tc = t - tr * tc0;
+  int64_t r0, c0;
+  int nr, nc;
+  tile_rows(in, g, b, tr, r0, nr);
+  tile_cols(in, g, b, tc, c0, nc);
+  const int h = g.te / (NT / 32), nh = min(h, nr - warp * h);
+  if (nh > 0)
+    carried_warp(in, g.te, b, r0 + warp * h, nh, c0, nc, z0, cur, lin, &s_cand[warp], nullptr);
+  else if (lane == 0)
+    s_cand[warp].row = -2;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    KeyBest best{0ull, LLONG_MAX, -1, -1};
+    for (int w = 0; w < NT / 32; ++w)
+      kb_take_any(best, KeyBest{s_cand[w].key, s_cand[w].lin, s_cand[w].row, s_cand[w].col});
+    cand += in.prec == P_FP64 ? atomicAdd(&in.ctrl->ntiles[b], 1) : t;
+    *cand = Cand{best.key, best.lin, best.row, best.col};
+    if (stride > 0) {
+      const double v = in.bond[b].E[best.row * in.bond[b].ldR + best.col];
+      in.bond[b].tstate[(int64_t)tr * stride + tc] = TileState{abs_up(v), cur, v, best.lin, best.row, best.col};
+    }
+    const unsigned long long e = (unsigned long long)nr * nc;
+    fma += e * (unsigned long long)(cur - z0);
+    bytes += (cur > z0 ? 16 : 8) * e;
+  }
+}
+
+// carried tiles a CTA below which CTAs take them one at a time
+constexpr int TOGETHER = 4;
+
+// Queue B of the stored screen (below) so taken, an item a tile: first < 0 is a CTA that
+// started on the other queue.  (Out of line: inlined, its registers cost the
+// large screens 1 %.)
+__device__ __noinline__ void carried_together(const InstDev &in, const int32_t *r, const TileGeo *geo,
+                                              const int32_t *tr0, const int32_t *tc0,
+                                              const int32_t *pend, const int32_t *stride,
+                                              const int32_t *nf, int32_t first, int32_t H, int32_t N,
+                                              int64_t *lin, int32_t &item, unsigned long long &fma,
+                                              unsigned long long &bytes) {
+  int32_t nxt = 0;
+  if (threadIdx.x == 0) item = first >= 0 ? first : H < N ? H + atomicAdd(&in.ctrl->steal2, 1) : N;
+  for (;;) {
+    __syncthreads();
+    int32_t j = item;
+    __syncthreads();
+    if (j >= N) break;
+    if (threadIdx.x == 0) nxt = H + atomicAdd(&in.ctrl->steal2, 1);
+    int b = 0;
+    for (; j >= tr0[b] * tc0[b]; ++b) j -= tr0[b] * tc0[b];
+    const int32_t cur = r[b] - 1;
+    carried_cta(in, geo[b], b, j, tc0[b], pend[b] ? cur - 1 : cur, cur, stride[b], lin,
+                in.cand + in.bond[b].cand_base + nf[b], fma, bytes);
+    if (threadIdx.x == 0) item = nxt;
+  }
+}
+
 // The stored screen of one instance.  Work items come from two queues:
 //   A: tiles new to a superblock (fresh: A - T R, r_k FMAs per entry, FP64
 //      pipe or FP32 pipe in the mixed forms), one tile (or quarter) per item;
@@ -1904,7 +1969,11 @@ __device__ __forceinline__ void carried_run(const InstDev &in, const TileGeo &g,
 // round trip overlaps it.  The decide phase clears both counters.  A run is a
 // sixth of a warp's even share (at most 32 tiles: its lanes; a warp's tile
 // takes 40 us beside seven others and a CTA on fresh tiles, so runs of eight
-// tiles per CTA left tails of half a sweep).
+// tiles per CTA left tails of half a sweep).  Where every carried tile is due and
+// they are fewer than TOGETHER a CTA, CTAs take them one at a time (a warp at a tile
+// each is 3D n = 70 Hilbert in 1.00 ms for 0.78, 6D n = 64 in 1.42 for 1.25, 8 of them
+// in a batch 6.70 for 4.96; from two a CTA on: 1.27 and 5.19, from eight 1.25 and
+// 4.96, 6D n = 64 with two pieces a mode 1.47 for 1.40).
 // A bond's candidate slots are its fresh items' (nfresh), then its carried
 // tiles' (ntiles).
 
@@ -1921,24 +1990,27 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
   __shared__ unsigned long long s_fma, s_byte;
   __syncthreads();
   if (threadIdx.x == 0) s_fma = s_byte = 0ull;
+  const bool lazy = ld_cg(cr.lazy);  // carried tiles wait for their steps
+  const int32_t qs = ld_cg(cr.qsplit);  // eighths of the CTAs that start on A (0: half)
   if (threadIdx.x < in.nb) {
     const int b = threadIdx.x;
-    const TileGeo g = planned_geo(in, cr, b);
     const int32_t sr = ld_cg(cr.st_rows[b]);
     const int32_t sc = ld_cg(cr.st_cols[b]);
+    const int32_t pend = ld_cg(cr.e_pend[b]);
+    const TileGeo g = planned_geo(in, cr, b);
     int32_t tr0, tc0, ptr, ptc;
     carried_tiles(in, g, b, sr, sc, tr0, tc0);
     stateful_tiles(in, cr, g, b, ptr, ptc);
     s_geo[b] = g;
     s_sr[b] = sr;
     s_sc[b] = sc;
-    s_pend[b] = ld_cg(cr.e_pend[b]);
+    s_pend[b] = pend;
     s_tr0[b] = tr0;
     s_tc0[b] = tc0;
     s_str[b] = state_stride(in, cr, g, b);
-    const bool waits = s_str[b] > 0 && ld_cg(cr.lazy);
-    s_ptr[b] = waits ? ptr : 0;
-    s_ptc[b] = waits ? ptc : 0;
+    const bool has = s_str[b] > 0 && lazy;
+    s_ptr[b] = has ? ptr : 0;
+    s_ptc[b] = has ? ptc : 0;
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1955,16 +2027,16 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
     nc_all += nc;
   }
   const int32_t G = gridDim.x;
-  const int32_t run = max(1, min(32, nc_all / (6 * G * (NT / 32))));  // tiles of a B item
+  const bool together = !lazy && nc_all < TOGETHER * G;
+  const int32_t run = together ? 1 : max(1, min(32, nc_all / (6 * G * (NT / 32))));  // tiles of a B item
   int32_t nB = 0;
   for (int b = 0; b < in.nb; ++b) nB += (s_tr0[b] * s_tc0[b] + run - 1) / run;
   const bool quarters = s_geo[0].te == 64 && nf < (int32_t)gridDim.x;
   const int32_t spt = quarters ? STORED_SLOTS : 1;  // items per tile
   const int32_t nA = spt * nf;
-  const int32_t qs = ld_cg(cr.qsplit);  // eighths of the CTAs that start on A (0: half)
   const int32_t HA = nA == 0 ? 0 : nB == 0 ? G : qs > 0 ? max(1, min(G - 1, G * qs / 8))
                                                          : (G + 1) / 2;
-  const int32_t HB = (G - HA) * (NT / 32);  // warps that start on B
+  const int32_t HB = (G - HA) * (together ? 1 : NT / 32);  // CTAs or warps that start on B
   __shared__ int32_t s_nf[TTC_MAXB], s_nc[TTC_MAXB];  // slots of the fresh items, carried tiles
   if (threadIdx.x < in.nb) {
     const int b = threadIdx.x, nc = s_tr0[b] * s_tc0[b];
@@ -1977,9 +2049,10 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
   const bool a_first = s_place < HA;
   for (int part = 0; part < 2; ++part) {
     if ((part == 0) == a_first) {
-      // queue A, the CTA together
+      // queue A, the CTA together (a CTA that started on B asks only if there is
+      // more than the others' first items)
       int32_t nxt = 0;
-      if (threadIdx.x == 0) s_item = a_first ? s_place : HA + atomicAdd(ctr[0], 1);
+      if (threadIdx.x == 0) s_item = a_first ? s_place : HA < nA ? HA + atomicAdd(ctr[0], 1) : nA;
       for (;;) {
         __syncthreads();
         int32_t j = s_item;
@@ -2032,11 +2105,14 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
         }
         if (threadIdx.x == 0) s_item = nxt;
       }
+    } else if (together) {
+      carried_together(in, r, s_geo, s_tr0, s_tc0, s_pend, s_str, s_nf, a_first ? -1 : s_place - HA, HB, nB,
+                       reinterpret_cast<int64_t *>(&sm.s.op) + warp * BM, s_item, s_fma, s_byte);
     } else {
       // queue B, each warp on its own
       int64_t *lin = reinterpret_cast<int64_t *>(&sm.s.op) + warp * BM;
-      int32_t item = a_first ? 0 : (s_place - HA) * (NT / 32) + warp;
-      if (a_first) {
+      int32_t item = a_first ? nB : (s_place - HA) * (NT / 32) + warp;
+      if (a_first && HB < nB) {
         if (lane == 0) item = HB + atomicAdd(ctr[1], 1);
         item = __shfl_sync(0xffffffffu, item, 0);
       }
@@ -3805,18 +3881,17 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
       // the last screen; only a lazy screen leaves steps pending, and only for a
       // lazy one are the new step's maxima formed)
       __shared__ LazyGeo s_lazy[TTC_MAXB];
-      __shared__ bool s_waits, s_bounds;
+      __shared__ bool s_bounds;
       const bool lazy = in.lazy != 0;
       if (lazy) __syncthreads();
-      if (lazy && threadIdx.x == NT - 1) s_waits = lazy_at(in, ro);
-      if (lazy && threadIdx.x == NT - 2) s_bounds = lazy_at(in, rn);
+      if (lazy && threadIdx.x == NT - 1) s_bounds = lazy_at(in, rn);
       if (lazy && threadIdx.x < in.nb) {
         const int b = threadIdx.x;
         // (the owner CTA writes the next plan's rows, columns and counts meanwhile)
         LazyGeo q;
         q.g = planned_cut(in, cr, b);
         stateful_tiles(in, cr, q.g, b, q.tr, q.tc);
-        q.stride = state_stride(in, cr, q.g, b);
+        q.stride = lazy_at(in, ro) ? state_stride(in, cr, q.g, b) : 0;
         s_lazy[b] = q;
       }
       if (lazy) __syncthreads();
@@ -3843,9 +3918,8 @@ __device__ void phase_update(const RunArgs &ra, PhaseSmem &sm) {
           const int z = ro[b];
           const int64_t rows = rows_of(in, ro, b), cols = cols_of(in, ro, b);
           const int64_t as = B.prow[z], cs = B.pcol[z];
-          LazyGeo lg = s_lazy[b];
+          const LazyGeo &lg = s_lazy[b];
           const bool bounds = lazy && s_bounds;
-          if (!lazy || !s_waits) lg.stride = 0;
           double *ew = B.ew + (int64_t)z * B.ldw, *erow = B.erow + (int64_t)z * B.lde;
           if (item0(base) < base + rows) {
             const double ep = stored_entry(in, lg, b, as, cs, z - 1);
