@@ -491,11 +491,13 @@ __device__ __forceinline__ TileGeo planned_cut(const InstDev &in, const Ctrl &cr
 }
 // geometry of bond b as planned (cheap: no tile counting)
 __device__ __forceinline__ TileGeo planned_geo(const InstDev &in, const Ctrl &cr, int b) {
+  const int32_t rows = ld_cg(cr.plan_rows[b]), cols = ld_cg(cr.plan_cols[b]);
+  const int32_t nrt = ld_cg(cr.plan_nrt[b]), nct = ld_cg(cr.plan_nct[b]);
   TileGeo g = planned_cut(in, cr, b);
-  g.rows = ld_cg(cr.plan_rows[b]);
-  g.cols = ld_cg(cr.plan_cols[b]);
-  g.nrt = ld_cg(cr.plan_nrt[b]);
-  g.nct = ld_cg(cr.plan_nct[b]);
+  g.rows = rows;
+  g.cols = cols;
+  g.nrt = nrt;
+  g.nct = nct;
   return g;
 }
 
@@ -1506,14 +1508,17 @@ __device__ __forceinline__ void stateful_tiles(const InstDev &in, const Ctrl &cr
 // column tiles at the run's rank caps: the stride of the states' rows; 0 if the
 // instance has none or they would not fit their slots (then every carried tile
 // is brought up to date by every screen)
-__device__ __forceinline__ int32_t state_stride(const InstDev &in, const Ctrl &cr, const TileGeo &g,
-                                                int b) {
+__device__ __forceinline__ int32_t state_stride(const InstDev &in, const TileGeo &g, int b,
+                                                int32_t capL, int32_t capR) {
   if (!in.lazy) return 0;
   // (superblock extents stay below 2^31)
-  const int32_t capL = b == 0 ? 1 : cr.maxr[b - 1], capR = b == in.nb - 1 ? 1 : cr.maxr[b + 1];
   const int32_t nr = g.pr > 0 ? capL * g.P.tpb : (capL * (int32_t)in.n[b] - 1) / g.te + 1;
   const int32_t nc = g.pc > 0 ? capR * g.Q.tpb : (capR * (int32_t)in.n[b + 1] - 1) / g.te + 1;
   return (int64_t)nr * nc <= in.bond[b].cand_cap ? nc : 0;
+}
+__device__ __forceinline__ int32_t state_stride(const InstDev &in, const Ctrl &cr, const TileGeo &g,
+                                                int b) {
+  return state_stride(in, g, b, b == 0 ? 1 : cr.maxr[b - 1], b == in.nb - 1 ? 1 : cr.maxr[b + 1]);
 }
 
 constexpr int LAZY_MAX = 24;  // pending steps a tile may have (a screen's pass applies them)
@@ -1994,20 +1999,22 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
   const int32_t qs = ld_cg(cr.qsplit);  // eighths of the CTAs that start on A (0: half)
   if (threadIdx.x < in.nb) {
     const int b = threadIdx.x;
-    const int32_t sr = ld_cg(cr.st_rows[b]);
-    const int32_t sc = ld_cg(cr.st_cols[b]);
+    // (every word in one round of loads: each more is 0.4 us of a small sweep)
+    const int32_t sr = ld_cg(cr.st_rows[b]), sc = ld_cg(cr.st_cols[b]);
+    const int32_t pr = ld_cg(cr.pv_rows[b]), pc = ld_cg(cr.pv_cols[b]);
     const int32_t pend = ld_cg(cr.e_pend[b]);
+    const int32_t capL = b == 0 ? 1 : ld_cg(cr.maxr[b - 1]), capR = b == in.nb - 1 ? 1 : ld_cg(cr.maxr[b + 1]);
     const TileGeo g = planned_geo(in, cr, b);
     int32_t tr0, tc0, ptr, ptc;
     carried_tiles(in, g, b, sr, sc, tr0, tc0);
-    stateful_tiles(in, cr, g, b, ptr, ptc);
+    carried_tiles(in, g, b, pr, pc, ptr, ptc);
     s_geo[b] = g;
     s_sr[b] = sr;
     s_sc[b] = sc;
     s_pend[b] = pend;
     s_tr0[b] = tr0;
     s_tc0[b] = tc0;
-    s_str[b] = state_stride(in, cr, g, b);
+    s_str[b] = state_stride(in, g, b, capL, capR);
     const bool has = s_str[b] > 0 && lazy;
     s_ptr[b] = has ? ptr : 0;
     s_ptc[b] = has ? ptc : 0;
@@ -2029,8 +2036,8 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
   const int32_t G = gridDim.x;
   const bool together = !lazy && nc_all < TOGETHER * G;
   const int32_t run = together ? 1 : max(1, min(32, nc_all / (6 * G * (NT / 32))));  // tiles of a B item
-  int32_t nB = 0;
-  for (int b = 0; b < in.nb; ++b) nB += (s_tr0[b] * s_tc0[b] + run - 1) / run;
+  int32_t nB = run == 1 ? nc_all : 0;
+  for (int b = 0; b < in.nb && run > 1; ++b) nB += (s_tr0[b] * s_tc0[b] + run - 1) / run;
   const bool quarters = s_geo[0].te == 64 && nf < (int32_t)gridDim.x;
   const int32_t spt = quarters ? STORED_SLOTS : 1;  // items per tile
   const int32_t nA = spt * nf;
@@ -2044,7 +2051,7 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
     s_nf[b] = (s_geo[b].nrt * s_geo[b].nct - nc) * spt;
   }
   __syncthreads();
-  if (blockIdx.x == 0 && threadIdx.x == 0)
+  if (s_place == G - 1 && threadIdx.x == 0)  // (the place the items reach last)
     screen_bookkeeping(in, r, s_geo, s_sr, s_sc, s_tr0, s_tc0, s_pend, s_nf, s_nc);
   const bool a_first = s_place < HA;
   for (int part = 0; part < 2; ++part) {
