@@ -1978,7 +1978,8 @@ __device__ __noinline__ void carried_together(const InstDev &in, const int32_t *
 // they are fewer than TOGETHER a CTA, CTAs take them one at a time (a warp at a tile
 // each is 3D n = 70 Hilbert in 1.00 ms for 0.78, 6D n = 64 in 1.42 for 1.25, 8 of them
 // in a batch 6.70 for 4.96; from two a CTA on: 1.27 and 5.19, from eight 1.25 and
-// 4.96, 6D n = 64 with two pieces a mode 1.47 for 1.40).
+// 4.96, 6D n = 64 with two pieces a mode 1.47 for 1.40).  Not the mixed forms' 32-wide
+// tiles, of which a warp has but four rows: 6D n = 64 with two pieces 1.38 for 1.33 ms.
 // A bond's candidate slots are its fresh items' (nfresh), then its carried
 // tiles' (ntiles).
 
@@ -2034,7 +2035,8 @@ __device__ void screen_stored_instance(const InstDev &in, const int32_t *r, Phas
     nc_all += nc;
   }
   const int32_t G = gridDim.x;
-  const bool together = !lazy && nc_all < TOGETHER * G;
+  const bool together =
+      !lazy && nc_all < TOGETHER * G && (s_geo[0].te == 64 || in.prec == P_FP64);
   const int32_t run = together ? 1 : max(1, min(32, nc_all / (6 * G * (NT / 32))));  // tiles of a B item
   int32_t nB = run == 1 ? nc_all : 0;
   for (int b = 0; b < in.nb && run > 1; ++b) nB += (s_tr0[b] * s_tc0[b] + run - 1) / run;
