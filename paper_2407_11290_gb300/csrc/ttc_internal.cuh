@@ -31,7 +31,9 @@ constexpr int RCAP = 256;         // largest rank capacity the kernels accept
 constexpr int GRID_CAP = 4096;    // largest persistent grid (partial-sum slots)
 // Bytes of E from which on a screen's carried tiles are lazy (lazy_at).  What laziness
 // saves is E's passes over HBM, for a phase and a grid barrier a sweep, and E this
-// small stays in the L2 (129 MB on two dies) beside the factors.  Measured (ms; lazy
+// small stays in the L2 (129 MB on two dies) beside the factors.  Measured, with a warp at
+// each carried tile (few of them now go to whole CTAs, which is faster below the line: 6D
+// n = 64 in 1.25, 8 of them in 4.96; TOGETHER in ttc_kernels.cu), in ms (lazy
 // throughout, from 32, 48, 64 and 129 MB on): 6D n = 64 Hilbert, 23 MB: 1.56, 1.41
 // from any line; 6D n = 100, 61 MB: 2.21, 2.12, 2.10, 2.07, 2.06; 6D n = 128, 114 MB: 2.85,
 // 2.78, 2.74, 2.68, 2.63; 4D n = 96 Maxwellian, 30 MB: 8.07, 6.60, 6.59, 6.60, 6.57; 6D
